@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(128) k_list(const KArgs a) {
     node_force<T, LT>(a, n, fl, Fx, Fy, Fz);
     if (MODE == 0) {
       const Coll<T> c = make_coll<LAT, T>(a);
-      collide<LAT, CM, T>(f, Fx, Fy, Fz, c);
+      collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
       scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
     } else {
       write_fields<LAT, T>(a, n, f, Fx, Fy, Fz);
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(256) k_local(const KArgs a) {
   node_force<T, LT>(a, n, fl, Fx, Fy, Fz);
   if (MODE == 0) {
     const Coll<T> c = make_coll<LAT, T>(a);
-    collide<LAT, CM, T>(f, Fx, Fy, Fz, c);
+    collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
     scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
   } else {
     write_fields<LAT, T>(a, n, f, Fx, Fy, Fz);
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(128) k_refill(const KArgs a) {
   T Fx, Fy, Fz;
   node_force<T, T>(a, n, a.flags[n], Fx, Fy, Fz);
   const Coll<T> c = make_coll<LAT, T>(a);
-  collide<LAT, CM, T>(f, Fx, Fy, Fz, c);
+  collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
   scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
 }
 
@@ -852,7 +852,7 @@ __global__ void __launch_bounds__(128) k_face(const KArgs a) {
   }
   if (MODE == 0) {
     const Coll<T> c = make_coll<LAT, T>(a);
-    collide<LAT, CM, T>(f, Fx, Fy, Fz, c);
+    collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
     scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
   } else if (MODE == 1) {
     write_fields<LAT, T>(a, n, f, Fx, Fy, Fz);
@@ -936,10 +936,8 @@ __global__ void __launch_bounds__(256) k_kempe(const KArgs a) {
 inline int div_up(long long a, int b) { return (int)((a + b - 1) / b); }
 
 // The vector bulk sweep: W words per thread and direction (bulk_vec_words 2
-// or 4; 0 = 2) and the node-pair collision packed (bulk_vec_packed 1) or
-// node by node (0); -1 picks what measured fastest on the 128^3 sphere
-// lattice: 8-byte vectors, node by node for FP32 storage, packed for 16-bit
-// storage.  Returns false where nx or the direction stride is not a
+// or 4; 0 = 2) and the node-pair collision packed (bulk_vec_packed 1, and -1,
+// the default: figures at vec_regs) or node by node (0).  Returns false where nx or the direction stride is not a
 // multiple of the V nodes of a vector.
 template <int LAT, int CM, typename S, int W>
 bool launch_bulk_vec_w(const KArgs &a, int want, bool packed, cudaStream_t st) {
@@ -953,7 +951,7 @@ bool launch_bulk_vec_w(const KArgs &a, int want, bool packed, cudaStream_t st) {
 }
 template <int LAT, int CM, typename S>
 bool launch_bulk_vec(const KArgs &a, int want, cudaStream_t st) {
-  const bool packed = a.bulk_vec_packed >= 0 ? a.bulk_vec_packed != 0 : sizeof(S) == 2;
+  const bool packed = a.bulk_vec_packed != 0;
   if (a.bulk_vec_words == 4) return launch_bulk_vec_w<LAT, CM, S, 4>(a, want, packed, st);
   return launch_bulk_vec_w<LAT, CM, S, 2>(a, want, packed, st);
 }
@@ -1040,14 +1038,11 @@ bool launch_group_t(const KArgs *as, int n, cudaStream_t st) {
           as[k].bulk_vec_packed != a0.bulk_vec_packed || as[k].bulk_block != a0.bulk_block)
         return false;
     if (a0.bulk_mode < 1 || n < 1 || n > kMaxGroup) return false;
-    // only the default vector shape of the storage type is built grouped (2
-    // words; node by node for FP32, packed pairs for 16-bit storage): each
-    // grouped variant inlines the update kMaxGroup times
-    constexpr bool kPacked = sizeof(S) == 2;
-    const bool packed = a0.bulk_vec_packed >= 0 ? a0.bulk_vec_packed != 0 : kPacked;
-    if (a0.bulk_vec_words == 4 || packed != kPacked) return false;
+    // only the default vector shape is built grouped (2 words, packed pairs):
+    // each grouped variant inlines the update kMaxGroup times
+    if (a0.bulk_vec_words == 4 || a0.bulk_vec_packed == 0) return false;
     const int want = a0.bulk_block > 0 ? a0.bulk_block : 128;
-    return launch_group_w<LAT, CM, S, 2, kPacked>(as, n, want, st);
+    return launch_group_w<LAT, CM, S, 2, true>(as, n, want, st);
   }
 }
 

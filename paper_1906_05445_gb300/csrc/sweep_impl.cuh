@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(512) k_bulk_sweep(const KArgs a) {
   gather_pull<LAT, S, T, (HINT & 1)>((const S *)a.src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
   const Coll<T> c = make_coll<LAT, T>(a);
   const T gon = (fl & FL_NOG) ? (T)0 : (T)1;
-  collide<LAT, CM, T>(f, gon * kg<T>(a, 0), gon * kg<T>(a, 1), gon * kg<T>(a, 2), c);
+  collide<LAT, CM, S, T>(f, gon * kg<T>(a, 0), gon * kg<T>(a, 1), gon * kg<T>(a, 2), c);
   scatter<LAT, S, T, (HINT & 2) != 0>((S *)a.dst, a.fs, n, isc, f);
 }
 

@@ -6,9 +6,9 @@
 // the pulled values are the row shifted by one node: the thread takes the
 // missing end node from its neighbour lane's vector (or loads it itself at a
 // row or warp edge).  The collision then runs on pairs of nodes in packed
-// FP32x2 arithmetic (one instruction for two nodes), with the same pair form
-// as `collide` in lbm_device.cuh: Eq. 1 (BGK) or Eq. 3 (MRT) with Guo
-// forcing, where MRT differs from BGK only on the energy-flux (q) moments.
+// FP32x2 arithmetic (one instruction for two nodes) or node by node, both
+// through collide_two_rate in lbm_device.cuh: Eq. 1 (BGK) or Eq. 3 (MRT) with
+// Guo forcing, where MRT differs from BGK only on the energy-flux (q) moments.
 //
 // Requirements (checked by the launcher, which otherwise runs the one-node
 // kernel): nx % V == 0 and a direction stride that is a multiple of V.
@@ -16,168 +16,11 @@
 
 #include "sweep_impl.cuh"
 
-
 namespace lbm {
 
 // ---------------------------------------------------------------- FP32x2
 __device__ __forceinline__ float2 bc2(float s) { return make_float2(s, s); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b, exactly as a scalar subtraction (b * -1 is exact)
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, bc2(-1.f), a); }
-
-// e_I . v for the first direction of an opposite pair (which has a positive
-// component on both lattices' orderings)
-template <int LAT, int I>
-__device__ __forceinline__ float2 edot2(float2 vx, float2 vy, float2 vz) {
-  using L = Lat<LAT>;
-  constexpr int a = L::ex(I), b = L::ey(I), c = L::ez(I);
-  static_assert(a == 1 || b == 1 || c == 1, "pair leader without a positive component");
-  constexpr int first = a == 1 ? 0 : (b == 1 ? 1 : 2);
-  float2 r = first == 0 ? vx : (first == 1 ? vy : vz);
-  if constexpr (first < 1 && b == 1) r = add2(r, vy);
-  if constexpr (first < 2 && c == 1) r = add2(r, vz);
-  if constexpr (a == -1) r = sub2(r, vx);
-  if constexpr (b == -1) r = sub2(r, vy);
-  if constexpr (c == -1) r = sub2(r, vz);
-  return r;
-}
-
-// sum_a q_a,I v_a over the q-moment rows of direction I
-template <int LAT, int I>
-__device__ __forceinline__ float2 qdot2(const float2 (&v)[3]) {
-  constexpr int q0 = qrow<LAT>(0, I), q1 = qrow<LAT>(1, I);
-  constexpr int q2 = Lat<LAT>::D == 3 ? qrow<LAT>(2, I) : 0;
-  static_assert(q0 != 0 || q1 != 0 || q2 != 0, "direction without a q component");
-  float2 r;
-  if constexpr (q0 != 0) r = q0 == 1 ? v[0] : mul2(bc2((float)q0), v[0]);
-  if constexpr (q1 != 0) {
-    if constexpr (q0 != 0) r = fma2(bc2((float)q1), v[1], r);
-    else r = q1 == 1 ? v[1] : mul2(bc2((float)q1), v[1]);
-  }
-  if constexpr (q2 != 0) {
-    if constexpr (q0 != 0 || q1 != 0) r = fma2(bc2((float)q2), v[2], r);
-    else r = q2 == 1 ? v[2] : mul2(bc2((float)q2), v[2]);
-  }
-  return r;
-}
-
-// Collide two nodes at once (lane x and lane y of every float2): BGK, or MRT
-// whose only non-BGK rates are those of the q moments.  Same algebra as
-// `collide`: feq and Fbar split into parts even and odd in e over each
-// opposite pair (i, j),
-//   S  = w[drho - 1.5 u^2 + 4.5 (e.u)^2],  A  = 3 w (e.u),
-//   SF = w[9 (e.u)(e.F) - 3 u.F],           AF = 3 w (e.F),
-//   f_i* = (1 - omega) f_i + omega (S + A) + (1 - omega/2)(SF + AF),
-//   f_j* = (1 - omega) f_j + omega (S - A) + (1 - omega/2)(SF - AF),
-// and the q-moment correction (omega - s_q) m_q M_q,i / |M_q|^2 with m_q the
-// q moments of Delta + Fbar/2, i.e. of f_i - f_j - 2A + AF over the pairs.
-// Grouped for few operations:
-//   P = omega S + cforce SF = w B + A g,  B = omega (drho - 1.5 u^2) - 3 cforce u.F,
-//       g = 1.5 omega e.u + 3 cforce e.F,
-//   M = omega A + cforce AF = omega A + w (3 cforce e.F),
-//   m_q,a = sum_i q_a,i (f_i - f_j) + sum_b K_ab (F_b - 2 u_b)   (qk above).
-// With SL > 0 the populations and the force come in units of 2^-SL (FP16
-// storage's scaled deviations) and the results go out in them: everything
-// but the terms quadratic in u and F is linear, and those take their
-// constants times 2^-SL.  Every operation then gives 2^SL times its unscaled
-// result exactly (power-of-two scaling commutes with rounding), so the
-// stored values equal those of colliding the unscaled deviations.
-template <int LAT, int CM, int SL = 0>
-__device__ __forceinline__ void collide_x2(float2 (&f)[Lat<LAT>::Q], float2 Fx, float2 Fy,
-                                           float2 Fz, const Coll<float> &c) {
-  using L = Lat<LAT>;
-  constexpr int Q = L::Q;
-  static_assert(CM != CM_MRT, "general MRT rates run in the one-node kernel");
-  constexpr float wa = (float)L::w(1), wb = (float)L::w(Q - 1);
-  constexpr float kInv = 1.0f / (float)(1 << SL);  // exact
-  constexpr float kS = (float)(1 << SL);
-  float2 drho = f[0];
-  float2 jx = bc2(0.f), jy = bc2(0.f), jz = bc2(0.f);
-  float2 mq[3] = {bc2(0.f), bc2(0.f), bc2(0.f)};  // sum_i q_a,i (f_i - f_j)
-  static_for<Q>([&](auto ic) {
-    constexpr int i = decltype(ic)::value;
-    if constexpr (i > 0 && L::opp(i) > i) {
-      constexpr int j = L::opp(i);
-      static_assert(L::w(i) == L::w(1) || L::w(i) == L::w(Q - 1), "two weight classes");
-      drho = add2(drho, add2(f[i], f[j]));
-      const float2 d = sub2(f[i], f[j]);
-      if constexpr (L::ex(i) == 1) jx = add2(jx, d);
-      if constexpr (L::ex(i) == -1) jx = sub2(jx, d);
-      if constexpr (L::ey(i) == 1) jy = add2(jy, d);
-      if constexpr (L::ey(i) == -1) jy = sub2(jy, d);
-      if constexpr (L::ez(i) == 1) jz = add2(jz, d);
-      if constexpr (L::ez(i) == -1) jz = sub2(jz, d);
-      if constexpr (CM == CM_MRT_Q) {
-        static_for<L::D>([&](auto ac) {
-          constexpr int ax = decltype(ac)::value;
-          constexpr int q = qrow<LAT>(ax, i);
-          if constexpr (q == 1) mq[ax] = add2(mq[ax], d);
-          else if constexpr (q == -1) mq[ax] = sub2(mq[ax], d);
-          else if constexpr (q != 0) mq[ax] = fma2(bc2((float)q), d, mq[ax]);
-        });
-      }
-    }
-  });
-  const float2 half = bc2(0.5f);
-  const float2 ux = fma2(half, Fx, jx), uy = fma2(half, Fy, jy), uz = fma2(half, Fz, jz);
-  const float2 uu = fma2(uz, uz, fma2(uy, uy, mul2(ux, ux)));
-  const float2 uF = fma2(uz, Fz, fma2(uy, Fy, mul2(ux, Fx)));
-  const float2 base = fma2(bc2(-1.5f * kInv), uu, drho);
-  const float2 om = bc2(c.omega), omc = bc2(c.omc);
-  // the constants of the terms quadratic in u and F carry 2^-SL: 1.5 omega,
-  // 3 cforce (each the power-of-two multiple of its unscaled rounding)
-  const float om15 = c.omega * (1.5f * kInv), cf3 = c.cforce * (3.f * kInv);
-  const float2 B = fma2(bc2(-cf3), uF, mul2(om, base));
-  {
-    constexpr float w0 = (float)L::w(0);
-    f[0] = fma2(omc, f[0], mul2(bc2(w0), B));
-  }
-  const float2 Ba = mul2(bc2(wa), B), Bb = mul2(bc2(wb), B);
-  static_for<Q>([&](auto ic) {
-    constexpr int i = decltype(ic)::value;
-    if constexpr (i > 0 && L::opp(i) > i) {
-      constexpr int j = L::opp(i);
-      constexpr bool ca = L::w(i) == L::w(1);
-      constexpr float w = (float)L::w(i), w3 = (float)(3.0 * L::w(i));
-      const float2 eu = edot2<LAT, i>(ux, uy, uz);
-      const float2 eF = edot2<LAT, i>(Fx, Fy, Fz);
-      const float2 A = mul2(bc2(w3), eu);
-      const float2 t = mul2(bc2(cf3), eF);     // 3 cforce e.F (times 2^-SL)
-      const float2 g = fma2(bc2(om15), eu, t);  // 1.5 omega e.u + 3 cforce e.F
-      const float2 P = fma2(A, g, ca ? Ba : Bb);
-      const float2 M = fma2(om, A, mul2(bc2(w * kS), t));
-      f[i] = fma2(omc, f[i], add2(P, M));
-      f[j] = fma2(omc, f[j], sub2(P, M));
-    }
-  });
-  if constexpr (CM == CM_MRT_Q) {
-    // the pairs' -2 A + AF terms of the q moments, then the correction: all q
-    // rows share one rate; the rows are odd in e, so the opposite direction
-    // of a pair gets the negative correction
-    const float2 fu[3] = {fma2(bc2(-2.f), ux, Fx), fma2(bc2(-2.f), uy, Fy), fma2(bc2(-2.f), uz, Fz)};
-    static_for<L::D>([&](auto ac) {
-      constexpr int ax = decltype(ac)::value;
-      static_for<L::D>([&](auto bc) {
-        constexpr int b = decltype(bc)::value;
-        constexpr float K = (float)qk<LAT>(ax, b);
-        if constexpr (K != 0.f) mq[ax] = fma2(bc2(K), fu[b], mq[ax]);
-      });
-    });
-    const float2 k = bc2(c.ds[4] * (float)(1.0 / mnorm<LAT>(4)));
-    const float2 aq[3] = {mul2(k, mq[0]), mul2(k, mq[1]), mul2(k, mq[2])};
-    static_for<Q>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      if constexpr (i > 0 && L::opp(i) > i) {
-        constexpr int j = L::opp(i);
-        const float2 cq = qdot2<LAT, i>(aq);
-        f[i] = add2(f[i], cq);
-        f[j] = sub2(f[j], cq);
-      }
-    });
-  }
-}
 
 // ---------------------------------------------------------------- storage
 // W words of a direction's vector; node k of the vector is word k (FP32) or
@@ -354,7 +197,7 @@ __device__ __forceinline__ void vec_collide_store(const KArgs &a, Words<W> (&v)[
     const float g0 = (flag(2 * p) & FL_NOG) ? 0.f : 1.f;
     const float g1 = (flag(2 * p + 1) & FL_NOG) ? 0.f : 1.f;
     if constexpr (PACKED) {
-      collide_x2<LAT, CM, SL>(f, make_float2(g0 * gx, g1 * gx), make_float2(g0 * gy, g1 * gy),
+      collide_two_rate<LAT, CM, SL, (sizeof(S) > 2), float2, float>(f, make_float2(g0 * gx, g1 * gx), make_float2(g0 * gy, g1 * gy),
                               make_float2(g0 * gz, g1 * gz), c);
     } else {
       float fa[Q], fb[Q];
@@ -363,8 +206,8 @@ __device__ __forceinline__ void vec_collide_store(const KArgs &a, Words<W> (&v)[
         fa[i] = f[i].x;
         fb[i] = f[i].y;
       });
-      collide<LAT, CM, float>(fa, g0 * gx, g0 * gy, g0 * gz, c);
-      collide<LAT, CM, float>(fb, g1 * gx, g1 * gy, g1 * gz, c);
+      collide<LAT, CM, S, float>(fa, g0 * gx, g0 * gy, g0 * gz, c);
+      collide<LAT, CM, S, float>(fb, g1 * gx, g1 * gy, g1 * gz, c);
       static_for<Q>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         f[i] = make_float2(fa[i], fb[i]);
@@ -455,15 +298,24 @@ __device__ __forceinline__ void bulk_vec_update(const KArgs &a, unsigned t, unsi
 }
 
 
+// Registers a thread of the 2-word kernels: FP32 80 (6 blocks of 128 per SM),
+// BF16 112, FP16 128.  Measured on 128^3 / 160^3 / 192^3 lattices without
+// solids, us per step: FP32 packed 54.2 / 102.5 / 174 at 64 registers (it
+// spills), 48.1 / 92.2 / 157.3 at 72, 47.2 / 90.7 / 154.6 at 80, 47.3 / 90.7 /
+// 154.1 at 96; FP32 node by node 48.1 / 92.6 / 158.2 at 64, 47.8 / 91.9 /
+// 156.8 at 72.  BF16 29.8 / 55.3 / 91.6 at 96, 26.7 / 49.0 / 82.0 at 112,
+// 26.8 / 50.7 / 84.4 at 128; FP16 30.8 / 57.3 / 95.8 at 96, 27.8 / 51.5 / 87.8
+// at 112, 26.7 / 49.5 / 84.0 at 128.  4-word vectors are left unbounded.
+template <typename S, int W> constexpr int vec_regs() {
+  return W == 4 ? 255 : sizeof(S) == 4 ? 80 : std::is_same<S, __nv_bfloat16>::value ? 112 : 128;
+}
+
 // One thread per vector.  (A persistent grid walking the lattice measured
 // slower: it holds more registers and leaves the boundary kernels less room;
 // so did one that kept the next vector's loads in flight through a cp.async
-// ring in shared memory.)  The 8-byte 16-bit kernels are held to 128
-// registers, 4 blocks of 128 per SM (130 unbounded: 3 blocks); the FP32
-// node-by-node kernel to 64, 8 blocks of 128 per SM (88 unbounded: 5 blocks),
-// whose extra warps hide more of the boundary kernel's share of the SMs.
+// ring in shared memory.)
 template <int LAT, int CM, typename S, int W, bool PACKED>
-__global__ void __launch_bounds__(256, (sizeof(S) == 2 && W == 2) ? 2 : ((sizeof(S) == 4 && W == 2 && !PACKED) ? 4 : 0))
+__global__ void __maxnreg__((vec_regs<S, W>()))
     k_bulk_vec(const KArgs a) {
   constexpr int V = W * VecS<S>::per_word;
   bulk_vec_update<LAT, CM, S, W, PACKED>(a, blockIdx.x * blockDim.x + threadIdx.x,
@@ -476,11 +328,9 @@ __global__ void __launch_bounds__(256, (sizeof(S) == 2 && W == 2) ? 2 : ((sizeof
 // arguments stay constant-bank operands (indexing the argument array by a
 // run-time k holds them in registers: 92 instead of 80, one block per SM
 // fewer).
-// Register limits near the single-lattice kernel's: 80 for the FP32
-// node-by-node variant (6 blocks of 128 per SM), 128 for the 2-word 16-bit
-// ones; 4-word vectors are left unbounded.
+// The single-lattice kernel's register limits.
 template <int LAT, int CM, typename S, int W, bool PACKED>
-__global__ void __launch_bounds__(256, W == 4 ? 1 : (sizeof(S) == 4 && !PACKED) ? 3 : 2)
+__global__ void __maxnreg__((vec_regs<S, W>()))
     k_bulk_vec_group(const __grid_constant__ GroupArgs g) {
   constexpr int V = W * VecS<S>::per_word;
   const int b = (int)blockIdx.x;
