@@ -1281,6 +1281,7 @@ lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
   a.src = ctx->f[cur];
   a.dst = ctx->f[nxt];
   a.force_acc = acc;
+  a.rev = cur;  // alternates from step to step
   // fork: the boundary nodes (and the IBM pre-pass that feeds them) on the
   // auxiliary stream, the bulk nodes on the main stream; they read the same
   // f*(t) and write disjoint nodes of f*(t+1)

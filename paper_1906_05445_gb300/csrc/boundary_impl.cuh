@@ -939,14 +939,33 @@ inline int div_up(long long a, int b) { return (int)((a + b - 1) / b); }
 // or 4; 0 = 2) and the node-pair collision packed (bulk_vec_packed 1, and -1,
 // the default: figures at vec_regs) or node by node (0).  Returns false where nx or the direction stride is not a
 // multiple of the V nodes of a vector.
+//
+// Both arrays together up to kReuseBytes (1.5 times the 129 MB L2): the reads
+// are evict-first, so that L2 keeps what the step writes, which the next step
+// reads.  us per step without / with it, lattices without solids: FP32 96^3
+// (134 MB) 20.6 / 18.5, 112^3 (213 MB) 32.6 / 30.9, 128^3 (319 MB) 48.0 / 47.2,
+// 160^3 (623 MB) 92.5 / 93.2; FP16 112^3 (107 MB) 18.5 / 16.5, 128^3 (159 MB)
+// 26.7 / 24.7, 192^3 (538 MB) 84.0 / 84.6.  The line lies below the sizes that
+// gain little alone: two 128^3 FP32 lattices stepped side by side on their own
+// streams lose 4% with it (100.0 -> 104.0 us per step of both).
+constexpr long long kReuseBytes = 192LL << 20;
 template <int LAT, int CM, typename S, int W>
 bool launch_bulk_vec_w(const KArgs &a, int want, bool packed, cudaStream_t st) {
   constexpr int V = W * VecS<S>::per_word;
   if (a.nx % V != 0 || a.fs % V != 0) return false;
   const int nt = (int)(a.N / V);
   const int grid = div_up(nt, want);
-  if (packed) k_bulk_vec<LAT, CM, S, W, true><<<grid, want, 0, st>>>(a);
-  else k_bulk_vec<LAT, CM, S, W, false><<<grid, want, 0, st>>>(a);
+  // the hint is built for the default shape only
+  if (W == 2 && packed) {
+    if (2 * Lat<LAT>::Q * a.fs * (long long)sizeof(S) <= kReuseBytes)
+      k_bulk_vec<LAT, CM, S, W, true, W == 2><<<grid, want, 0, st>>>(a);
+    else
+      k_bulk_vec<LAT, CM, S, W, true, false><<<grid, want, 0, st>>>(a);
+  } else if (packed) {
+    k_bulk_vec<LAT, CM, S, W, true, false><<<grid, want, 0, st>>>(a);
+  } else {
+    k_bulk_vec<LAT, CM, S, W, false, false><<<grid, want, 0, st>>>(a);
+  }
   return true;
 }
 template <int LAT, int CM, typename S>

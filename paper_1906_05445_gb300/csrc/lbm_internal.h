@@ -94,6 +94,7 @@ struct KArgs {
   int bulk_vec_words;  // vector sweep: 32-bit words per thread and direction (2 or 4; 0 = 2)
   int bulk_vec_packed; // vector sweep: 1 (and -1, the default) packed FP32x2 collision of
                        // node pairs, 0 node by node
+  int rev;             // bulk sweep: blocks walk the lattice from its end
   int *wait_err;       // set to 1 by a kernel whose wait for its asynchronous copies gave up
   // domain faces x-, x+, y-, y+, z-, z+ (LBM_FACE_*), their wall velocities,
   // the nodes next to a non-periodic face, and the outflow face's kept

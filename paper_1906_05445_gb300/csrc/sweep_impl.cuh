@@ -131,7 +131,8 @@ __device__ __forceinline__ void scatter(S *__restrict__ dst, long long fs,
 // direction's loads and stores of a warp are contiguous
 template <int LAT, int CM, typename S, typename T, int HINT>
 __global__ void __launch_bounds__(512) k_bulk_sweep(const KArgs a) {
-  const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
+  // from the lattice's end every other step (see k_bulk_vec)
+  const unsigned n = (a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
   if (n >= (unsigned)a.N) return;
   // plain fluid nodes; nodes inside an IBM solid (FL_NOG) also run here,
   // without the external force, and so do nodes refilled this step (FL_NEW)

@@ -28,14 +28,18 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 template <int W> struct Words {
   uint32_t w[W];
 };
-template <int W> __device__ __forceinline__ Words<W> ld_words(const void *p) {
+// ONCE: the line is not needed again before the array is overwritten (L2
+// evicts it first); see launch_bulk_vec_w.
+template <int W, bool ONCE = false> __device__ __forceinline__ Words<W> ld_words(const void *p) {
   Words<W> r;
   if constexpr (W == 4) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+    const uint4 *q = reinterpret_cast<const uint4 *>(p);
+    const uint4 v = ONCE ? __ldcs(q) : __ldg(q);
     r.w[0] = v.x, r.w[1] = v.y, r.w[2] = v.z, r.w[3] = v.w;
   } else {
     static_assert(W == 2, "8- or 16-byte vectors");
-    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+    const uint2 *q = reinterpret_cast<const uint2 *>(p);
+    const uint2 v = ONCE ? __ldcs(q) : __ldg(q);
     r.w[0] = v.x, r.w[1] = v.y;
   }
   return r;
@@ -240,7 +244,7 @@ __device__ __forceinline__ void vec_collide_store(const KArgs &a, Words<W> (&v)[
 // Thread t updates the vector of nodes [V t, V t + V), pulling the shifted
 // rows straight from global memory.  Every lane of the warp calls this
 // (threads past the end with t >= nt), for the shuffles.
-template <int LAT, int CM, typename S, int W, bool PACKED>
+template <int LAT, int CM, typename S, int W, bool PACKED, bool ONCE = false>
 __device__ __forceinline__ void bulk_vec_update(const KArgs &a, unsigned t, unsigned nt) {
   using L = Lat<LAT>;
   using VS = VecS<S>;
@@ -276,7 +280,7 @@ __device__ __forceinline__ void bulk_vec_update(const KArgs &a, unsigned t, unsi
   static_for<Q>([&](auto ic) {
     constexpr int i = decltype(ic)::value;
     const S *row = src + (long long)i * a.fs + r[1 - L::ez(i)][1 - L::ey(i)];
-    v[i] = ld_words<W>(row + x0);
+    v[i] = ld_words<W, ONCE>(row + x0);
     edge[i] = 0u;
     if constexpr (L::ex(i) == 1) {
       if (!lnb) edge[i] = VS::left_word(row + xl);
@@ -314,12 +318,17 @@ template <typename S, int W> constexpr int vec_regs() {
 // slower: it holds more registers and leaves the boundary kernels less room;
 // so did one that kept the next vector's loads in flight through a cp.async
 // ring in shared memory.)
-template <int LAT, int CM, typename S, int W, bool PACKED>
+// Blocks walk the lattice from its end when a.rev is set (every other step):
+// a step then starts on the nodes that the previous one wrote last, which L2
+// still holds, instead of on those it has already evicted.  128^3 without
+// solids, FP32: 50.9 -> 48.0 us per step (and 47.2 with evict-first reads,
+// ONCE); 112^3 36.1 -> 32.6 (30.9); FP16 128^3 28.8 -> 26.7 (24.7).
+template <int LAT, int CM, typename S, int W, bool PACKED, bool ONCE>
 __global__ void __maxnreg__((vec_regs<S, W>()))
     k_bulk_vec(const KArgs a) {
   constexpr int V = W * VecS<S>::per_word;
-  bulk_vec_update<LAT, CM, S, W, PACKED>(a, blockIdx.x * blockDim.x + threadIdx.x,
-                                         (unsigned)a.N / V);
+  const unsigned b = a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  bulk_vec_update<LAT, CM, S, W, PACKED, ONCE>(a, b * blockDim.x + threadIdx.x, (unsigned)a.N / V);
 }
 
 // The same update for several lattices in one grid: block b belongs to the
@@ -338,7 +347,10 @@ __global__ void __maxnreg__((vec_regs<S, W>()))
     constexpr int k = decltype(kc)::value;
     if (k < g.n && b >= g.block_start[k] && b < g.block_start[k + 1])
       bulk_vec_update<LAT, CM, S, W, PACKED>(
-          g.a[k], (unsigned)(b - g.block_start[k]) * blockDim.x + threadIdx.x, (unsigned)g.a[k].N / V);
+          g.a[k],
+          (unsigned)(g.a[k].rev ? g.block_start[k + 1] - 1 - b : b - g.block_start[k]) * blockDim.x +
+              threadIdx.x,
+          (unsigned)g.a[k].N / V);
   });
 }
 
