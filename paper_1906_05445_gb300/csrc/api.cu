@@ -1426,8 +1426,7 @@ void run_query(lbm_ctx *ctx, KArgs a) {
     sweep(ctx, OP_LOCAL_QUERY, a);
   } else {
     a.local_gather = 0;
-    sweep(ctx, OP_BULK_QUERY, a);
-    sweep(ctx, OP_LIST_QUERY, a);
+    sweep(ctx, OP_QUERY, a);
     if (ctx->nface) sweep(ctx, OP_FACE_QUERY, a);
   }
 }

@@ -53,78 +53,102 @@ __device__ __forceinline__ T ibb_value(const KArgs &a, const S *__restrict__ src
   return v;
 }
 
-// FP64 outputs of a query at one node from pre-collision deviations f.
+// FP64 outputs of a query at one node from pre-collision deviations f.  The
+// second moments of feq are closed forms, sum e_a e_b feq_i = drho/3 delta_ab
+// + u_a u_b on both lattices, so the non-equilibrium stress is a few sums of
+// the pairs' f_i + f_j: about 90 FP64 operations per D3Q19 node against some
+// 700 when feq_i is formed and multiplied out per direction, which GB300's
+// FP64 rate makes the query's bound (96^3 FP64 strain rate: 670 us before).
 template <int LAT, typename T>
 __device__ __forceinline__ void write_fields(const KArgs &a, long long n,
                                              const T (&f)[Lat<LAT>::Q], T Fx,
                                              T Fy, T Fz) {
   using L = Lat<LAT>;
   constexpr int Q = L::Q, D = L::D;
-  double fd[Q];
-  double drho = 0, j[3] = {0, 0, 0};
-#pragma unroll
-  for (int i = 0; i < Q; i++) {
-    fd[i] = (double)f[i];
-    drho += fd[i];
-    j[0] += L::ex(i) * fd[i];
-    j[1] += L::ey(i) * fd[i];
-    j[2] += L::ez(i) * fd[i];
-  }
-  const double F[3] = {(double)Fx, (double)Fy, (double)Fz};
-  const double u[3] = {j[0] + 0.5 * F[0], j[1] + 0.5 * F[1], j[2] + 0.5 * F[2]};
-  if (a.out_rho) a.out_rho[n] = 1.0 + drho;
-  if (a.out_u)
-    for (int c = 0; c < D; c++) a.out_u[c * a.N + n] = u[c];
+  const bool stress = a.out_S || a.out_stress || a.out_eps;
   if (a.out_f)
-#pragma unroll
-    for (int i = 0; i < Q; i++) a.out_f[(long long)i * a.N + n] = L::w(i) + fd[i];
-  if (a.out_S || a.out_stress || a.out_eps) {
-    const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    double P[3][3];
-    for (int p = 0; p < 3; p++)
-      for (int q = 0; q < 3; q++) P[p][q] = 0.5 * (F[p] * u[q] + u[p] * F[q]);
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      const double neq = fd[i] - feq_dev<LAT, double>(i, drho, u[0], u[1], u[2], uu);
-      const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
-      for (int p = 0; p < 3; p++)
-        for (int q = 0; q < 3; q++) P[p][q] += neq * e[p] * e[q];
-    }
-    double tr = 0;
-    for (int p = 0; p < D; p++) tr += P[p][p];
-    const int nc = D == 2 ? 3 : 6;
-    const int ca[6] = {0, 1, D == 2 ? 0 : 2, 0, 1, 0};
-    const int cb[6] = {0, 1, D == 2 ? 1 : 2, 1, 2, 2};
-    double ss = 0;
-    for (int c = 0; c < nc; c++) {
-      const int p = ca[c], q = cb[c];
-      const double iso = p == q ? tr / D : 0.0;
-      const double S = -1.5 * (a.omega * (P[p][q] - iso) + a.s_bulk * iso);
-      if (a.out_S) a.out_S[c * a.N + n] = S;
-      if (a.out_stress)
-        a.out_stress[c * a.N + n] = (p == q ? -(1.0 + drho) / 3.0 : 0.0) + 2.0 * a.nu * S;
-      ss += (p == q ? 1.0 : 2.0) * S * S;
-    }
-    if (a.out_eps) a.out_eps[n] = 2.0 * a.nu * ss;
+    static_for<Q>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      a.out_f[(long long)i * a.N + n] = L::w(i) + (double)f[i];
+    });
+  if (!a.out_rho && !a.out_u && !stress) return;
+  const double F[3] = {(double)Fx, (double)Fy, (double)Fz};
+  // momentum from the pairs' differences; an axis pair comes first and starts
+  // each sum
+  double u[3] = {0, 0, 0};
+  if (a.out_u || stress) {
+    static_for<Q>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      if constexpr (i > 0 && L::opp(i) > i) {
+        const double d = (double)f[i] - (double)f[L::opp(i)];
+        static_for<D>([&](auto ac) {
+          constexpr int c = decltype(ac)::value;
+          constexpr int e = ecomp<LAT>(c, i);
+          if constexpr (e != 0) {
+            if constexpr (enorm2<LAT>(i) == 1) u[c] = d;
+            else if constexpr (e == 1) u[c] += d;
+            else u[c] -= d;
+          }
+        });
+      }
+    });
+    for (int c = 0; c < D; c++) u[c] += 0.5 * F[c];
+    if (a.out_u)
+      for (int c = 0; c < D; c++) a.out_u[c * a.N + n] = u[c];
   }
+  if (!a.out_rho && !stress) return;
+  // density and second moments from the pairs' sums
+  double drho = (double)f[0];
+  double Pd[3] = {0, 0, 0};  // xx, yy, zz
+  double Po[3] = {0, 0, 0};  // xy, yz, xz
+  static_for<Q>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    if constexpr (i > 0 && L::opp(i) > i) {
+      const double sp = (double)f[i] + (double)f[L::opp(i)];
+      drho += sp;
+      static_for<D>([&](auto ac) {
+        constexpr int c = decltype(ac)::value;
+        if constexpr (ecomp<LAT>(c, i) != 0) {
+          if constexpr (enorm2<LAT>(i) == 1) Pd[c] = sp;
+          else Pd[c] += sp;
+        }
+      });
+      if constexpr (enorm2<LAT>(i) == 2) {
+        constexpr int p = L::ex(i) ? 0 : 1, q = L::ez(i) ? 2 : 1;
+        constexpr int k = p == 1 ? 1 : (q == 1 ? 0 : 2);
+        if constexpr (ecomp<LAT>(p, i) * ecomp<LAT>(q, i) > 0) Po[k] += sp;
+        else Po[k] -= sp;
+      }
+    }
+  });
+  if (a.out_rho) a.out_rho[n] = 1.0 + drho;
+  if (!stress) return;
+  // P = Pi^neq + (F u + u F) / 2
+  double tr = 0;
+  for (int c = 0; c < D; c++) {
+    Pd[c] = Pd[c] - drho * (1.0 / 3.0) + u[c] * (F[c] - u[c]);
+    tr += Pd[c];
+  }
+  constexpr int pa[3] = {0, 1, 0}, pb[3] = {1, 2, 2};
+  for (int k = 0; k < (D == 2 ? 1 : 3); k++)
+    Po[k] += 0.5 * (F[pa[k]] * u[pb[k]] + u[pa[k]] * F[pb[k]]) - u[pa[k]] * u[pb[k]];
+  // S = -1.5 [omega (P - tr P / D) + s_bulk tr P / D]
+  const double iso = tr * (1.0 / D), ko = -1.5 * a.omega, ki = -1.5 * (a.s_bulk - a.omega) * iso;
+  double ss = 0;
+  constexpr int nc = D == 2 ? 3 : 6;
+#pragma unroll
+  for (int c = 0; c < nc; c++) {
+    const bool dg = c < D;
+    const double S = dg ? ko * Pd[c] + ki : ko * Po[c - D];
+    if (a.out_S) a.out_S[c * a.N + n] = S;
+    if (a.out_stress)
+      a.out_stress[c * a.N + n] = (dg ? -(1.0 + drho) * (1.0 / 3.0) : 0.0) + 2.0 * a.nu * S;
+    ss += (dg ? 1.0 : 2.0) * S * S;
+  }
+  if (a.out_eps) a.out_eps[n] = 2.0 * a.nu * ss;
 }
 
 // ---------------------------------------------------------------- kernels
-template <int LAT, typename S>
-__global__ void __launch_bounds__(512) k_bulk_query(const KArgs a) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y, z = blockIdx.z;
-  if (x >= a.nx) return;
-  const long long n = x + (long long)a.nx * (y + (long long)a.ny * z);
-  const uint8_t fl = a.flags[n];
-  if (fl & (uint8_t)~(FL_NOG | FL_NEW)) return;
-  double f[Lat<LAT>::Q];
-  gather_pull<LAT, S, double>((const S *)a.src, a.fs, x, y, z, a.nx, a.ny, a.nz,
-                              a.inv_scale, f);
-  const double gon = (fl & FL_NOG) ? 0.0 : 1.0;
-  write_fields<LAT, double>(a, n, f, gon * a.g[0], gon * a.g[1], gon * a.g[2]);
-}
-
 // Density and velocity only, for FP32 and 16-bit storage: the same moments
 // as write_fields (u = sum e_i d_i + F / 2, rho = 1 + sum d_i) summed in FP32
 // arithmetic over the stored values, written as FP64.  GB300's FP64 rate
@@ -132,15 +156,10 @@ __global__ void __launch_bounds__(512) k_bulk_query(const KArgs a) {
 // about the FP32 rounding of the sums (1e-7 of the largest term), well
 // inside the storage's own error.
 template <int LAT, typename S>
-__global__ void __launch_bounds__(512) k_bulk_query_u(const KArgs a) {
+__device__ __forceinline__ void bulk_query_u(const KArgs &a, long long n, uint8_t fl, int x, int y,
+                                             int z) {
   using L = Lat<LAT>;
   constexpr int Q = L::Q, D = L::D;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y, z = blockIdx.z;
-  if (x >= a.nx) return;
-  const long long n = x + (long long)a.nx * (y + (long long)a.ny * z);
-  const uint8_t fl = a.flags[n];
-  if (fl & (uint8_t)~(FL_NOG | FL_NEW)) return;
   float f[Q];
   gather_pull<LAT, S, float>((const S *)a.src, a.fs, x, y, z, a.nx, a.ny, a.nz, a.inv_scale_f, f);
   float drho = 0.f, j[3] = {0.f, 0.f, 0.f};
@@ -164,8 +183,79 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Boundary-node sweep (MODE 0) or query (MODE 1): one thread per list node.
-template <int LAT, int CM, typename S, typename T, typename LT, int MODE>
+// Query at list node t: the pre-collision populations pulled from a.src with
+// the bounce-back rules (Eq. 16: the kept ones), in FP64.
+template <int LAT, typename S, typename LT>
+__device__ __forceinline__ void list_query_node(const KArgs &a, int t) {
+  constexpr int Q = Lat<LAT>::Q;
+  const long long n = a.list_node[t];
+  const uint8_t fl = a.flags[n];
+  if (fl & FL_FACE) return;
+  const double isc = a.inv_scale;
+  const S *__restrict__ src = (const S *)a.src;
+  double f[Q];
+  if (a.zy_pre) {
+#pragma unroll
+    for (int i = 0; i < Q; i++) f[i] = (double)((const LT *)a.zy_pre)[(long long)i * a.fs + n];
+  } else {
+    const uint32_t mask = a.list_mask[t];
+    int link = a.list_link[t];
+    int x, y, z;
+    node_xyz(n, a.nx, a.ny, x, y, z);
+    gather_pull<LAT, S, double>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
+    if (mask) {
+#pragma unroll
+      for (int i = 1; i < Q; i++) {
+        if (!((mask >> i) & 1u)) continue;
+        double fs;
+        f[i] = ibb_value<LAT, S, double, LT>(a, src, i, x, y, z, n, link, isc, fs);
+        link++;
+      }
+    }
+  }
+  double Fx, Fy, Fz;
+  node_force<double, LT>(a, n, fl, Fx, Fy, Fz);
+  write_fields<LAT, double>(a, n, f, Fx, Fy, Fz);
+}
+
+// A query in one launch: the first list_blocks blocks take the list nodes
+// (long chains of dependent loads, a thread per node), the others the plain
+// nodes, a thread each; the list blocks start first and run beside the rest
+// (as a launch of their own they took 46 us after a 96^3 FP64 lattice's plain
+// nodes).  U32: density and velocity of FP32 and 16-bit storage.
+template <int LAT, typename S, typename LT, bool U32>
+__global__ void __launch_bounds__(128) k_query(const KArgs a, int list_blocks) {
+  const int b = (int)blockIdx.x - list_blocks;
+  if (b < 0) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    int cnt = a.counts[0];
+    if (cnt > a.list_cap) cnt = a.list_cap;
+    if (t < cnt) list_query_node<LAT, S, LT>(a, t);
+    return;
+  }
+  const long long n = (long long)b * blockDim.x + threadIdx.x;
+  if (n >= a.N) return;
+  const uint8_t fl = a.flags[n];
+  if (fl & (uint8_t)~(FL_NOG | FL_NEW)) return;
+  int x, y, z;
+  {
+    const unsigned yz = (unsigned)n / (unsigned)a.nx;
+    x = (int)((unsigned)n - yz * (unsigned)a.nx);
+    z = (int)(yz / (unsigned)a.ny);
+    y = (int)(yz - (unsigned)z * (unsigned)a.ny);
+  }
+  if constexpr (U32) {
+    bulk_query_u<LAT, S>(a, n, fl, x, y, z);
+  } else {
+    double f[Lat<LAT>::Q];
+    gather_pull<LAT, S, double>((const S *)a.src, a.fs, x, y, z, a.nx, a.ny, a.nz, a.inv_scale, f);
+    const double gon = (fl & FL_NOG) ? 0.0 : 1.0;
+    write_fields<LAT, double>(a, n, f, gon * a.g[0], gon * a.g[1], gon * a.g[2]);
+  }
+}
+
+// Boundary-node sweep: one thread per list node.
+template <int LAT, int CM, typename S, typename T>
 __global__ void __launch_bounds__(128) k_list(const KArgs a) {
   using L = Lat<LAT>;
   constexpr int Q = L::Q;
@@ -191,28 +281,22 @@ __global__ void __launch_bounds__(128) k_list(const KArgs a) {
     int x, y, z;
     node_xyz(n, a.nx, a.ny, x, y, z);
     T f[Q];
-    const bool zy_query = MODE == 1 && a.zy_pre && !a.local_gather;
-    if (a.local_gather)
-      gather_local<LAT, S, T>(src, a.fs, n, isc, f);
-    else if (zy_query)  // Eq. 16 keeps the current pre-collision values here
-      for (int i = 0; i < Q; i++) f[i] = (T)((const LT *)a.zy_pre)[(long long)i * a.fs + n];
-    else
-      gather_pull<LAT, S, T>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
-    if (mask && !a.local_gather && !zy_query) {
+    gather_pull<LAT, S, T>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
+    if (mask) {
 #pragma unroll
       for (int i = 1; i < Q; i++) {
         if (!((mask >> i) & 1u)) continue;
         T fs;
-        const T v = ibb_value<LAT, S, T, LT>(a, src, i, x, y, z, n, link, isc, fs);
+        const T v = ibb_value<LAT, S, T, T>(a, src, i, x, y, z, n, link, isc, fs);
         f[i] = v;
-        if (MODE == 0) {
+        {
           const int s = a.links.sid[link];
           if (sa < 0) sa = s;
           const T e[3] = {(T)L::ex(i), (T)L::ey(i), (T)L::ez(i)};
-          const LT *uw0 = (const LT *)a.links.uw[0], *uw1 = (const LT *)a.links.uw[1],
-                   *uw2 = (const LT *)a.links.uw[2];
-          const LT *ar0 = (const LT *)a.links.arm[0], *ar1 = (const LT *)a.links.arm[1],
-                   *ar2 = (const LT *)a.links.arm[2];
+          const T *uw0 = (const T *)a.links.uw[0], *uw1 = (const T *)a.links.uw[1],
+                   *uw2 = (const T *)a.links.uw[2];
+          const T *ar0 = (const T *)a.links.arm[0], *ar1 = (const T *)a.links.arm[1],
+                   *ar2 = (const T *)a.links.arm[2];
           const T uw[3] = {(T)uw0[link], (T)uw1[link], (T)uw2[link]};
           const T r[3] = {(T)ar0[link], (T)ar1[link], (T)ar2[link]};
           if (s == sa) {
@@ -244,23 +328,19 @@ __global__ void __launch_bounds__(128) k_list(const KArgs a) {
         }
         link++;
       }
-      if (MODE == 0 && sa >= 0)
+      if (sa >= 0)
         for (int c = 0; c < 6; c++) acc[c] = a.list_cst[c * a.list_cap + t] + (double)dacc[c];
     }
-    if (MODE == 0 && a.zy_pre)  // the next step's Eq. 16 reads them
-      for (int i = 0; i < Q; i++) ((LT *)a.zy_pre)[(long long)i * a.fs + n] = (LT)f[i];
+    if (a.zy_pre)  // the next step's Eq. 16 reads them
+      for (int i = 0; i < Q; i++) ((T *)a.zy_pre)[(long long)i * a.fs + n] = f[i];
     const uint8_t fl = a.flags[n];
     T Fx, Fy, Fz;
-    node_force<T, LT>(a, n, fl, Fx, Fy, Fz);
-    if (MODE == 0) {
-      const Coll<T> c = make_coll<LAT, T>(a);
-      collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
-      scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
-    } else {
-      write_fields<LAT, T>(a, n, f, Fx, Fy, Fz);
-    }
+    node_force<T, T>(a, n, fl, Fx, Fy, Fz);
+    const Coll<T> c = make_coll<LAT, T>(a);
+    collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
+    scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
   }
-  if (MODE == 0 && a.force_acc) {
+  if (a.force_acc) {
     const int lane = threadIdx.x & 31;
     for (int s = 0; s < a.nsolids; s++) {
       if (!__any_sync(0xffffffffu, sa == s)) continue;
@@ -1080,8 +1160,6 @@ bool launch_group_precision(const KArgs *as, int n, int lattice, int collision, 
 template <int LAT, int CM, typename S, typename T>
 void launch_one(SweepOp op, const KArgs &a, cudaStream_t st) {
   const int want = a.bulk_block > 0 ? a.bulk_block : 128;
-  const int bx = a.nx >= want ? want : ((a.nx + 31) / 32) * 32;
-  const dim3 gbulk(div_up(a.nx, bx), a.ny, a.nz);
   const int lc = a.list_cap > 0 ? a.list_cap : 1;
   switch (op) {
   case OP_BULK_SWEEP:
@@ -1099,15 +1177,18 @@ void launch_one(SweepOp op, const KArgs &a, cudaStream_t st) {
     default: k_bulk_sweep<LAT, CM, S, T, 0><<<div_up(a.N, want), want, 0, st>>>(a);
     }
     break;
-  case OP_BULK_QUERY:
+  case OP_QUERY: {
+    const int lb = a.list_cap > 0 ? div_up(a.list_cap, 128) : 0;
+    const int grid = lb + div_up(a.N, 128);
     if constexpr (std::is_same<T, float>::value) {
       if (!a.out_S && !a.out_stress && !a.out_eps && !a.out_f) {
-        k_bulk_query_u<LAT, S><<<gbulk, bx, 0, st>>>(a);
+        k_query<LAT, S, T, true><<<grid, 128, 0, st>>>(a, lb);
         break;
       }
     }
-    k_bulk_query<LAT, S><<<gbulk, bx, 0, st>>>(a);
+    k_query<LAT, S, T, false><<<grid, 128, 0, st>>>(a, lb);
     break;
+  }
   case OP_LIST_SWEEP:
     if (a.list_cap > 0) {
       if (CM != CM_MRT && !a.list_thread) {
@@ -1118,15 +1199,12 @@ void launch_one(SweepOp op, const KArgs &a, cudaStream_t st) {
         // general MRT rates, or IBM band nodes (no cut links): a thread per
         // node (small blocks spread the boundary nodes over many SMs)
         const int lb = a.list_block > 0 && a.list_block <= 128 ? a.list_block : 64;
-        k_list<LAT, CM, S, T, T, 0><<<div_up(lc, lb), lb, 0, st>>>(a);
+        k_list<LAT, CM, S, T><<<div_up(lc, lb), lb, 0, st>>>(a);
       }
     }
     break;
   case OP_ZY_SEED:
     if (a.list_cap > 0 && a.zy_pre) k_zy_seed<LAT, S, T><<<div_up(lc, 128), 128, 0, st>>>(a);
-    break;
-  case OP_LIST_QUERY:
-    if (a.list_cap > 0) k_list<LAT, CM, S, double, T, 1><<<div_up(lc, 64), 64, 0, st>>>(a);
     break;
   case OP_LOCAL_INIT:
     k_local<LAT, CM, S, T, T, 0><<<div_up(a.N, 256), 256, 0, st>>>(a);

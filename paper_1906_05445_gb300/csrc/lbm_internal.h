@@ -132,8 +132,7 @@ enum SweepOp {
   OP_BULK_SWEEP,   // pull + collide + store, plain fluid nodes
   OP_LIST_SWEEP,   // pull + bounce-back + collide + store + Eq. 17
   OP_ZY_SEED,      // Eq. 16: boundary nodes' pre-collision populations from a local state
-  OP_BULK_QUERY,   // pull, fields to FP64 outputs
-  OP_LIST_QUERY,
+  OP_QUERY,        // pull (plain and boundary nodes), fields to FP64 outputs
   OP_LOCAL_INIT,   // local read of a pre-collision state + collide + store
   OP_LOCAL_QUERY,  // local read of a pre-collision state, fields
   OP_REFILL,       // equilibrium refill of uncovered nodes (+ collide)
