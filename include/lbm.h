@@ -442,7 +442,8 @@ lbm_status lbm_batch_step(lbm_batch *batch, int nsteps);
 lbm_status lbm_batch_run_to_steady(lbm_batch *batch, double tol,
                                    int check_every, int max_steps,
                                    int64_t *steps_done, double *residual);
-/* block widths chosen for lattice i and the number of graph launches */
+/* block widths chosen for lattice i and the number of graph launches (and of
+ * multi-step launches of small lattices) */
 lbm_status lbm_batch_info(lbm_batch *batch, int i, int *bulk_block,
                           int *list_block, int64_t *graph_launches);
 const char *lbm_batch_last_error(const lbm_batch *batch);

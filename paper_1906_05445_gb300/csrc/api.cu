@@ -52,6 +52,20 @@ void launch_sweep(SweepOp op, int lattice, int collision, int precision, const K
   }
 }
 thread_local int g_bulk_kernel = BK_NODE;
+
+cudaError_t launch_run_f64(const RunArgs<kMaxRun> &, int, int, cudaStream_t);
+cudaError_t launch_run_f32(const RunArgs<kMaxRun> &, int, int, cudaStream_t);
+cudaError_t launch_run_bf16(const RunArgs<kMaxRun> &, int, int, cudaStream_t);
+cudaError_t launch_run_f16(const RunArgs<kMaxRun> &, int, int, cudaStream_t);
+cudaError_t launch_run(const RunArgs<kMaxRun> &g, int lattice, int collision, int precision,
+                       cudaStream_t st) {
+  switch (precision) {
+  case LBM_FP64: return launch_run_f64(g, lattice, collision, st);
+  case LBM_FP32: return launch_run_f32(g, lattice, collision, st);
+  case LBM_FP32_BF16STORE: return launch_run_bf16(g, lattice, collision, st);
+  default: return launch_run_f16(g, lattice, collision, st);
+  }
+}
 }  // namespace lbm
 
 using namespace lbm;
@@ -85,14 +99,12 @@ struct lbm_ctx {
   long long N = 0;
   long long fs = 0;  // direction stride of the distribution arrays (elements)
   int bulk_block = 128;
-  int list_block = 256;
+  int list_block = 128;  // threads per block of the boundary-node kernels (reported only)
   int cache_hints = 0;
   int bulk_mode = 1;
   int bulk_kernel = -1;  // the bulk sweep kernel of the last step (BulkKernel), -1 none yet
   int bulk_vec_words = 0;
   int bulk_vec_packed = -1;
-  int ibm_list_thread = 1;  // IBM band nodes: a thread per node in the boundary sweep
-  int ibb_list_thread = 0;  // bounce-back boundary nodes too (measured slower: off)
   int coll_mode = 0;  // CM_BGK, CM_MRT or CM_MRT_Q
   cudaStream_t st = 0;
   // auxiliary high-priority stream: the boundary-node sweep and the IBM
@@ -183,15 +195,23 @@ struct lbm_ctx {
   void *mk_wts = nullptr;
   bool markers_dirty = false;
   int nmark = 0;
+  // tables of markers at rest (ibm_device.cuh): tab.nmark 0 without them
+  IbmTab tab{};
+  std::vector<void *> tab_mem;
   int mk_start[kMaxSolids + 1] = {0};  // markers of solid k: mk_start[k] .. mk_start[k+1] - 1
   // the forcing loop in one cluster per solid (see ibm.cu), taken with
   // LBM_IBM_CLUSTER=1 where it fits the device (decided when the markers are
   // built); off by default: it measured slower than the warp-per-marker
   // kernels spread over every SM
   bool ibm_cluster = false, ibm_cluster_on = false;
+  bool ibm_tables = true;  // LBM_IBM_TABLES=0: scatter with atomics for solids at rest too
   void *u_band = nullptr, *f_ibm = nullptr;
   // forces
   double *hist = nullptr;
+  unsigned *run_bar = nullptr;  // k_run's barrier counters (zero between launches)
+  int zero_slot = -1;           // the record a k_run launch left zeroed for the step after it
+  bool run_on = true;           // LBM_RUN=0: every step as launches of its own
+  int sms = 0;
   int slot = 0;
   long long records = 0;
   // queries / residual
@@ -372,9 +392,8 @@ KArgs base_args(lbm_ctx *ctx) {
   a.bulk_mode = ctx->bulk_mode;
   a.bulk_vec_words = ctx->bulk_vec_words;
   a.bulk_vec_packed = ctx->bulk_vec_packed;
-  a.list_thread = (ctx->scheme.scheme == LBM_IBM_DIRECT && ctx->ibm_list_thread) ||
-                          ctx->ibb_list_thread ? 1 : 0;
-  a.list_block = ctx->list_block;
+  a.ibm = ctx->scheme.scheme == LBM_IBM_DIRECT ? 1 : 0;
+  a.tab = ctx->tab;
   a.zy_pre = ctx->scheme.scheme == LBM_ZHAO_YONG ? ctx->zy_pre : nullptr;
   for (int k = 0; k < 6; k++) {
     a.face[k] = ctx->dom.type[k];
@@ -905,6 +924,83 @@ lbm_status build_markers(lbm_ctx *ctx) {
 
 void ibm_prepare(lbm_ctx *ctx);
 void ibm_prepare(lbm_ctx *ctx, cudaStream_t s);
+IbmArgs ibm_args(lbm_ctx *ctx, double *acc);
+
+void free_tables(lbm_ctx *ctx) {
+  for (void *p : ctx->tab_mem) dfree(ctx, p);
+  ctx->tab_mem.clear();
+  ctx->tab = IbmTab{};
+}
+
+lbm_status tab_alloc(lbm_ctx *ctx, void **p, size_t bytes) {
+  TRY(dalloc(ctx, p, std::max<size_t>(bytes, 8)));
+  ctx->tab_mem.push_back(*p);
+  return LBM_OK;
+}
+
+bool run_small(const lbm_ctx *ctx);
+
+// The row and coupling tables of IBM solids at rest, after the geometry and
+// the stencils are built: for lattices whose steps k_run takes, and for the
+// others where forcing passes repeat (48^3, five passes, by launches: 48 us
+// per step against 75).  One pass on a large lattice keeps the scattering
+// kernel: two 128^3 lattices 98.9 us per step against 101.4 with the band
+// nodes gathering beside the sweep.  Axes of at least 8 nodes: two stencils then meet at
+// one periodic shift only, and a node lies in a stencil once.
+lbm_status build_tables(lbm_ctx *ctx) {
+  const bool small = ctx->d.nx < 8 || ctx->d.ny < 8 || (ctx->D == 3 && ctx->d.nz < 8);
+  if (ctx->scheme.scheme != LBM_IBM_DIRECT || ctx->nmark == 0 || any_moving(ctx) || small ||
+      ctx->list_count <= 0 || ctx->ibm_cluster_on || !ctx->ibm_tables ||
+      (ctx->scheme.ibm_iters <= 1 && !run_small(ctx)))
+    return LBM_OK;
+  const int nm = ctx->nmark, nl = ctx->list_count;
+  const bool iterate = ctx->scheme.ibm_iters > 1;
+  IbmTab tb{};
+  tb.base = ctx->mk_base;
+  tb.wts = ctx->mk_wts;
+  tb.dV = ctx->mk_dV;
+  tb.msid = ctx->mk_sid;
+  tb.Fm = ctx->mk_F;
+  IbmArgs ib = ibm_args(ctx, nullptr);
+  int *nrow = nullptr, *ncol = nullptr, *mrow = nullptr, *mcol = nullptr;
+  void *nw = nullptr, *mw = nullptr;
+  double *Ud = nullptr, *arm = nullptr;
+  TRY(tab_alloc(ctx, (void **)&nrow, sizeof(int) * ((size_t)nl + 1)));
+  TRY(tab_alloc(ctx, (void **)&mrow, sizeof(int) * ((size_t)nm + 1)));
+  TRY(tab_alloc(ctx, (void **)&Ud, sizeof(double) * 3 * nm));
+  TRY(tab_alloc(ctx, (void **)&arm, sizeof(double) * 3 * nm));
+  TRY(tab_alloc(ctx, (void **)&tb.dF, sizeof(double) * 3 * nm));
+  TRY(tab_alloc(ctx, &tb.dFT, ctx->tsz * 6 * nm));
+  TRY(tab_alloc(ctx, &tb.FdV, ctx->tsz * 3 * nm));
+  launch_tab_desired(ib, Ud, arm, ctx->st);
+  launch_tab_nodes(ib, ctx->list_node, nl, nrow, nullptr, nullptr, ctx->d.precision, ctx->st);
+  if (iterate) launch_tab_markers(ib, mrow, nullptr, nullptr, ctx->d.precision, ctx->st);
+  int ne = 0, me = 0;
+  CK(cudaMemcpyAsync(&ne, nrow + nl, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+  if (iterate) CK(cudaMemcpyAsync(&me, mrow + nm, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+  CK(cudaStreamSynchronize(ctx->st));
+  TRY(tab_alloc(ctx, (void **)&ncol, sizeof(int) * (size_t)ne));
+  TRY(tab_alloc(ctx, &nw, ctx->tsz * (size_t)ne));
+  launch_tab_nodes(ib, ctx->list_node, nl, nrow, ncol, nw, ctx->d.precision, ctx->st);
+  if (iterate) {
+    TRY(tab_alloc(ctx, (void **)&mcol, sizeof(int) * (size_t)me));
+    TRY(tab_alloc(ctx, &mw, ctx->tsz * (size_t)me));
+    launch_tab_markers(ib, mrow, mcol, mw, ctx->d.precision, ctx->st);
+  }
+  ctx->launches += iterate ? 7 : 4;
+  CK(cudaGetLastError());
+  tb.Ud = Ud;
+  tb.arm = arm;
+  tb.nrow = nrow;
+  tb.ncol = ncol;
+  tb.nw = nw;
+  tb.mrow = mrow;
+  tb.mcol = mcol;
+  tb.mw = mw;
+  tb.nmark = nm;
+  ctx->tab = tb;
+  return LBM_OK;
+}
 
 lbm_status read_counts(lbm_ctx *ctx, int out[16]) {
   CK(cudaMemcpyAsync(out, ctx->counts, 16 * sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
@@ -916,6 +1012,7 @@ lbm_status read_counts(lbm_ctx *ctx, int out[16]) {
 // boundary nodes and links first, size the lists exactly, then build.
 lbm_status rebuild_full(lbm_ctx *ctx) {
   if (ctx) ctx->gen++;
+  free_tables(ctx);
   free_spare(ctx);  // capacities may change; the next moving step prefetches again
   TRY(motion_pull(ctx));
   if (!ctx->restore_geometry)
@@ -958,6 +1055,7 @@ lbm_status rebuild_full(lbm_ctx *ctx) {
   ctx->list_count = moving ? -1 : cnt[0];
   ctx->link_count = moving ? -1 : cnt[1];
   ibm_prepare(ctx);
+  TRY(build_tables(ctx));
   {
     IbmClusterArgs cl;
     ctx->ibm_cluster = ctx->ibm_cluster_on && ibm_cluster_args(ctx, cl) &&
@@ -1100,7 +1198,9 @@ bool ibm_zeroes_record(const lbm_ctx *ctx) {
 }
 
 // IBM: unforced velocity at the band, n_it interpolation/force iterations,
-// spreading, and the solid's force (into the given record slot).
+// spreading, and the solid's force (into the given record slot).  With tables
+// the boundary nodes gather the force when they collide; `dense` has it
+// written to the dense field as well (a state that is not swept next).
 // whether [o1, o1 + w1) and [o2, o2 + w2) are disjoint on a periodic axis of n
 bool disjoint_mod(int o1, int w1, int o2, int w2, int n) {
   if (w1 + w2 > n) return false;
@@ -1160,7 +1260,8 @@ bool ibm_cluster_args(const lbm_ctx *ctx, IbmClusterArgs &cl) {
   return true;
 }
 
-void ibm_prepass(lbm_ctx *ctx, const void *src, bool local, double *acc, cudaStream_t s) {
+void ibm_prepass(lbm_ctx *ctx, const void *src, bool local, bool dense, double *acc,
+                 cudaStream_t s) {
   if (ctx->scheme.scheme != LBM_IBM_DIRECT || ctx->nmark == 0) return;
   Timed tm(ctx, TK_IBM, 0, s);
   if (ctx->markers_dirty) ibm_prepare(ctx, s);  // moving solids: every step
@@ -1169,8 +1270,17 @@ void ibm_prepass(lbm_ctx *ctx, const void *src, bool local, double *acc, cudaStr
   a.local_gather = local ? 1 : 0;
   a.force_acc = acc;  // cleared by the band-velocity kernel
   sweep(ctx, OP_BAND_VEL, a, s);
-  IbmArgs ib = ibm_args(ctx, acc);
   const int iters = std::max(1, ctx->scheme.ibm_iters);
+  if (ctx->tab.nmark > 0) {
+    // solids at rest: the forcing passes on the markers' tables; the sweep's
+    // boundary nodes gather the force themselves
+    for (int it = 0; it < iters; it++)
+      launch_marker_pass(a, ctx->D, it, it == iters - 1, ctx->d.precision, s);
+    ctx->launches += iters;
+    if (dense) sweep(ctx, OP_IBM_GATHER, a, s);
+    return;
+  }
+  IbmArgs ib = ibm_args(ctx, acc);
   IbmClusterArgs cl;
   if (ctx->ibm_cluster && ibm_cluster_args(ctx, cl)) {
     launch_ibm_cluster(ib, cl, ctx->d.precision, s);
@@ -1207,10 +1317,11 @@ lbm_status init_collide(lbm_ctx *ctx) {
   if (ctx) ctx->gen++;
   TRY(ensure_geometry(ctx));
   const int prev = 1 - ctx->cur;
+  ctx->zero_slot = -1;
   ctx->slot = (ctx->slot + 1) % kHistCap;
   double *acc = force_slot(ctx, ctx->slot);
   CK(cudaMemsetAsync(acc, 0, sizeof(double) * kMaxSolids * 6, ctx->st));
-  ibm_prepass(ctx, ctx->f[prev], true, acc, ctx->st);
+  ibm_prepass(ctx, ctx->f[prev], true, true, acc, ctx->st);
   KArgs a = base_args(ctx);
   a.src = ctx->f[prev];
   a.dst = ctx->f[ctx->cur];
@@ -1276,6 +1387,7 @@ lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
     sweep(ctx, OP_REFILL, a);
   }
   ctx->slot = (ctx->slot + 1) % kHistCap;
+  ctx->zero_slot = -1;
   double *acc = force_slot(ctx, ctx->slot);
   a = base_args(ctx);
   a.src = ctx->f[cur];
@@ -1290,7 +1402,7 @@ lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
   // the IBM band-velocity kernel clears the record itself (one launch fewer
   // on the IBM lattice's critical chain); otherwise a memset does
   if (!ibm_zeroes_record(ctx)) CK(cudaMemsetAsync(acc, 0, sizeof(double) * kMaxSolids * 6, ctx->aux));
-  ibm_prepass(ctx, ctx->f[cur], false, acc, ctx->aux);
+  ibm_prepass(ctx, ctx->f[cur], false, false, acc, ctx->aux);
   {
     Timed tm(ctx, TK_LIST, ctx->list_count >= 0 ? ctx->list_count : 0, ctx->aux);
     sweep(ctx, OP_LIST_SWEEP, a, ctx->aux);
@@ -1339,11 +1451,126 @@ lbm_status step_end(lbm_ctx *ctx, const StepState &ss) {
   return LBM_OK;
 }
 
+// ---- several steps in one launch (run_impl.cuh)
+
+bool run_small(const lbm_ctx *ctx);
+
+// Whether a lattice's steps can run in k_run: solids at rest (IBM: with
+// tables), a periodic box, the default kernels, untimed, and small enough
+// that launches and phase latencies, not bandwidth, set its step.
+bool run_ok(const lbm_ctx *ctx) {
+  const bool ibm = ctx->scheme.scheme == LBM_IBM_DIRECT && ctx->nmark > 0;
+  return ctx->run_on && ctx->sms > 0 && run_small(ctx) && !any_moving(ctx) && !ctx->nface &&
+         ctx->timing == 0 && ctx->coll_mode != CM_MRT && ctx->bulk_mode == 1 &&
+         (ctx->bulk_vec_words == 0 || ctx->bulk_vec_words == 2) && ctx->bulk_vec_packed != 0 &&
+         ctx->cache_hints == 0 && (!ibm || ctx->tab.nmark > 0);
+}
+
+// nodes per vector of the 2-word kernels, 0 where the one-node update runs
+bool run_vec(const lbm_ctx *ctx) {
+  if (ctx->d.precision == LBM_FP64) return false;
+  const int V = ctx->d.precision == LBM_FP32 ? 2 : 4;
+  return ctx->d.nx % V == 0 && ctx->fs % V == 0;
+}
+
+// Largest lattice (populations, nodes x Q) whose steps k_run takes, from us
+// per step of k_run against the step's own launches (3D spheres of R = 3/32
+// of the edge, 2D Couette flows):
+//   FP32 bounce-back  64^3 8.2 / 14.2, 80^3 12.4 / 14.3, 88^3 18.7 / 16.1;
+//                     301^2 5.2 / 11.3, 512^2 6.3 / 11.9
+//   FP32 IBM, 1 pass  64^3 14.8 / 24.1, 72^3 20.7 / 24.0, 80^3 23.8 / 24.2
+//   FP32 IBM, 5       80^3 33.4 / 49.6, 96^3 47.6 / 57.4
+//   FP16 bounce-back  80^3 11.0 / 14.4, 88^3 14.2 / 14.2; IBM 72^3 22.1 / 22.7
+//   FP64 bounce-back  48^3 41.9 / 51.9, 56^3 60.8 / 59.7; 512^2 34.4 / 41.1
+//   FP64 IBM, 1       32^3 27.7 / 30.9, 41^3 38.2 / 37.2; 5: 48^3 67 / 79, 64^3 110 / 111
+// Beyond, the one block per SM keeps too few loads in flight for the sweep.
+bool run_small(const lbm_ctx *ctx) {
+  const bool f64 = ctx->d.precision == LBM_FP64;
+  const long long v = ctx->N * ctx->Q;
+  if (ctx->scheme.scheme != LBM_IBM_DIRECT || ctx->nmark == 0) return v <= (f64 ? 2400000 : 10000000);
+  if (ctx->scheme.ibm_iters <= 1) return v <= (f64 ? 700000 : 7200000);
+  return v <= (f64 ? 2400000 : 17000000);
+}
+
+// nsteps steps of the lattices in `ctxs` (run_ok, same lattice, collision and
+// precision, all or none with IBM tables, at most kMaxRun) in one launch on `st`, which follows their own
+// streams' earlier work and precedes their later work (the caller's order).
+lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
+  lbm_ctx *ctx = ctxs[0];
+  if (nsteps < 1) return LBM_OK;
+  RunArgs<kMaxRun> g;
+  memset(&g, 0, sizeof(g));
+  g.n = n;
+  // blocks in proportion to the nodes, at least four each, one per SM in all
+  double w[kMaxRun], sum = 0;
+  for (int k = 0; k < n; k++) {
+    const lbm_ctx *c = ctxs[k];
+    w[k] = (double)c->N * c->Q;
+    sum += w[k];
+  }
+  int at = 0;
+  for (int k = 0; k < n; k++) {
+    lbm_ctx *c = ctxs[k];
+    const bool vec = run_vec(c);
+    const int V = !vec ? 1 : c->d.precision == LBM_FP32 ? 2 : 4;
+    // no more blocks than warps of nodes and groups of boundary nodes
+    const long long warps = (c->N / V + 31) / 32 + std::max(0, c->list_count) / 16;
+    const long long share =
+        n == 1 ? c->sms : std::max<long long>(4, (long long)(w[k] / sum * (c->sms - 4 * n)) + 4);
+    const int nb = (int)std::max<long long>(1, std::min(share, warps));
+    g.block_start[k] = at;
+    at += nb;
+    RunLat &r = g.l[k];
+    r.a = base_args(c);
+    r.f[0] = c->f[0];
+    r.f[1] = c->f[1];
+    r.cur = c->cur;
+    r.nsteps = nsteps;
+    r.slot0 = c->slot;
+    r.hist_cap = kHistCap;
+    r.hist = c->hist;
+    r.bar = c->run_bar;
+    r.iters = std::max(1, c->scheme.ibm_iters);
+    r.vec = vec ? 1 : 0;
+    const int first = (c->slot + 1) % kHistCap;
+    // the record the launch starts with: left zeroed by the launch before
+    // (never relied on in a capture, whose replays find their own sums there)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &cap));
+    if (c->zero_slot != first || cap != cudaStreamCaptureStatusNone)
+      CK(cudaMemsetAsync(force_slot(c, first), 0, sizeof(double) * kMaxSolids * 6, st));
+  }
+  g.block_start[n] = at;
+  for (int k = n; k < kMaxRun; k++) g.block_start[k + 1] = at;
+  CK(launch_run(g, ctx->d.lattice, ctx->coll_mode, ctx->d.precision, st));
+  for (int k = 0; k < n; k++) {
+    lbm_ctx *c = ctxs[k];
+    c->slot = (c->slot + nsteps) % kHistCap;
+    c->zero_slot = (c->slot + 1) % kHistCap;
+    c->cur = (c->cur + nsteps) & 1;
+    c->prev_local = false;
+    c->records = std::min<long long>(c->records + nsteps, kHistCap);
+    c->step += nsteps;
+    c->launches++;
+    c->bulk_kernel = run_vec(c) ? BK_VEC : BK_NODE;
+  }
+  return LBM_OK;
+}
+
 lbm_status step_once(lbm_ctx *ctx) {
   StepState ss;
   TRY(step_begin(ctx, ss));
   step_bulk(ctx, ss);
   return step_end(ctx, ss);
+}
+
+// A call of one step keeps its own launches: k_run's set-up (the threads' step
+// constants) is then not shared by any other step, and two lattices stepped in
+// turn on their own streams could not overlap (64^3 pair: 34 us against 30).
+lbm_status step_many(lbm_ctx *ctx, int nsteps) {
+  if (nsteps >= 2 && run_ok(ctx)) return run_steps(&ctx, 1, nsteps, ctx->st);
+  for (int k = 0; k < nsteps; k++) TRY(step_once(ctx));
+  return LBM_OK;
 }
 
 // The bulk sweeps of the lattices in `idx` (same lattice, collision and
@@ -1592,6 +1819,8 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
       return LBM_ERR_CUDA;
     }
   }
+  if (cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess)
+    ctx->sms = 0;
   ctx->ssz = d.precision == LBM_FP64 ? 8 : d.precision == LBM_FP32 ? 4 : 2;
   ctx->tsz = d.precision == LBM_FP64 ? 8 : 4;
   set_collision_constants(ctx);
@@ -1610,17 +1839,13 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
       if (b >= 32 && b <= 512 && b % 32 == 0) ctx->bulk_block = b;
     }
     if (const char *e = getenv("LBM_CACHE_HINTS")) ctx->cache_hints = atoi(e) & 3;
-    if (const char *e = getenv("LBM_LIST_BLOCK")) {
-      const int v = atoi(e);
-      if (v == 32 || v == 64 || v == 128 || v == 256) ctx->list_block = v;
-    }
     if (const char *e = getenv("LBM_BULK_MODE")) ctx->bulk_mode = atoi(e);
     if (const char *e = getenv("LBM_VEC_WORDS")) ctx->bulk_vec_words = atoi(e);
     if (const char *e = getenv("LBM_GEOM_PREFETCH")) ctx->geom_prefetch = atoi(e) != 0;
     if (const char *e = getenv("LBM_VEC_PACKED")) ctx->bulk_vec_packed = atoi(e);
-    if (const char *e = getenv("LBM_IBM_LIST_THREAD")) ctx->ibm_list_thread = atoi(e) != 0;
+    if (const char *e = getenv("LBM_RUN")) ctx->run_on = atoi(e) != 0;
+    if (const char *e = getenv("LBM_IBM_TABLES")) ctx->ibm_tables = atoi(e) != 0;
     if (const char *e = getenv("LBM_IBM_CLUSTER")) ctx->ibm_cluster_on = atoi(e) != 0;
-    if (const char *e = getenv("LBM_IBB_LIST_THREAD")) ctx->ibb_list_thread = atoi(e) != 0;
     if (const char *e = getenv("LBM_MRT_GENERAL"))
       if (atoi(e) && ctx->coll_mode == CM_MRT_Q) ctx->coll_mode = CM_MRT;
   }
@@ -1633,6 +1858,7 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
       (s = dalloc(ctx, (void **)&ctx->sid, 2 * padN)) != LBM_OK ||
       (s = dalloc(ctx, (void **)&ctx->counts, 16 * sizeof(int))) != LBM_OK ||
       (s = dalloc(ctx, (void **)&ctx->hist, sizeof(double) * kHistCap * kMaxSolids * 6)) != LBM_OK ||
+      (s = dalloc(ctx, (void **)&ctx->run_bar, 2 * sizeof(unsigned))) != LBM_OK ||
       (s = dalloc(ctx, (void **)&ctx->red2, 2 * sizeof(double))) != LBM_OK) {
     lbm_destroy(ctx);
     return s;
@@ -1640,6 +1866,7 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
   cudaMemsetAsync(ctx->flags, 0, padN, ctx->st);
   cudaMemsetAsync(ctx->sid, 0, 2 * padN, ctx->st);
   cudaMemsetAsync(ctx->counts, 0, 16 * sizeof(int), ctx->st);
+  cudaMemsetAsync(ctx->run_bar, 0, 2 * sizeof(unsigned), ctx->st);
   cudaMemsetAsync(ctx->hist, 0, sizeof(double) * kHistCap * kMaxSolids * 6, ctx->st);
   // rest state f = w as a pre-collision state, collided on first use
   KArgs a = base_args(ctx);
@@ -1862,7 +2089,7 @@ lbm_status lbm_get_distributions(lbm_ctx *ctx, double *host_f, size_t n) {
 lbm_status lbm_step(lbm_ctx *ctx, int nsteps) {
   if (!ctx || nsteps < 0) return LBM_ERR_ARG;
   TRY(prepare(ctx));
-  for (int k = 0; k < nsteps; k++) TRY(step_once(ctx));
+  TRY(step_many(ctx, nsteps));
   CK(cudaGetLastError());
   return LBM_OK;
 }
@@ -1919,7 +2146,7 @@ lbm_status lbm_run_to_steady(lbm_ctx *ctx, double tol, int check_every, int max_
   lbm_status st = LBM_OK;
   while (done < max_steps) {
     const int k = std::min(check_every, max_steps - done);
-    for (int j = 0; j < k; j++) TRY(step_once(ctx));
+    TRY(step_many(ctx, k));
     done += k;
     TRY(velocity_to(ctx, ctx->u_now));
     launch_residual(ctx->u_now, ctx->u_snap, 0, ctx->flags, ctx->N, ctx->D, ctx->red2, ctx->st);
@@ -2095,6 +2322,11 @@ lbm_status lbm_set_solid_dynamics(lbm_ctx *ctx, int id, double density_ratio,
       ctx->scheme.ibm_inertia == LBM_INERTIA_UHLMANN)
     return fail(ctx, LBM_ERR_ARG, "Eq. 22 needs a solid denser than the fluid");
   TRY(solids_to_host(ctx, true));
+  if (density_ratio > 0 && ctx->tab.nmark > 0) {
+    // the markers will move: their tables go
+    CK(cudaStreamSynchronize(ctx->st));
+    free_tables(ctx);
+  }
   SolidHost &h = ctx->solids[id];
   h.rho_p = density_ratio > 0 ? density_ratio : 0;
   h.have_Ip = false;
@@ -2258,10 +2490,11 @@ lbm_status lbm_load(lbm_ctx *ctx, const void *host_buf, size_t size) {
   TRY(rebuild_full(ctx));
   if (!ctx->need_collide && ctx->scheme.scheme == LBM_IBM_DIRECT) {
     // the IBM force of the current time is recomputed from the restored state
+    ctx->zero_slot = -1;
     ctx->slot = (ctx->slot + 1) % kHistCap;
     double *acc = force_slot(ctx, ctx->slot);
     CK(cudaMemsetAsync(acc, 0, sizeof(double) * kMaxSolids * 6, ctx->st));
-    ibm_prepass(ctx, ctx->f[1], ctx->prev_local, acc, ctx->st);
+    ibm_prepass(ctx, ctx->f[1], ctx->prev_local, true, acc, ctx->st);
   }
   CK(cudaStreamSynchronize(ctx->st));
   return LBM_OK;
@@ -2345,7 +2578,8 @@ lbm_status lbm_sync(lbm_ctx *ctx) {
                 "stress-free face, R + 5 from an outflow face)");
   if (cnt[5])
     return fail(ctx, LBM_ERR_TIMEOUT,
-                "a bulk sweep gave up waiting (one second) for its asynchronous row copies");
+                "a kernel gave up waiting (one second): a bulk sweep for its asynchronous row "
+                "copies, or a multi-step kernel for its other blocks");
   return LBM_OK;
 }
 
@@ -2403,7 +2637,6 @@ lbm_status bfail(lbm_batch *b, lbm_status s, const std::string &m) {
 // fastest (writes go to a scratch buffer: the simulation state is untouched).
 lbm_status autotune(lbm_ctx *ctx, void *scratch) {
   const int cand_bulk[3] = {64, 128, 256};
-  const int cand_list[3] = {64, 128, 256};
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -2428,24 +2661,6 @@ lbm_status autotune(lbm_ctx *ctx, void *scratch) {
     }
   }
   ctx->bulk_block = best_b;
-  best = 1e30f;
-  int best_l = ctx->list_block;
-  if (a.list_cap > 0)
-    for (int c : cand_list) {
-      a.list_block = c;
-      sweep(ctx, OP_LIST_SWEEP, a);
-      cudaEventRecord(e0, ctx->st);
-      for (int r = 0; r < 3; r++) sweep(ctx, OP_LIST_SWEEP, a);
-      cudaEventRecord(e1, ctx->st);
-      cudaEventSynchronize(e1);
-      float ms = 0;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (ms < best) {
-        best = ms;
-        best_l = c;
-      }
-    }
-  ctx->list_block = best_l;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   // forget the scratch force record written while tuning
@@ -2462,7 +2677,45 @@ void drop_graph(lbm_batch *b) {
 // solids, or solids that move on the device (a free solid present).  Solids
 // with a prescribed motion move on the host, which prefetches their next
 // geometry: those lattices step directly.
-bool graphable(const lbm_ctx *c) { return !any_moving(c) || dev_motion(c); }
+// Small lattices run their steps in k_run, outside the graph.
+bool graphable(const lbm_ctx *c) { return (!any_moving(c) || dev_motion(c)) && !run_ok(c); }
+
+// All nsteps of the active lattices that k_run takes, up to kMaxRun of one
+// kind per launch (eight lattices of edges 24..64, alternately bounce-back and
+// IBM: 12 + 26 us per step in two launches, 52 in one whose threads hold both
+// kinds' constants, 45 as graph replays).
+lbm_status batch_run(lbm_batch *b, int nsteps) {
+  const int n = (int)b->ctx.size();
+  std::vector<char> done(n, 0);
+  for (int i = 0; i < n; i++) {
+    if (!b->active[i] || done[i] || !run_ok(b->ctx[i])) continue;
+    lbm_ctx *grp[kMaxRun];
+    int idx[kMaxRun], m = 0;
+    for (int j = i; j < n && m < kMaxRun; j++) {
+      const lbm_ctx *c = b->ctx[j], *c0 = b->ctx[i];
+      if (!b->active[j] || done[j] || !run_ok(c) || c->d.lattice != c0->d.lattice ||
+          c->coll_mode != c0->coll_mode || c->d.precision != c0->d.precision ||
+          (c->tab.nmark > 0) != (c0->tab.nmark > 0))
+        continue;
+      grp[m] = b->ctx[j];
+      idx[m++] = j;
+      done[j] = 1;
+    }
+    for (int k = 0; k < m; k++) {
+      BCK(cudaEventRecord(b->ev_done[idx[k]], grp[k]->st));
+      BCK(cudaStreamWaitEvent(b->origin, b->ev_done[idx[k]], 0));
+    }
+    const lbm_status s = run_steps(grp, m, nsteps, b->origin);
+    if (s != LBM_OK) return bfail(b, s, lbm_last_error(grp[0]));
+    BCK(cudaEventRecord(b->ev_origin, b->origin));
+    for (int k = 0; k < m; k++) {
+      BCK(cudaStreamWaitEvent(grp[k]->st, b->ev_origin, 0));
+      b->steps_done[idx[k]] += nsteps;
+    }
+    b->graph_launches++;
+  }
+  return LBM_OK;
+}
 
 // Capture two steps of every active lattice with static geometry or solids
 // moving on the device.
@@ -2607,7 +2860,16 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
       lbm_status s = prepare(b->ctx[i]);
       if (s != LBM_OK) return bfail(b, s, lbm_last_error(b->ctx[i]));
     }
-  int done = 0;
+  // small lattices first, all their steps at once
+  std::vector<char> ran(n, 0);
+  if (nsteps >= 2) {
+    for (int i = 0; i < n; i++) ran[i] = b->active[i] && run_ok(b->ctx[i]);
+    const lbm_status s = batch_run(b, nsteps);
+    if (s != LBM_OK) return s;
+  }
+  bool rest = false;
+  for (int i = 0; i < n; i++) rest |= b->active[i] && !ran[i];
+  int done = rest ? 0 : nsteps;
   while (done < nsteps) {
     const bool pair = nsteps - done >= 2;
     bool any_static = false;
@@ -2636,7 +2898,7 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
       }
       // lattices outside the graph (solids with a prescribed motion) step directly
       for (int i = 0; i < n; i++) {
-        if (!b->active[i] || b->in_graph[i]) continue;
+        if (!b->active[i] || b->in_graph[i] || ran[i]) continue;
         for (int k = 0; k < 2; k++) {
           lbm_status s = step_once(b->ctx[i]);
           if (s != LBM_OK) return bfail(b, s, lbm_last_error(b->ctx[i]));
@@ -2646,7 +2908,7 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
       done += 2;
     } else {
       for (int i = 0; i < n; i++) {
-        if (!b->active[i]) continue;
+        if (!b->active[i] || ran[i]) continue;
         lbm_status s = step_once(b->ctx[i]);
         if (s != LBM_OK) return bfail(b, s, lbm_last_error(b->ctx[i]));
         b->steps_done[i] += 1;
@@ -2721,7 +2983,6 @@ lbm_status lbm_batch_create(lbm_batch **out, lbm_ctx *const *ctxs, int n, void *
             same = j;
         if (same >= 0) {
           b->ctx[i]->bulk_block = b->ctx[same]->bulk_block;
-          b->ctx[i]->list_block = b->ctx[same]->list_block;
         } else if (autotune(b->ctx[i], scratch) != LBM_OK) {
           e = cudaErrorUnknown;
           break;

@@ -15,41 +15,38 @@ namespace lbm {
 // deviations (coefficients of Sec. 2.2, precomputed per link):
 //   f_i(x_f,t+1) = c0 f*_ib(x_f) + c1 f*_ib(x_ff) + c2 f*_ib(x_fff)
 //                + c3 f*_i(x_f) + c4 f*_i(x_ff) + mw.
-template <int LAT, typename S, typename T, typename LT>
-__device__ __forceinline__ T ibb_value(const KArgs &a, const S *__restrict__ src,
-                                       int i, int x, int y, int z, long long n,
-                                       int link, T isc, T &fs) {
-  using L = Lat<LAT>;
-  const int ib = L::opp(i);
+template <int LAT, typename S, typename T, typename LT, int POL = LD_NC>
+__device__ __forceinline__ T ibb_value(const KArgs &a, const S *src, int i, int ib, int ex, int ey,
+                                       int ez, int x, int y, int z, long long n, int link, T isc,
+                                       T &fs) {
   const LT *c0 = (const LT *)a.links.c[0], *c1 = (const LT *)a.links.c[1],
            *c2 = (const LT *)a.links.c[2], *c3 = (const LT *)a.links.c[3],
            *c4 = (const LT *)a.links.c[4], *mw = (const LT *)a.links.mw;
   const long long N = a.fs;
-  const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
-  fs = Store<S>::ld(src + (long long)ib * N + n, isc);
+  fs = Store<S>::template ld<POL>(src + (long long)ib * N + n, isc);
   if (a.zy_pre) {
     // Eq. 16: the post-collision value leaving the wall at x_f (c3), the
     // pre-collision value arriving at x_f from the previous step (c1) and
     // the moving-wall term
     const LT *pre = (const LT *)a.zy_pre;
-    return (T)c3[link] * Store<S>::ld(src + (long long)i * N + n, isc) +
-           (T)c1[link] * (T)pre[(long long)ib * N + n] + (T)mw[link];
+    return vfma((T)c3[link], Store<S>::template ld<POL>(src + (long long)i * N + n, isc),
+                vfma((T)c1[link], (T)pre[(long long)ib * N + n], (T)mw[link]));
   }
-  T v = (T)c0[link] * fs + (T)mw[link];
+  T v = vfma((T)c0[link], fs, (T)mw[link]);
   const T k1 = (T)c1[link], k2 = (T)c2[link], k3 = (T)c3[link], k4 = (T)c4[link];
   if (k1 != (T)0 || k2 != (T)0 || k4 != (T)0) {
     const long long nff = wrap(x + ex, a.nx) +
                           (long long)a.nx * (wrap(y + ey, a.ny) + (long long)a.ny * wrap(z + ez, a.nz));
-    if (k1 != (T)0) v += k1 * Store<S>::ld(src + (long long)ib * N + nff, isc);
-    if (k4 != (T)0) v += k4 * Store<S>::ld(src + (long long)i * N + nff, isc);
+    if (k1 != (T)0) v = vfma(k1, Store<S>::template ld<POL>(src + (long long)ib * N + nff, isc), v);
+    if (k4 != (T)0) v = vfma(k4, Store<S>::template ld<POL>(src + (long long)i * N + nff, isc), v);
     if (k2 != (T)0) {
       const long long nfff = wrap(x + 2 * ex, a.nx) +
                              (long long)a.nx * (wrap(y + 2 * ey, a.ny) +
                                                 (long long)a.ny * wrap(z + 2 * ez, a.nz));
-      v += k2 * Store<S>::ld(src + (long long)ib * N + nfff, isc);
+      v = vfma(k2, Store<S>::template ld<POL>(src + (long long)ib * N + nfff, isc), v);
     }
   }
-  if (k3 != (T)0) v += k3 * Store<S>::ld(src + (long long)i * N + n, isc);
+  if (k3 != (T)0) v = vfma(k3, Store<S>::template ld<POL>(src + (long long)i * N + n, isc), v);
   return v;
 }
 
@@ -208,7 +205,9 @@ __device__ __forceinline__ void list_query_node(const KArgs &a, int t) {
       for (int i = 1; i < Q; i++) {
         if (!((mask >> i) & 1u)) continue;
         double fs;
-        f[i] = ibb_value<LAT, S, double, LT>(a, src, i, x, y, z, n, link, isc, fs);
+        f[i] = ibb_value<LAT, S, double, LT>(a, src, i, Lat<LAT>::opp(i), Lat<LAT>::ex(i),
+                                                 Lat<LAT>::ey(i), Lat<LAT>::ez(i), x, y, z, n, link,
+                                                 isc, fs);
         link++;
       }
     }
@@ -254,111 +253,6 @@ __global__ void __launch_bounds__(128) k_query(const KArgs a, int list_blocks) {
   }
 }
 
-// Boundary-node sweep: one thread per list node.
-template <int LAT, int CM, typename S, typename T>
-__global__ void __launch_bounds__(128) k_list(const KArgs a) {
-  using L = Lat<LAT>;
-  constexpr int Q = L::Q;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  int cnt = a.counts[0];
-  if (cnt > a.list_cap) cnt = a.list_cap;
-  // IBM band nodes next to a domain face run in the face kernel
-  const bool active = t < cnt && !(a.flags[a.list_node[t]] & FL_FACE);
-  const T isc = kisc<T>(a);
-  const S *__restrict__ src = (const S *)a.src;
-  // momentum exchange (Eq. 17) of this thread for solid `sa` (the solid of
-  // its first cut link): the state-independent part -2 w_i e_i of every
-  // link was summed per node in FP64 when the geometry was built; the part
-  // linear in the deviations is formed here in the compute type and the
-  // sums are reduced in FP64
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  T dacc[6] = {0, 0, 0, 0, 0, 0};
-  int sa = -1;
-  if (active) {
-    const long long n = a.list_node[t];
-    const uint32_t mask = a.list_mask[t];
-    int link = a.list_link[t];
-    int x, y, z;
-    node_xyz(n, a.nx, a.ny, x, y, z);
-    T f[Q];
-    gather_pull<LAT, S, T>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
-    if (mask) {
-#pragma unroll
-      for (int i = 1; i < Q; i++) {
-        if (!((mask >> i) & 1u)) continue;
-        T fs;
-        const T v = ibb_value<LAT, S, T, T>(a, src, i, x, y, z, n, link, isc, fs);
-        f[i] = v;
-        {
-          const int s = a.links.sid[link];
-          if (sa < 0) sa = s;
-          const T e[3] = {(T)L::ex(i), (T)L::ey(i), (T)L::ez(i)};
-          const T *uw0 = (const T *)a.links.uw[0], *uw1 = (const T *)a.links.uw[1],
-                   *uw2 = (const T *)a.links.uw[2];
-          const T *ar0 = (const T *)a.links.arm[0], *ar1 = (const T *)a.links.arm[1],
-                   *ar2 = (const T *)a.links.arm[2];
-          const T uw[3] = {(T)uw0[link], (T)uw1[link], (T)uw2[link]};
-          const T r[3] = {(T)ar0[link], (T)ar1[link], (T)ar2[link]};
-          if (s == sa) {
-            // f*_ib(e_ib - u_w) - f_i(e_i - u_w) = -2 w_i e_i
-            //   - d*_ib (e_i + u_w) - d_i (e_i - u_w)   (d: deviations)
-            T dp[3];
-            for (int c = 0; c < 3; c++) dp[c] = -fs * (e[c] + uw[c]) - v * (e[c] - uw[c]);
-            dacc[0] += dp[0];
-            dacc[1] += dp[1];
-            dacc[2] += dp[2];
-            dacc[3] += r[1] * dp[2] - r[2] * dp[1];
-            dacc[4] += r[2] * dp[0] - r[0] * dp[2];
-            dacc[5] += r[0] * dp[1] - r[1] * dp[0];
-          } else {
-            // a second solid seen from the same node (narrow gap): full FP64
-            const double wi = L::w(i);
-            const double fsd = wi + (double)fs, fid = wi + (double)v;
-            double dp[3];
-            for (int c = 0; c < 3; c++)
-              dp[c] = fsd * (-(double)e[c] - (double)uw[c]) - fid * ((double)e[c] - (double)uw[c]);
-            const double rr[3] = {(double)r[0], (double)r[1], (double)r[2]};
-            atomicAdd(a.force_acc + 6 * s + 0, dp[0]);
-            atomicAdd(a.force_acc + 6 * s + 1, dp[1]);
-            atomicAdd(a.force_acc + 6 * s + 2, dp[2]);
-            atomicAdd(a.force_acc + 6 * s + 3, rr[1] * dp[2] - rr[2] * dp[1]);
-            atomicAdd(a.force_acc + 6 * s + 4, rr[2] * dp[0] - rr[0] * dp[2]);
-            atomicAdd(a.force_acc + 6 * s + 5, rr[0] * dp[1] - rr[1] * dp[0]);
-          }
-        }
-        link++;
-      }
-      if (sa >= 0)
-        for (int c = 0; c < 6; c++) acc[c] = a.list_cst[c * a.list_cap + t] + (double)dacc[c];
-    }
-    if (a.zy_pre)  // the next step's Eq. 16 reads them
-      for (int i = 0; i < Q; i++) ((T *)a.zy_pre)[(long long)i * a.fs + n] = f[i];
-    const uint8_t fl = a.flags[n];
-    T Fx, Fy, Fz;
-    node_force<T, T>(a, n, fl, Fx, Fy, Fz);
-    const Coll<T> c = make_coll<LAT, T>(a);
-    collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
-    scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
-  }
-  if (a.force_acc) {
-    const int lane = threadIdx.x & 31;
-    for (int s = 0; s < a.nsolids; s++) {
-      if (!__any_sync(0xffffffffu, sa == s)) continue;
-      for (int c = 0; c < 6; c++) {
-        const double v = warp_sum(sa == s ? acc[c] : 0.0);
-        if (lane == 0) atomicAdd(a.force_acc + 6 * s + c, v);
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------- warp per
-// boundary node.  Lane i (< Q) owns direction i: it pulls f_i or rebuilds it
-// with the bounce-back rule, the moments and the q-moment correction are
-// warp reductions, and each lane writes its own f*_i.  Compared with a thread
-// per node this puts Q times more independent loads in flight for the few
-// thousand boundary nodes, which otherwise sit on the critical path.
-
 // per-lane direction tables packed into compile-time integers
 template <int LAT> __host__ __device__ constexpr unsigned long long pack_dir(int comp) {
   unsigned long long r = 0;
@@ -370,7 +264,7 @@ template <int LAT> __host__ __device__ constexpr unsigned long long pack_dir(int
 }
 template <int LAT> __host__ __device__ constexpr unsigned long long pack_opp() {
   unsigned long long r = 0;
-  for (int i = 0; i < Lat<LAT>::Q; i++) r |= (unsigned long long)Lat<LAT>::opp(i) << (5 * (i % 12));
+  for (int i = 0; i < Lat<LAT>::Q && i < 12; i++) r |= (unsigned long long)Lat<LAT>::opp(i) << (5 * i);
   return r;
 }
 template <int LAT> __host__ __device__ constexpr unsigned long long pack_opp_hi() {
@@ -414,126 +308,229 @@ __device__ __forceinline__ T collide_lane(const KArgs &a, T fi, bool dir, int ex
   return out;
 }
 
-template <int LAT, int CM, typename S, typename T>
-__global__ void __launch_bounds__(256) k_list_warp(const KArgs a) {
+// ---------------------------------------------------------------- boundary
+// nodes.  A block takes NT / Q list nodes at a time, a thread per (node,
+// direction): it pulls f_i or rebuilds it with the bounce-back rule, so that
+// every load of the nodes is in flight at once, and forms its cut link's part
+// of Eq. 17.  A thread per node then collides the populations from
+// shared memory with the same code as the bulk sweep, and the links' parts
+// are summed in FP64 by strips.  A warp per node, with the moments and the
+// q correction as warp reductions, took 11.3 us for the 2.6 k nodes of the
+// 128^3 sphere and 29 us in FP64 (96^3; 14.8 us for the 300 nodes of a 64^2
+// Couette flow): its chains of shuffles and dependent FP64 additions are what
+// this form leaves out.
+template <typename T, int NT> struct ListSmem {
+  T f[NT];
+  T red[6][NT];
+  double cst[6][NT / 9];
+  int sid0[NT / 9];
+};
+
+template <int LAT, int CM, typename S, typename T, int NT, int POL>
+__device__ __forceinline__ void list_group(const KArgs &a, const S *src, S *dst, double *force_acc,
+                                           int group, int cnt, ListSmem<T, NT> &sm) {
   using L = Lat<LAT>;
-  constexpr int Q = L::Q;
+  constexpr int Q = L::Q, NG = NT / Q;
   constexpr unsigned long long PX = pack_dir<LAT>(0), PY = pack_dir<LAT>(1), PZ = pack_dir<LAT>(2);
   constexpr unsigned long long PO = pack_opp<LAT>(), POH = pack_opp_hi<LAT>();
-  __shared__ double part[8][6];
-  __shared__ int psid[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int t = blockIdx.x * (blockDim.x >> 5) + warp;  // list entry of this warp
-  int cnt = a.counts[0];
-  if (cnt > a.list_cap) cnt = a.list_cap;
-  const bool active = t < cnt && !(a.flags[a.list_node[t]] & FL_FACE);
-  const bool dir = lane < Q;
+  const int tid = threadIdx.x;
+  const int i = tid / NG, k = tid - i * NG;
+  const int t = group * NG + k;
+  const bool item = i < Q && t < cnt;
   const T isc = kisc<T>(a);
-  const S *__restrict__ src = (const S *)a.src;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  int sa = -1;
-  if (active) {
-    const long long n = a.list_node[t];
-    const uint32_t mask = a.list_mask[t];
-    const int lo = a.list_link[t];
-    int x, y, z;
-    node_xyz(n, a.nx, a.ny, x, y, z);
-    const int ex = (int)((PX >> (2 * lane)) & 3ull) - 1;
-    const int ey = (int)((PY >> (2 * lane)) & 3ull) - 1;
-    const int ez = (int)((PZ >> (2 * lane)) & 3ull) - 1;
-    const int cls = ex * ex + ey * ey + ez * ez;
-    const T w = cls == 0 ? (T)L::w(0) : (cls == 1 ? (T)L::w(1) : (T)L::w(Q - 1));
-    const int ib = lane < 12 ? (int)((PO >> (5 * lane)) & 31ull) : (int)((POH >> (5 * (lane - 12))) & 31ull);
-    const bool cut = dir && ((mask >> lane) & 1u);
-    T fi = 0, fs = 0;
-    int link = 0;
-    if (cut) {
-      link = lo + __popc(mask & ((1u << lane) - 1u));
-      fi = ibb_value<LAT, S, T, T>(a, src, lane, x, y, z, n, link, isc, fs);
-      (void)ib;
-    } else if (dir) {
-      const long long sn = wrap(x - ex, a.nx) +
-                           (long long)a.nx * (wrap(y - ey, a.ny) + (long long)a.ny * wrap(z - ez, a.nz));
-      fi = Store<S>::ld(src + (long long)lane * a.fs + sn, isc);
+  long long n = 0;
+  uint32_t mask = 0;
+  uint8_t fl = 0;
+  T fi = 0, part[6] = {0, 0, 0, 0, 0, 0};
+  if (item) {
+    n = a.list_node[t];
+    fl = a.flags[n];
+    mask = a.list_mask[t];
+    if (mask) {
+      // the node's state-independent sums, and the solid they belong to
+      if (i < 6) sm.cst[i][k] = a.list_cst[(long long)i * a.list_cap + t];
+      if (i == 0) sm.sid0[k] = (fl & FL_FACE) ? -1 : a.links.sid[a.list_link[t]];
+    } else if (i == 0) {
+      sm.sid0[k] = -1;
     }
-    if (a.zy_pre) {
-      // every lane has read its Eq. 16 input before any lane replaces it
-      __syncwarp();
-      if (dir) ((T *)a.zy_pre)[(long long)lane * a.fs + n] = fi;
+    if (!(fl & FL_FACE)) {
+      int x, y, z;
+      node_xyz(n, a.nx, a.ny, x, y, z);
+      const int ex = (int)((PX >> (2 * i)) & 3ull) - 1;
+      const int ey = (int)((PY >> (2 * i)) & 3ull) - 1;
+      const int ez = (int)((PZ >> (2 * i)) & 3ull) - 1;
+      if ((mask >> i) & 1u) {
+        const int ib = i < 12 ? (int)((PO >> (5 * i)) & 31ull) : (int)((POH >> (5 * (i - 12))) & 31ull);
+        const int lo = a.list_link[t];
+        const int link = lo + __popc(mask & ((1u << i) - 1u));
+        T fs;
+        fi = ibb_value<LAT, S, T, T, POL>(a, src, i, ib, ex, ey, ez, x, y, z, n, link, isc, fs);
+        // f*_ib(e_ib - u_w) - f_i(e_i - u_w) = -2 w_i e_i
+        //   - d*_ib (e_i + u_w) - d_i (e_i - u_w)   (d: deviations); the first
+        // term of the links to the node's first solid was summed per node
+        // when the geometry was built
+        const int s = a.links.sid[link];
+        const int s0 = a.links.sid[lo];
+        const T uw[3] = {((const T *)a.links.uw[0])[link], ((const T *)a.links.uw[1])[link],
+                         ((const T *)a.links.uw[2])[link]};
+        const T r[3] = {((const T *)a.links.arm[0])[link], ((const T *)a.links.arm[1])[link],
+                        ((const T *)a.links.arm[2])[link]};
+        const T e[3] = {(T)ex, (T)ey, (T)ez};
+        if (s == s0) {
+          for (int c = 0; c < 3; c++) part[c] = -fs * (e[c] + uw[c]) - fi * (e[c] - uw[c]);
+          part[3] = r[1] * part[2] - r[2] * part[1];
+          part[4] = r[2] * part[0] - r[0] * part[2];
+          part[5] = r[0] * part[1] - r[1] * part[0];
+        } else {
+          // a second solid seen from this node (narrow gap): full FP64
+          const int cls = ex * ex + ey * ey + ez * ez;
+          const double w = cls == 1 ? L::w(1) : L::w(Q - 1);
+          const double fsd = w + (double)fs, fid = w + (double)fi;
+          double q[3];
+          for (int c = 0; c < 3; c++)
+            q[c] = fsd * (-(double)e[c] - (double)uw[c]) - fid * ((double)e[c] - (double)uw[c]);
+          const double rr[3] = {(double)r[0], (double)r[1], (double)r[2]};
+          atomicAdd(force_acc + 6 * s + 0, q[0]);
+          atomicAdd(force_acc + 6 * s + 1, q[1]);
+          atomicAdd(force_acc + 6 * s + 2, q[2]);
+          atomicAdd(force_acc + 6 * s + 3, rr[1] * q[2] - rr[2] * q[1]);
+          atomicAdd(force_acc + 6 * s + 4, rr[2] * q[0] - rr[0] * q[2]);
+          atomicAdd(force_acc + 6 * s + 5, rr[0] * q[1] - rr[1] * q[0]);
+        }
+      } else {
+        const long long sn = wrap(x - ex, a.nx) +
+                             (long long)a.nx * (wrap(y - ey, a.ny) + (long long)a.ny * wrap(z - ez, a.nz));
+        fi = Store<S>::template ld<POL>(src + (long long)i * a.fs + sn, isc);
+      }
     }
-    const uint8_t fl = a.flags[n];
+  }
+  sm.f[tid] = fi;
+#pragma unroll
+  for (int c = 0; c < 6; c++) sm.red[c][tid] = part[c];
+  __syncthreads();
+  // Eq. 16 reads a node's kept populations in the threads above
+  if (item && a.zy_pre && !(fl & FL_FACE)) ((T *)a.zy_pre)[(long long)i * a.fs + n] = fi;
+  if (item && i == 0 && !(fl & FL_FACE)) {
     T Fx, Fy, Fz;
     node_force<T, T>(a, n, fl, Fx, Fy, Fz);
-    const T out = collide_lane<LAT, CM, T>(a, fi, dir, ex, ey, ez, cls, w, Fx, Fy, Fz);
-    if (dir) Store<S>::st((S *)a.dst + (long long)lane * a.fs + n, out, isc);
-    // Eq. 17 on this node's cut links (first solid: deviation part here,
-    // state-independent part from the geometry build)
-    const int first = mask ? __ffs(mask) - 1 : -1;
-    if (first >= 0) {
-      sa = a.links.sid[lo];
-      T dp[3] = {0, 0, 0}, tq[3] = {0, 0, 0};
-      if (cut) {
-        const int s = a.links.sid[link];
-        const T *uw0 = (const T *)a.links.uw[0], *uw1 = (const T *)a.links.uw[1],
-                *uw2 = (const T *)a.links.uw[2];
-        const T *ar0 = (const T *)a.links.arm[0], *ar1 = (const T *)a.links.arm[1],
-                *ar2 = (const T *)a.links.arm[2];
-        const T uw[3] = {uw0[link], uw1[link], uw2[link]};
-        const T r[3] = {ar0[link], ar1[link], ar2[link]};
-        const T e[3] = {(T)ex, (T)ey, (T)ez};
-        T d[3];
-        for (int k = 0; k < 3; k++) d[k] = -fs * (e[k] + uw[k]) - fi * (e[k] - uw[k]);
-        if (s == sa) {
-          for (int k = 0; k < 3; k++) dp[k] = d[k];
-          tq[0] = r[1] * d[2] - r[2] * d[1];
-          tq[1] = r[2] * d[0] - r[0] * d[2];
-          tq[2] = r[0] * d[1] - r[1] * d[0];
-        } else {
-          // a second solid seen from this node: full FP64 contribution
-          const double wi = (double)w;
-          const double fsd = wi + (double)fs, fid = wi + (double)fi;
-          double q[3];
-          for (int k = 0; k < 3; k++)
-            q[k] = fsd * (-(double)e[k] - (double)uw[k]) - fid * ((double)e[k] - (double)uw[k]);
-          const double rr[3] = {(double)r[0], (double)r[1], (double)r[2]};
-          atomicAdd(a.force_acc + 6 * s + 0, q[0]);
-          atomicAdd(a.force_acc + 6 * s + 1, q[1]);
-          atomicAdd(a.force_acc + 6 * s + 2, q[2]);
-          atomicAdd(a.force_acc + 6 * s + 3, rr[1] * q[2] - rr[2] * q[1]);
-          atomicAdd(a.force_acc + 6 * s + 4, rr[2] * q[0] - rr[0] * q[2]);
-          atomicAdd(a.force_acc + 6 * s + 5, rr[0] * q[1] - rr[1] * q[0]);
+    T f[Q];
+#pragma unroll
+    for (int d = 0; d < Q; d++) f[d] = sm.f[d * NG + k];
+    const Coll<T> c = make_coll<LAT, T>(a);
+    collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
+    scatter<LAT, S, T>(dst, a.fs, n, isc, f);
+  }
+  if (force_acc) {
+    // Eq. 17: the links' parts of each node in the compile-time order of the
+    // directions (compute type), then the nodes in FP64: the sums do not
+    // depend on the order of the list beyond FP64 rounding
+    for (int q = tid; q < 6 * NG; q += NT) {
+      const int c = q / NG, kk = q - c * NG;
+      if (group * NG + kk >= cnt) continue;
+      T v = 0;
+#pragma unroll
+      for (int d = 1; d < Q; d++) v += sm.red[c][d * NG + kk];
+      if (sm.sid0[kk] >= 0) sm.cst[c][kk] += (double)v;
+    }
+    __syncthreads();
+    for (int s = 0; s < a.nsolids; s++) {
+      if (tid < 96) {
+        // 16 threads per component
+        const int c = tid >> 4, p = tid & 15;
+        double v = 0;
+        bool any = false;
+        for (int kk = p; kk < NG && group * NG + kk < cnt; kk += 16)
+          if (sm.sid0[kk] == s) {
+            v += sm.cst[c][kk];
+            any = true;
+          }
+        if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, 16);
+          if (p == 0 && v != 0.0) atomicAdd(force_acc + 6 * s + c, v);
         }
       }
-      for (int k = 0; k < 3; k++) {
-        acc[k] = a.list_cst[k * a.list_cap + t] + (double)wsum<T>(dp[k]);
-        acc[3 + k] = a.list_cst[(3 + k) * a.list_cap + t] + (double)wsum<T>(tq[k]);
-      }
     }
   }
-  // block reduction of the per-node sums, one FP64 atomic per component
-  if (lane == 0) {
-    psid[warp] = sa;
-    for (int k = 0; k < 6; k++) part[warp][k] = acc[k];
+  __syncthreads();  // the next group reuses the shared arrays
+}
+
+constexpr int kListBlock = 128;
+template <int LAT, int CM, typename S, typename T>
+__global__ void __launch_bounds__(kListBlock) k_list(const KArgs a) {
+  __shared__ ListSmem<T, kListBlock> sm;
+  int cnt = a.counts[0];
+  if (cnt > a.list_cap) cnt = a.list_cap;
+  if ((int)blockIdx.x * (kListBlock / Lat<LAT>::Q) >= cnt) return;
+  list_group<LAT, CM, S, T, kListBlock, LD_NC>(a, (const S *)a.src, (S *)a.dst, a.force_acc,
+                                               (int)blockIdx.x, cnt, sm);
+}
+
+// The force spread to list node t: its row of markers (solids at rest).
+template <typename T, int POL>
+__device__ __forceinline__ void gather_force(const KArgs &a, int t, T (&s)[3]) {
+  const T *F = (const T *)a.tab.FdV, *nw = (const T *)a.tab.nw;
+  const int nm = a.tab.nmark;
+  const int e0 = a.tab.nrow[t], e1 = a.tab.nrow[t + 1];
+  s[0] = s[1] = s[2] = 0;
+#pragma unroll 4
+  for (int e = e0; e < e1; e++) {
+    const int m = a.tab.ncol[e];
+    const T w = nw[e];
+    s[0] += w * ld_pol<POL>(F + m);
+    s[1] += w * ld_pol<POL>(F + nm + m);
+    s[2] += w * ld_pol<POL>(F + 2 * nm + m);
   }
-  __syncthreads();
-  if (threadIdx.x < 6) {
-    const int k = threadIdx.x, nw = blockDim.x >> 5;
-    int s0 = -1;
-    for (int wi = 0; wi < nw; wi++)
-      if (psid[wi] >= 0) {
-        s0 = psid[wi];
-        break;
-      }
-    double sum = 0;
-    for (int wi = 0; wi < nw; wi++) {
-      if (psid[wi] < 0) continue;
-      if (psid[wi] == s0)
-        sum += part[wi][k];
-      else
-        atomicAdd(a.force_acc + 6 * psid[wi] + k, part[wi][k]);
-    }
-    if (s0 >= 0) atomicAdd(a.force_acc + 6 * s0 + k, sum);
+}
+
+// IBM band node t (no cut links): pull, the spread force (gathered from the
+// markers' rows and kept in the dense field for queries and the face kernel,
+// or already there), collide.  A thread per node: the thousands of band nodes
+// of a large lattice run beside its bulk sweep, whose SMs they should hold as
+// little as possible (as a block of threads per node's directions the 160^3
+// FP16 IBM step took 77 us instead of 68).
+template <int LAT, int CM, typename S, typename T, int POL>
+__device__ __forceinline__ void ibm_list_node(const KArgs &a, const S *src, S *dst, int t) {
+  const long long n = a.list_node[t];
+  const uint8_t fl = a.flags[n];
+  if (a.tab.nmark > 0) {
+    T s[3];
+    gather_force<T, POL>(a, t, s);
+    for (int c = 0; c < 3; c++) ((T *)const_cast<void *>(a.f_ibm))[c * a.N + n] = s[c];
   }
+  if (fl & FL_FACE) return;  // the face kernel's
+  int x, y, z;
+  node_xyz(n, a.nx, a.ny, x, y, z);
+  const T isc = kisc<T>(a);
+  T f[Lat<LAT>::Q];
+  gather_pull<LAT, S, T, POL>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
+  T Fx, Fy, Fz;
+  node_force<T, T>(a, n, fl, Fx, Fy, Fz);
+  const Coll<T> c = make_coll<LAT, T>(a);
+  collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
+  scatter<LAT, S, T>(dst, a.fs, n, isc, f);
+}
+
+template <int LAT, int CM, typename S, typename T>
+__global__ void __launch_bounds__(64) k_list_ibm(const KArgs a) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  int cnt = a.counts[0];
+  if (cnt > a.list_cap) cnt = a.list_cap;
+  if (t < cnt) ibm_list_node<LAT, CM, S, T, LD_NC>(a, (const S *)a.src, (S *)a.dst, t);
+}
+
+// The spread force of every list node from the markers' rows, for a state
+// that is not swept next (right after an initialisation or a restart).
+template <typename T>
+__global__ void __launch_bounds__(128) k_ibm_gather(const KArgs a) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  int cnt = a.counts[0];
+  if (cnt > a.list_cap) cnt = a.list_cap;
+  if (t >= cnt) return;
+  const long long n = a.list_node[t];
+  T s[3];
+  gather_force<T, LD_NC>(a, t, s);
+  for (int c = 0; c < 3; c++) ((T *)const_cast<void *>(a.f_ibm))[c * a.N + n] = s[c];
 }
 
 template <int LAT, int CM, typename S, typename T>
@@ -681,16 +678,9 @@ template <int LAT, typename S, typename T>
 __device__ __forceinline__ T face_pull(const KArgs &a, const S *__restrict__ src, int x, int y,
                                        int z, int i, T isc);
 
-template <int LAT, typename S, typename T>
-__global__ void __launch_bounds__(64) k_band_vel(const KArgs a) {
+template <int LAT, typename S, typename T, int POL>
+__device__ __forceinline__ void band_velocity(const KArgs &a, const S *src, int t) {
   using L = Lat<LAT>;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  // this step's force record, accumulated by the IBM kernels that follow on
-  // the same stream, starts at zero
-  if (a.force_acc && t < 6 * kMaxSolids) a.force_acc[t] = 0.0;
-  int cnt = a.counts[0];
-  if (cnt > a.list_cap) cnt = a.list_cap;
-  if (t >= cnt) return;
   const long long n = a.list_node[t];
   const uint8_t fl = a.flags[n];
   if (!(fl & FL_BAND)) return;
@@ -699,25 +689,38 @@ __global__ void __launch_bounds__(64) k_band_vel(const KArgs a) {
   T f[L::Q];
   const T isc = kisc<T>(a);
   if (a.local_gather)
-    gather_local<LAT, S, T>((const S *)a.src, a.fs, n, isc, f);
+    gather_local<LAT, S, T>(src, a.fs, n, isc, f);
   else if (fl & FL_FACE)  // next to a velocity or stress-free domain face
-    for (int i = 0; i < L::Q; i++) f[i] = face_pull<LAT, S, T>(a, (const S *)a.src, x, y, z, i, isc);
+    for (int i = 0; i < L::Q; i++) f[i] = face_pull<LAT, S, T>(a, src, x, y, z, i, isc);
   else
-    gather_pull<LAT, S, T>((const S *)a.src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
+    gather_pull<LAT, S, T, POL>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
   T j[3] = {0, 0, 0};
-#pragma unroll
-  for (int i = 0; i < L::Q; i++) {
-    j[0] += (T)L::ex(i) * f[i];
-    j[1] += (T)L::ey(i) * f[i];
-    j[2] += (T)L::ez(i) * f[i];
-  }
+  static_for<L::Q>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    static_for<3>([&](auto ac) {
+      constexpr int c = decltype(ac)::value;
+      if constexpr (ecomp<LAT>(c, i) == 1) j[c] += f[i];
+      if constexpr (ecomp<LAT>(c, i) == -1) j[c] -= f[i];
+    });
+  });
   const bool g = !(fl & FL_NOG);
   T *ub = (T *)a.u_band;
-  T *fi = (T *)a.f_ibm;
+  T *fi = (T *)const_cast<void *>(a.f_ibm);
   for (int c = 0; c < 3; c++) {
     ub[c * a.N + n] = j[c] + (g ? (T)0.5 * kg<T>(a, c) : (T)0);
-    fi[c * a.N + n] = (T)0;
+    if (a.tab.nmark == 0) fi[c * a.N + n] = (T)0;  // the markers add their forces
   }
+}
+
+template <int LAT, typename S, typename T>
+__global__ void __launch_bounds__(64) k_band_vel(const KArgs a) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  // this step's force record, accumulated by the IBM kernels that follow on
+  // the same stream, starts at zero
+  if (a.force_acc && t < 6 * kMaxSolids) a.force_acc[t] = 0.0;
+  int cnt = a.counts[0];
+  if (cnt > a.list_cap) cnt = a.list_cap;
+  if (t < cnt) band_velocity<LAT, S, T, LD_NC>(a, (const S *)a.src, t);
 }
 
 // Full FP64 f -> stored deviations (solid nodes get 0).
@@ -1012,6 +1015,12 @@ __global__ void __launch_bounds__(256) k_kempe(const KArgs a) {
   }
 }
 
+}  // namespace lbm
+
+#include "run_impl.cuh"
+
+namespace lbm {
+
 // ---------------------------------------------------------------- launch
 inline int div_up(long long a, int b) { return (int)((a + b - 1) / b); }
 
@@ -1038,13 +1047,13 @@ bool launch_bulk_vec_w(const KArgs &a, int want, bool packed, cudaStream_t st) {
   // the hint is built for the default shape only
   if (W == 2 && packed) {
     if (2 * Lat<LAT>::Q * a.fs * (long long)sizeof(S) <= kReuseBytes)
-      k_bulk_vec<LAT, CM, S, W, true, W == 2><<<grid, want, 0, st>>>(a);
+      k_bulk_vec<LAT, CM, S, W, true, W == 2 ? LD_ONCE : LD_NC><<<grid, want, 0, st>>>(a);
     else
-      k_bulk_vec<LAT, CM, S, W, true, false><<<grid, want, 0, st>>>(a);
+      k_bulk_vec<LAT, CM, S, W, true, LD_NC><<<grid, want, 0, st>>>(a);
   } else if (packed) {
-    k_bulk_vec<LAT, CM, S, W, true, false><<<grid, want, 0, st>>>(a);
+    k_bulk_vec<LAT, CM, S, W, true, LD_NC><<<grid, want, 0, st>>>(a);
   } else {
-    k_bulk_vec<LAT, CM, S, W, false, false><<<grid, want, 0, st>>>(a);
+    k_bulk_vec<LAT, CM, S, W, false, LD_NC><<<grid, want, 0, st>>>(a);
   }
   return true;
 }
@@ -1190,18 +1199,14 @@ void launch_one(SweepOp op, const KArgs &a, cudaStream_t st) {
     break;
   }
   case OP_LIST_SWEEP:
-    if (a.list_cap > 0) {
-      if (CM != CM_MRT && !a.list_thread) {
-        // a warp per boundary node, list_block / 32 nodes per block
-        const int lb = a.list_block >= 64 ? (a.list_block > 256 ? 256 : a.list_block) : 256;
-        if constexpr (CM != CM_MRT) k_list_warp<LAT, CM, S, T><<<div_up(lc, lb / 32), lb, 0, st>>>(a);
-      } else {
-        // general MRT rates, or IBM band nodes (no cut links): a thread per
-        // node (small blocks spread the boundary nodes over many SMs)
-        const int lb = a.list_block > 0 && a.list_block <= 128 ? a.list_block : 64;
-        k_list<LAT, CM, S, T><<<div_up(lc, lb), lb, 0, st>>>(a);
-      }
-    }
+    if (a.list_cap > 0 && a.ibm)
+      k_list_ibm<LAT, CM, S, T><<<div_up(lc, 64), 64, 0, st>>>(a);
+    else if (a.list_cap > 0)
+      k_list<LAT, CM, S, T>
+          <<<div_up(lc, kListBlock / Lat<LAT>::Q), kListBlock, 0, st>>>(a);
+    break;
+  case OP_IBM_GATHER:
+    if (a.list_cap > 0) k_ibm_gather<T><<<div_up(lc, 128), 128, 0, st>>>(a);
     break;
   case OP_ZY_SEED:
     if (a.list_cap > 0 && a.zy_pre) k_zy_seed<LAT, S, T><<<div_up(lc, 128), 128, 0, st>>>(a);

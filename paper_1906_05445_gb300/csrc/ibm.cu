@@ -9,97 +9,13 @@
 // block in FP64.
 #include <cooperative_groups.h>
 
-#include "lbm_device.cuh"
-#include "lbm_internal.h"
+#include "ibm_device.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace lbm {
 
 namespace {
-
-// The one-dimensional delta-function kernels compared in Sec. 3.1:
-// Peskin's 4-point kernel (Eq. 6, the default), Roma, Peskin & Berger's
-// 3-point kernel, the 2-point linear kernel, and the 4-point cosine kernel of
-// Appendix B.  Each support lies inside the 4-point window from floor(X) - 1,
-// so every kernel uses the same 4^d stencil (points outside the support get
-// weight 0).
-template <typename T>
-__device__ __forceinline__ T phi_k(int kernel, T r) {
-  const T a = fabs(r);
-  switch (kernel) {
-  case LBM_DELTA_ROMA3:
-    if (a >= (T)1.5) return (T)0;
-    if (a <= (T)0.5) return ((T)1 + sqrt((T)1 - (T)3 * a * a)) / (T)3;
-    return ((T)5 - (T)3 * a - sqrt((T)1 - (T)3 * ((T)1 - a) * ((T)1 - a))) / (T)6;
-  case LBM_DELTA_LINEAR2:
-    return a >= (T)1 ? (T)0 : (T)1 - a;
-  case LBM_DELTA_COSINE4:
-    return a >= (T)2 ? (T)0 : ((T)1 + cospi(r / (T)2)) / (T)4;
-  default:
-    if (a >= (T)2) return (T)0;
-    if (a >= (T)1) return ((T)5 - (T)2 * a - sqrt((T)-7 + (T)12 * a - (T)4 * a * a)) / (T)8;
-    return ((T)3 - (T)2 * a + sqrt((T)1 + (T)4 * a - (T)4 * a * a)) / (T)8;
-  }
-}
-
-struct Marker {
-  double X[3];   // position
-  double r[3];   // X - centre (z dropped for cylinders and 2D)
-  int s;
-};
-
-__device__ __forceinline__ Marker marker(const IbmArgs &a, int m) {
-  Marker k;
-  k.s = a.msid[m];
-  const SolidDev b = solid_of(a, k.s);
-  const double dx = a.dir[m], dy = a.dir[a.nmark + m], dz = a.dir[2 * a.nmark + m];
-  k.X[0] = b.c[0] + b.RL * dx;
-  k.X[1] = b.c[1] + b.RL * dy;
-  if (a.dim == 2)
-    k.X[2] = 0.0;
-  else if (b.kind == LBM_CYLINDER_Z)
-    k.X[2] = dz;  // plane of the ring
-  else
-    k.X[2] = b.c[2] + b.RL * dz;
-  k.r[0] = k.X[0] - b.c[0];
-  k.r[1] = k.X[1] - b.c[1];
-  k.r[2] = (a.dim == 2 || b.kind == LBM_CYLINDER_Z) ? 0.0 : k.X[2] - b.c[2];
-  return k;
-}
-
-// Stencil of a marker: the 4^d nodes from floor(X) - 1; the marker position
-// is FP64, the offsets of the stencil points from it are formed once and the
-// per-point arithmetic runs in the compute type.
-template <typename T> struct Stencil {
-  int ix, iy, iz;  // first stencil node (unwrapped)
-  T dx, dy, dz;    // first node - X
-};
-
-template <typename T>
-__device__ __forceinline__ Stencil<T> stencil_of(const IbmArgs &a, const Marker &k) {
-  Stencil<T> st;
-  const double bx = floor(k.X[0]) - 1.0, by = floor(k.X[1]) - 1.0;
-  const double bz = a.dim == 3 ? floor(k.X[2]) - 1.0 : 0.0;
-  st.ix = (int)bx;
-  st.iy = (int)by;
-  st.iz = (int)bz;
-  st.dx = (T)(bx - k.X[0]);
-  st.dy = (T)(by - k.X[1]);
-  st.dz = a.dim == 3 ? (T)(bz - k.X[2]) : (T)0;
-  return st;
-}
-
-template <typename T>
-__device__ __forceinline__ long long stencil_point(const IbmArgs &a, const Stencil<T> &st,
-                                                   int p, T &wgt) {
-  const int kx = p & 3, ky = (p >> 2) & 3, kz = p >> 4;
-  wgt = phi_k<T>(a.kernel, st.dx + (T)kx) * phi_k<T>(a.kernel, st.dy + (T)ky);
-  if (a.dim == 3) wgt *= phi_k<T>(a.kernel, st.dz + (T)kz);
-  const int x = wrap(st.ix + kx, a.nx), y = wrap(st.iy + ky, a.ny);
-  const int z = a.dim == 3 ? wrap(st.iz + kz, a.nz) : 0;
-  return x + (long long)a.nx * (y + (long long)a.ny * z);
-}
 
 // Stencil base and the 4^dim weights of every marker, from its FP64
 // position (one warp per marker, a lane per stencil point).
@@ -119,13 +35,6 @@ __global__ void __launch_bounds__(128) k_prepare(const IbmArgs a) {
     wts[p] = wgt;
   }
   if (lane == 0) a.mk_base[m] = make_int4(stc.ix, stc.iy, stc.iz, k.s);
-}
-
-__device__ __forceinline__ long long table_node(const IbmArgs &a, int4 b, int p) {
-  const int kx = p & 3, ky = (p >> 2) & 3, kz = p >> 4;
-  const int x = wrap(b.x + kx, a.nx), y = wrap(b.y + ky, a.ny);
-  const int z = a.dim == 3 ? wrap(b.z + kz, a.nz) : 0;
-  return x + (long long)a.nx * (y + (long long)a.ny * z);
 }
 
 // interpolated velocity of marker m (all lanes get the sum)
@@ -278,6 +187,148 @@ __global__ void __launch_bounds__(128) k_fused(const IbmArgs a) {
     spread_marker<T>(a, m, lane, b, F);
   }
   if (a.reduce_force) reduce_solid_force(a, active, lane, warp, k, F, dV);
+}
+
+// ---------------------------------------------------------------- tables
+// Built once per geometry of solids at rest (ibm_device.cuh says what they
+// are for) by exhaustive search, a warp per row: the rows come out in marker
+// order without sorting or atomics.  COUNT: row lengths only.
+
+// whether node (x, y, z) lies in the stencil of base b, and its point
+__device__ __forceinline__ int stencil_index(const IbmArgs &a, int4 b, int x, int y, int z) {
+  const int kx = wrap(x - b.x, a.nx), ky = wrap(y - b.y, a.ny);
+  const int kz = a.dim == 3 ? wrap(z - b.z, a.nz) : 0;
+  return (kx < 4 && ky < 4 && kz < 4) ? kx + 4 * ky + 16 * kz : -1;
+}
+
+template <typename T, bool COUNT>
+__global__ void __launch_bounds__(128) k_tab_nodes(const IbmArgs a, const int *list_node, int nlist,
+                                                   int *row, int *col, T *wt) {
+  const int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (t >= nlist) return;
+  const int n = list_node[t];
+  const int x = n % a.nx, y = (n / a.nx) % a.ny, z = n / (a.nx * a.ny);
+  const int npts = a.dim == 3 ? 64 : 16;
+  int at = COUNT ? 0 : row[t];
+  for (int m0 = 0; m0 < a.nmark; m0 += 32) {
+    const int m = m0 + lane;
+    const int p = m < a.nmark ? stencil_index(a, a.mk_base[m], x, y, z) : -1;
+    const unsigned hit = __ballot_sync(0xffffffffu, p >= 0);
+    if (!COUNT && p >= 0) {
+      const int e = at + __popc(hit & ((1u << lane) - 1u));
+      col[e] = m;
+      wt[e] = ((const T *)a.mk_wts)[(long long)m * npts + p];
+    }
+    at += __popc(hit);
+  }
+  if (COUNT && lane == 0) row[t] = at;
+}
+
+// separation of two stencil bases on an axis of n >= 8 nodes, or 8 when the
+// stencils do not meet
+__device__ __forceinline__ int base_shift(int b0, int b1, int n) {
+  const int d = wrap(b1 - b0, n);
+  return d <= 3 ? d : (n - d <= 3 ? d - n : 8);
+}
+
+// sum_k phi(x0 + k) phi(x1 + k - d): node k of the first stencil is node k - d
+// of the second, whose base lies d nodes further
+template <typename T>
+__device__ __forceinline__ T overlap(int kernel, T x0, T x1, int d) {
+  T s = (T)0;
+  for (int k = 0; k < 4; k++) {
+    const int q = k - d;
+    if (q >= 0 && q < 4) s += phi_k<T>(kernel, x0 + (T)k) * phi_k<T>(kernel, x1 + (T)q);
+  }
+  return s;
+}
+
+template <typename T, bool COUNT>
+__global__ void __launch_bounds__(128) k_tab_markers(const IbmArgs a, int *row, int *col, T *wt) {
+  const int m = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (m >= a.nmark) return;
+  const int4 b = a.mk_base[m];
+  const Stencil<T> s0 = stencil_of<T>(a, marker(a, m));
+  int at = COUNT ? 0 : row[m];
+  for (int k0 = 0; k0 < a.nmark; k0 += 32) {
+    const int k = k0 + lane;
+    int dx = 8, dy = 8, dz = 8;
+    if (k < a.nmark) {
+      const int4 c = a.mk_base[k];
+      dx = base_shift(b.x, c.x, a.nx);
+      dy = base_shift(b.y, c.y, a.ny);
+      dz = a.dim == 3 ? base_shift(b.z, c.z, a.nz) : 0;
+    }
+    const bool meet = dx < 8 && dy < 8 && dz < 8;
+    const unsigned hit = __ballot_sync(0xffffffffu, meet);
+    if (!COUNT && meet) {
+      const int e = at + __popc(hit & ((1u << lane) - 1u));
+      const Stencil<T> s1 = stencil_of<T>(a, marker(a, k));
+      T w = overlap<T>(a.kernel, s0.dx, s1.dx, dx) * overlap<T>(a.kernel, s0.dy, s1.dy, dy);
+      if (a.dim == 3) w *= overlap<T>(a.kernel, s0.dz, s1.dz, dz);
+      col[e] = k;
+      wt[e] = w * (T)a.dV[k];
+    }
+    at += __popc(hit);
+  }
+  if (COUNT && lane == 0) row[m] = at;
+}
+
+// exclusive prefix sum of n counts in place, the total in v[n] (one block)
+__global__ void __launch_bounds__(1024) k_tab_scan(int *v, int n) {
+  __shared__ int sh[1024];
+  const int t = threadIdx.x;
+  const int per = (n + 1023) / 1024;
+  const int i0 = min(n, t * per), i1 = min(n, i0 + per);
+  int s = 0;
+  for (int i = i0; i < i1; i++) s += v[i];
+  sh[t] = s;
+  __syncthreads();
+  for (int o = 1; o < 1024; o <<= 1) {
+    const int add = t >= o ? sh[t - o] : 0;
+    __syncthreads();
+    sh[t] += add;
+    __syncthreads();
+  }
+  int at = sh[t] - s;
+  for (int i = i0; i < i1; i++) {
+    const int c = v[i];
+    v[i] = at;
+    at += c;
+  }
+  if (t == 1023) v[n] = sh[1023];
+}
+
+// desired velocity and lever arm of every marker (solids at rest)
+__global__ void __launch_bounds__(128) k_tab_desired(const IbmArgs a, double *Ud, double *arm) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= a.nmark) return;
+  const Marker k = marker(a, m);
+  const double zero[3] = {0, 0, 0};
+  double F[3];
+  direct_force(a, k, zero, F);
+  for (int c = 0; c < 3; c++) {
+    Ud[c * a.nmark + m] = F[c];
+    arm[c * a.nmark + m] = k.r[c];
+  }
+}
+
+// a warp per marker; pass 0 interpolates u~, the later ones iterate
+template <typename T>
+__global__ void __launch_bounds__(128) k_marker_pass(const KArgs a, int dim, int pass, bool last) {
+  __shared__ double part[4][6];
+  __shared__ int psid[4];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m = blockIdx.x * 4 + w;
+  if (lane == 0) psid[w] = -1;
+  __syncwarp();
+  if (m < a.tab.nmark) {
+    if (pass == 0) marker_first<T>(a.tab, a, dim, m, lane, last, part[w], &psid[w]);
+    else marker_next<T>(a.tab, dim, m, lane, pass, last, part[w], &psid[w]);
+  }
+  if (last) marker_block_force<4>(a.force_acc, a.nsolids, part, psid);
 }
 
 // ---------------------------------------------------------------- cluster
@@ -572,6 +623,43 @@ void launch_ibm_cluster(const IbmArgs &a, const IbmClusterArgs &cl, int precisio
     launch_cluster_t<double>(a, cl, smem, st);
   else
     launch_cluster_t<float>(a, cl, smem, st);
+}
+
+void launch_tab_nodes(const IbmArgs &a, const int *list_node, int nlist, int *row, int *col,
+                      void *wt, int precision, cudaStream_t st) {
+  const int grid = (nlist + 3) / 4;
+  if (!col) {
+    k_tab_nodes<float, true><<<grid, 128, 0, st>>>(a, list_node, nlist, row, nullptr, nullptr);
+    k_tab_scan<<<1, 1024, 0, st>>>(row, nlist);
+  } else if (precision == LBM_FP64) {
+    k_tab_nodes<double, false><<<grid, 128, 0, st>>>(a, list_node, nlist, row, col, (double *)wt);
+  } else {
+    k_tab_nodes<float, false><<<grid, 128, 0, st>>>(a, list_node, nlist, row, col, (float *)wt);
+  }
+}
+
+void launch_tab_markers(const IbmArgs &a, int *row, int *col, void *wt, int precision,
+                        cudaStream_t st) {
+  const int grid = (a.nmark + 3) / 4;
+  if (!col) {
+    k_tab_markers<float, true><<<grid, 128, 0, st>>>(a, row, nullptr, nullptr);
+    k_tab_scan<<<1, 1024, 0, st>>>(row, a.nmark);
+  } else if (precision == LBM_FP64) {
+    k_tab_markers<double, false><<<grid, 128, 0, st>>>(a, row, col, (double *)wt);
+  } else {
+    k_tab_markers<float, false><<<grid, 128, 0, st>>>(a, row, col, (float *)wt);
+  }
+}
+
+void launch_tab_desired(const IbmArgs &a, double *Ud, double *arm, cudaStream_t st) {
+  k_tab_desired<<<(a.nmark + 127) / 128, 128, 0, st>>>(a, Ud, arm);
+}
+
+void launch_marker_pass(const KArgs &a, int dim, int pass, bool last, int precision,
+                        cudaStream_t st) {
+  const int grid = (a.tab.nmark + 3) / 4;
+  if (precision == LBM_FP64) k_marker_pass<double><<<grid, 128, 0, st>>>(a, dim, pass, last);
+  else k_marker_pass<float><<<grid, 128, 0, st>>>(a, dim, pass, last);
 }
 
 }  // namespace lbm

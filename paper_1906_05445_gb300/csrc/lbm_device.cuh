@@ -133,41 +133,52 @@ __host__ __device__ constexpr bool conserved(int k) {
 }
 
 // ---------------------------------------------------------------- storage
+// How a kernel reads populations:
+//   LD_NC   read-only path: nothing writes the array while the kernel runs;
+//   LD_ONCE evict-first (the line is not needed again before it is rewritten);
+//   LD_L2   from L2: a kernel of several steps reads what other SMs wrote
+//           earlier in the same launch, which the read-only path and L1 may
+//           hold stale.
+enum : int { LD_NC = 0, LD_ONCE = 1, LD_L2 = 2 };
+template <int POL, typename P> __device__ __forceinline__ P ld_pol(const P *p) {
+  if constexpr (POL == LD_NC) return __ldg(p);
+  else if constexpr (POL == LD_ONCE) return __ldcs(p);
+  else return __ldcg(p);
+}
 template <typename S> struct Store;
-// ld/st: default caching; ld_stream/st_stream: evict-first (each element is
-// read once and written once per sweep)
+// st_stream: evict-first stores
 template <> struct Store<double> {
-  template <typename T> __device__ static T ld(const double *p, T) { return (T)__ldg(p); }
-  template <typename T> __device__ static T ld_stream(const double *p, T) { return (T)__ldcs(p); }
+  template <int POL = LD_NC, typename T> __device__ static T ld(const double *p, T) {
+    return (T)ld_pol<POL>(p);
+  }
   template <typename T> __device__ static void st(double *p, T v, T) { *p = (double)v; }
   template <typename T> __device__ static void st_stream(double *p, T v, T) { __stcs(p, (double)v); }
 };
 template <> struct Store<float> {
-  template <typename T> __device__ static T ld(const float *p, T) { return (T)__ldg(p); }
-  template <typename T> __device__ static T ld_stream(const float *p, T) { return (T)__ldcs(p); }
+  template <int POL = LD_NC, typename T> __device__ static T ld(const float *p, T) {
+    return (T)ld_pol<POL>(p);
+  }
   template <typename T> __device__ static void st(float *p, T v, T) { *p = (float)v; }
   template <typename T> __device__ static void st_stream(float *p, T v, T) { __stcs(p, (float)v); }
 };
 template <> struct Store<__nv_bfloat16> {
-  template <typename T> __device__ static T ld(const __nv_bfloat16 *p, T) {
-    return (T)__bfloat162float(__ldg(p));
+  template <int POL = LD_NC, typename T> __device__ static T ld(const __nv_bfloat16 *p, T) {
+    return (T)__bfloat162float(ld_pol<POL>(p));
   }
   template <typename T> __device__ static void st(__nv_bfloat16 *p, T v, T) {
     *p = __float2bfloat16_rn((float)v);
   }
-  template <typename T> __device__ static T ld_stream(const __nv_bfloat16 *p, T s) { return ld(p, s); }
   template <typename T> __device__ static void st_stream(__nv_bfloat16 *p, T v, T s) { st(p, v, s); }
 };
 // FP16 keeps d_i * scale (scale = 2^k) so that deviations stay in the normal
 // range; the scale is exact in binary, so it only shifts the exponent.
 template <> struct Store<__half> {
-  template <typename T> __device__ static T ld(const __half *p, T inv_scale) {
-    return (T)__half2float(__ldg(p)) * inv_scale;
+  template <int POL = LD_NC, typename T> __device__ static T ld(const __half *p, T inv_scale) {
+    return (T)__half2float(ld_pol<POL>(p)) * inv_scale;
   }
   template <typename T> __device__ static void st(__half *p, T v, T inv_scale) {
     *p = __float2half_rn((float)(v / inv_scale));
   }
-  template <typename T> __device__ static T ld_stream(const __half *p, T s) { return ld(p, s); }
   template <typename T> __device__ static void st_stream(__half *p, T v, T s) { st(p, v, s); }
 };
 
@@ -301,11 +312,15 @@ template <int LAT, typename C> struct CollW {
 // commutes with rounding, so the stored values equal those of colliding the
 // unscaled deviations.
 // EVEN_FIRST adds the small even part to the old value before the larger odd
-// one, so that the odd part is rounded once: FP32 and FP64 storage (the
-// stress noise of a step is half that of adding the parts first, and the
-// velocity error of a sphere flow started from rest at g = 3.4e-8 is 1.6e-6
-// after 2000 steps against 4.9e-6).  16-bit storage rounds the result to
-// 2^-12 or worse either way and adds the parts first.
+// one, so that the odd part is rounded once: the stress noise of an FP32 step is
+// half that of adding the parts first, and the velocity error of a sphere flow
+// started from rest at g = 3.4e-8 is 1.6e-6 after 2000 steps against 4.9e-6.
+// BF16 storage is also faster with it (160^3 51.7 us per step against 53.3);
+// FP16 storage, whose rounding hides the difference, is not (53.4 / 53.3) and
+// adds the parts first.
+template <typename ST> __host__ __device__ constexpr bool even_first() {
+  return !std::is_same<ST, __half>::value;
+}
 template <int LAT, int CM, int SL, bool EVEN_FIRST, typename V, typename C>
 __device__ __forceinline__ void collide_two_rate(V (&f)[Lat<LAT>::Q], V Fx, V Fy, V Fz,
                                                  const Coll<C> &c) {
@@ -395,10 +410,10 @@ __device__ __forceinline__ void collide_two_rate(V (&f)[Lat<LAT>::Q], V Fx, V Fy
         P = vfma(vbc<V>((C)rw), X[a], Ba);
         O = ga[a];
       } else {
-        constexpr int a = L::ex(i) ? 0 : 1, b = L::ez(i) ? 2 : 1, n = 3 - a - b;
+        constexpr int a = L::ex(i) ? 0 : 1, b = L::ez(i) ? 2 : 1;
         static_assert(enorm2<LAT>(i) == 2 && a < b, "two components");
         V base = Bd;
-        if constexpr (D == 3) base = vsub(Bd, X[n < D ? n : 0]);
+        if constexpr (D == 3) base = vsub(Bd, X[3 - a - b]);
         const V X2 = vfma(u[a], h[b], vmul(u[b], h[a]));
         P = ecomp<LAT>(a, i) * ecomp<LAT>(b, i) > 0 ? vadd(base, X2) : vsub(base, X2);
         O = edot_lead<LAT, i>(g[0], g[1], g[2]);
@@ -414,15 +429,15 @@ __device__ __forceinline__ void collide_two_rate(V (&f)[Lat<LAT>::Q], V Fx, V Fy
   });
 }
 
-// One node; S is the storage type of the populations.
-template <int LAT, int CM, typename S, typename T>
+// One node; ST is the storage type of the populations.
+template <int LAT, int CM, typename ST, typename T>
 __device__ __forceinline__ void collide(T (&f)[Lat<LAT>::Q], T Fx, T Fy, T Fz,
                                         const Coll<T> &c) {
   using L = Lat<LAT>;
   constexpr int Q = L::Q;
   constexpr bool MRT = CM == CM_MRT;
   if constexpr (!MRT) {
-    collide_two_rate<LAT, CM, 0, (sizeof(S) > 2), T, T>(f, Fx, Fy, Fz, c);
+    collide_two_rate<LAT, CM, 0, even_first<ST>(), T, T>(f, Fx, Fy, Fz, c);
     return;
   }
   T drho = 0, jx = 0, jy = 0, jz = 0;

@@ -37,6 +37,25 @@ struct LinkArrays {
   uint8_t *sid;
 };
 
+// IBM tables of solids at rest (ibm_device.cuh): rows of the band nodes and of
+// the markers, T the compute type; nmark 0 without tables.
+struct IbmTab {
+  int nmark;
+  const int4 *base;       // [nmark] first stencil node
+  const void *wts;        // T [nmark][4^dim] stencil weights
+  const double *dV;       // [nmark]
+  const uint8_t *msid;    // [nmark]
+  const double *Ud, *arm; // [3][nmark] desired velocity, lever arm
+  double *dF;             // [3][nmark] force increment
+  void *dFT;              // T [2][3][nmark] the same, of alternate passes
+  double *Fm;             // [3][nmark] force
+  void *FdV;              // T [3][nmark] total force times dV
+  const int *nrow, *ncol; // rows of the list nodes: markers,
+  const void *nw;         // T weights
+  const int *mrow, *mcol; // rows of the markers: coupled markers,
+  const void *mw;         // T coefficients
+};
+
 // FP16 storage keeps (f - w_i) * 2^kFp16ScaleLog2.
 constexpr int kFp16ScaleLog2 = 10;
 
@@ -67,6 +86,8 @@ struct KArgs {
   // IBM dense fields (type T, [3][N]) and flags
   const void *f_ibm;
   void *u_band;
+  int ibm;  // the scheme is direct forcing
+  IbmTab tab;
   // momentum exchange accumulators: [solid][6] doubles (F, T)
   double *force_acc;
   int nsolids;
@@ -85,8 +106,6 @@ struct KArgs {
   int local_gather;  // 1: read src locally (pre-collision state), 0: pull
   int bulk_block;    // threads per block of the bulk sweep (multiple of 32)
   int cache_hints;   // bulk sweep: bit 0 evict-first loads, bit 1 evict-first stores
-  int list_block;    // threads per block of the boundary-node sweep (32, 64 or 128)
-  int list_thread;   // boundary-node sweep: 1 = a thread per node (IBM band), 0 = a warp per node
   void *zy_pre;      // Eq. 16: T [Q][fs] pre-collision populations at the boundary nodes, or null
   int bulk_mode;       // bulk sweep: 0 one node per thread, 1 vectors of nodes per thread,
                        // 2 vectors fed by bulk copies of row segments (each where nx and
@@ -136,6 +155,7 @@ enum SweepOp {
   OP_LOCAL_INIT,   // local read of a pre-collision state + collide + store
   OP_LOCAL_QUERY,  // local read of a pre-collision state, fields
   OP_REFILL,       // equilibrium refill of uncovered nodes (+ collide)
+  OP_IBM_GATHER,   // IBM, solids at rest: the spread force of every list node from the rows
   OP_BAND_VEL,     // IBM: unforced velocity at band nodes, zero the IBM force
   OP_FROM_DOUBLE,  // convert a full-f FP64 array (out_f) into deviations (dst)
   OP_FILL_EQ,      // fill dst with equilibrium deviations (g[] = u, omega = rho)
@@ -159,6 +179,30 @@ struct GroupArgs {
 // (lattice, collision, storage, vector shape and block size); false, with
 // nothing launched, otherwise.
 bool launch_bulk_group(const KArgs *as, int n, int lattice, int collision, int precision,
+                       cudaStream_t st);
+
+// Many steps of small lattices in one launch (run_impl.cuh): lattice k runs on
+// blocks block_start[k] .. block_start[k + 1] - 1.
+constexpr int kMaxRun = 8;
+struct RunLat {
+  KArgs a;         // src, dst and force_acc are set per step from the fields below
+  void *f[2];      // the two distribution arrays
+  int cur;         // index of f*(t)
+  int nsteps;
+  int slot0, hist_cap;
+  double *hist;    // force records; step s adds to slot slot0 + 1 + s (modulo hist_cap)
+  unsigned *bar;   // [2] barrier arrivals, blocks that left (zero between launches)
+  int iters;       // IBM forcing passes
+  int vec;         // vectors of nodes (nx and the direction stride allow)
+};
+template <int NL> struct RunArgs {
+  int n;
+  int block_start[kMaxRun + 1];
+  RunLat l[NL];
+};
+// One cooperative launch; every lattice has this lattice kind, collision
+// (CM_BGK or CM_MRT_Q) and precision, and all or none have IBM tables.
+cudaError_t launch_run(const RunArgs<kMaxRun> &g, int lattice, int collision, int precision,
                        cudaStream_t st);
 
 // Launch one operation for the given lattice/collision/precision.  grid
@@ -265,6 +309,19 @@ void launch_ibm_prepare(const IbmArgs &a, int precision, cudaStream_t st);
 void launch_ibm_fused(const IbmArgs &a, int precision, cudaStream_t st);
 void launch_ibm_interp(const IbmArgs &a, int precision, cudaStream_t st);
 void launch_ibm_spread(const IbmArgs &a, int precision, cudaStream_t st);
+
+// tables of solids at rest: without `col` the row lengths and their prefix
+// sum (row[0 .. n]), with it the entries
+void launch_tab_nodes(const IbmArgs &a, const int *list_node, int nlist, int *row, int *col,
+                      void *wt, int precision, cudaStream_t st);
+void launch_tab_markers(const IbmArgs &a, int *row, int *col, void *wt, int precision,
+                        cudaStream_t st);
+void launch_tab_desired(const IbmArgs &a, double *Ud, double *arm, cudaStream_t st);
+// one forcing pass over the markers through the tables (a.tab): pass 0
+// interpolates u~, later ones iterate; the last keeps F dV and reduces the
+// solids' force into a.force_acc
+void launch_marker_pass(const KArgs &a, int dim, int pass, bool last, int precision,
+                        cudaStream_t st);
 
 // chunked upload of FP64 populations (transfer.cu)
 struct UploadArgs {

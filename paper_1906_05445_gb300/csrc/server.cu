@@ -68,7 +68,19 @@ size_t estimate_bytes(const lbm_request &r) {
   const size_t ssz = d.precision == LBM_FP64 ? 8 : d.precision == LBM_FP32 ? 4 : 2;
   const size_t tsz = d.precision == LBM_FP64 ? 8 : 4;
   size_t b = 2 * q * n * ssz + 3 * n;
-  if (r.scheme.scheme == LBM_IBM_DIRECT) b += 6 * n * tsz;
+  if (r.scheme.scheme == LBM_IBM_DIRECT) {
+    b += 6 * n * tsz;
+    // the markers' tables: up to 64 stencil points and about 70 coupled
+    // markers per marker, a 4-byte index and a coefficient each
+    double markers = 0;
+    const double dens = r.scheme.ibm_marker_density > 0 ? r.scheme.ibm_marker_density : 1.0;
+    for (int k = 0; k < r.nsolids; k++) {
+      const double R = r.solids[k].radius + r.scheme.ibm_retraction;
+      markers += dens * (d.lattice == LBM_D2Q9 ? 6.3 * R
+                         : r.solids[k].kind == LBM_SPHERE ? 12.6 * R * R : 6.3 * R * d.nz);
+    }
+    b += (size_t)(markers * (160.0 + 140.0 * (4 + tsz)));
+  }
   return b + b / 10 + (1u << 20) + run_bytes(r);
 }
 

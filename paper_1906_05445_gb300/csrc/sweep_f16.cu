@@ -10,4 +10,8 @@ bool launch_bulk_group_f16(const KArgs *as, int n, int lattice, int collision,
                              cudaStream_t st) {
   return launch_group_precision<__half>(as, n, lattice, collision, st);
 }
+cudaError_t launch_run_f16(const RunArgs<kMaxRun> &g, int lattice, int collision,
+                         cudaStream_t st) {
+  return launch_run_precision<__half, float>(g, lattice, collision, st);
+}
 }  // namespace lbm

@@ -10,4 +10,8 @@ bool launch_bulk_group_f32(const KArgs *as, int n, int lattice, int collision,
                              cudaStream_t st) {
   return launch_group_precision<float>(as, n, lattice, collision, st);
 }
+cudaError_t launch_run_f32(const RunArgs<kMaxRun> &g, int lattice, int collision,
+                         cudaStream_t st) {
+  return launch_run_precision<float, float>(g, lattice, collision, st);
+}
 }  // namespace lbm

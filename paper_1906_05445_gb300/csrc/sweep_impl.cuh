@@ -74,8 +74,8 @@ __device__ __forceinline__ void node_force(const KArgs &a, long long n,
 }
 
 // Pull the Q populations of node (x, y, z) from src with periodic wrap.
-template <int LAT, typename S, typename T, int EVICT_FIRST = 0>
-__device__ __forceinline__ void gather_pull(const S *__restrict__ src,
+template <int LAT, typename S, typename T, int POL = LD_NC>
+__device__ __forceinline__ void gather_pull(const S *src,
                                             long long fs, int x, int y, int z,
                                             int nx, int ny, int nz, T isc,
                                             T (&f)[Lat<LAT>::Q]) {
@@ -96,10 +96,7 @@ __device__ __forceinline__ void gather_pull(const S *__restrict__ src,
     // source node x - e_i
     const int sx = L::ex(i) > 0 ? xm : (L::ex(i) < 0 ? xp : x);
     const long long row = r[1 - L::ez(i)][1 - L::ey(i)];
-    if constexpr (EVICT_FIRST)
-      f[i] = Store<S>::ld_stream(src + (long long)i * fs + row + sx, isc);
-    else
-      f[i] = Store<S>::ld(src + (long long)i * fs + row + sx, isc);
+    f[i] = Store<S>::template ld<POL>(src + (long long)i * fs + row + sx, isc);
   });
 }
 
@@ -127,6 +124,29 @@ __device__ __forceinline__ void scatter(S *__restrict__ dst, long long fs,
 }
 
 // ---------------------------------------------------------------- bulk sweep
+// Node n: pull from src, collide, store in dst; plain fluid nodes only.  Nodes
+// inside an IBM solid (FL_NOG) also run here, without the external force, and
+// so do nodes refilled this step (FL_NEW).
+// EAGER pulls before it looks at the flag (one memory latency instead of two:
+// small lattices); otherwise the other nodes pull nothing.
+template <int LAT, int CM, typename S, typename T, int POL, bool STREAM, bool EAGER = false>
+__device__ __forceinline__ void bulk_node_update(const KArgs &a, const S *src, S *dst, unsigned n) {
+  const uint8_t fl = a.flags[n];
+  if (!EAGER && (fl & (uint8_t)~(FL_NOG | FL_NEW))) return;
+  const unsigned yz = n / (unsigned)a.nx;
+  const int x = (int)(n - yz * (unsigned)a.nx);
+  const int z = (int)(yz / (unsigned)a.ny);
+  const int y = (int)(yz - (unsigned)z * (unsigned)a.ny);
+  const T isc = kisc<T>(a);
+  T f[Lat<LAT>::Q];
+  gather_pull<LAT, S, T, POL>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
+  if (EAGER && (fl & (uint8_t)~(FL_NOG | FL_NEW))) return;
+  const Coll<T> c = make_coll<LAT, T>(a);
+  const T gon = (fl & FL_NOG) ? (T)0 : (T)1;
+  collide<LAT, CM, S, T>(f, gon * kg<T>(a, 0), gon * kg<T>(a, 1), gon * kg<T>(a, 2), c);
+  scatter<LAT, S, T, STREAM>(dst, a.fs, n, isc, f);
+}
+
 // one thread per node, nodes in memory order (x fastest) so that every
 // direction's loads and stores of a warp are contiguous
 template <int LAT, int CM, typename S, typename T, int HINT>
@@ -134,21 +154,8 @@ __global__ void __launch_bounds__(512) k_bulk_sweep(const KArgs a) {
   // from the lattice's end every other step (see k_bulk_vec)
   const unsigned n = (a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
   if (n >= (unsigned)a.N) return;
-  // plain fluid nodes; nodes inside an IBM solid (FL_NOG) also run here,
-  // without the external force, and so do nodes refilled this step (FL_NEW)
-  const uint8_t fl = a.flags[n];
-  if (fl & (uint8_t)~(FL_NOG | FL_NEW)) return;
-  const unsigned yz = n / (unsigned)a.nx;
-  const int x = (int)(n - yz * (unsigned)a.nx);
-  const int z = (int)(yz / (unsigned)a.ny);
-  const int y = (int)(yz - (unsigned)z * (unsigned)a.ny);
-  const T isc = kisc<T>(a);
-  T f[Lat<LAT>::Q];
-  gather_pull<LAT, S, T, (HINT & 1)>((const S *)a.src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
-  const Coll<T> c = make_coll<LAT, T>(a);
-  const T gon = (fl & FL_NOG) ? (T)0 : (T)1;
-  collide<LAT, CM, S, T>(f, gon * kg<T>(a, 0), gon * kg<T>(a, 1), gon * kg<T>(a, 2), c);
-  scatter<LAT, S, T, (HINT & 2) != 0>((S *)a.dst, a.fs, n, isc, f);
+  bulk_node_update<LAT, CM, S, T, (HINT & 1) ? LD_ONCE : LD_NC, (HINT & 2) != 0>(
+      a, (const S *)a.src, (S *)a.dst, n);
 }
 
 }  // namespace lbm

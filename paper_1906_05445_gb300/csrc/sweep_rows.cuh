@@ -203,7 +203,7 @@ __device__ __forceinline__ void update_tile(const KArgs &a, const RowTiles &g, u
       if (lane == 0) mbar_arrive(empty);
     }
     const unsigned n0 = (r0 + (unsigned)t) * (unsigned)a.nx + (unsigned)(V * xv);
-    vec_collide_store<LAT, CM, S, W, PACKED>(a, v, fl, n0, true);
+    vec_collide_store<LAT, CM, S, W, PACKED>(a, (S *)a.dst, v, fl, n0, true);
   }
 }
 

@@ -28,18 +28,14 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 template <int W> struct Words {
   uint32_t w[W];
 };
-// ONCE: the line is not needed again before the array is overwritten (L2
-// evicts it first); see launch_bulk_vec_w.
-template <int W, bool ONCE = false> __device__ __forceinline__ Words<W> ld_words(const void *p) {
+template <int W, int POL = LD_NC> __device__ __forceinline__ Words<W> ld_words(const void *p) {
   Words<W> r;
   if constexpr (W == 4) {
-    const uint4 *q = reinterpret_cast<const uint4 *>(p);
-    const uint4 v = ONCE ? __ldcs(q) : __ldg(q);
+    const uint4 v = ld_pol<POL>(reinterpret_cast<const uint4 *>(p));
     r.w[0] = v.x, r.w[1] = v.y, r.w[2] = v.z, r.w[3] = v.w;
   } else {
     static_assert(W == 2, "8- or 16-byte vectors");
-    const uint2 *q = reinterpret_cast<const uint2 *>(p);
-    const uint2 v = ONCE ? __ldcs(q) : __ldg(q);
+    const uint2 v = ld_pol<POL>(reinterpret_cast<const uint2 *>(p));
     r.w[0] = v.x, r.w[1] = v.y;
   }
   return r;
@@ -63,8 +59,12 @@ template <> struct VecS<float> {
   static constexpr int kScaleLog2 = 0;  // stored values are the deviations
   // the end node fetched from outside the vector, as the word the shift
   // below expects
-  __device__ static uint32_t left_word(const float *p) { return __float_as_uint(__ldg(p)); }
-  __device__ static uint32_t right_word(const float *p) { return __float_as_uint(__ldg(p)); }
+  template <int POL> __device__ static uint32_t left_word(const float *p) {
+    return __float_as_uint(ld_pol<POL>(p));
+  }
+  template <int POL> __device__ static uint32_t right_word(const float *p) {
+    return __float_as_uint(ld_pol<POL>(p));
+  }
   // shift by one node: e_x = +1 pulls from x - 1, e_x = -1 from x + 1
   template <int W> __device__ static void shift_in_left(Words<W> &v, uint32_t l) {
 #pragma unroll
@@ -92,12 +92,12 @@ template <> struct VecS<float> {
 template <typename H> struct VecS16 {
   static constexpr int per_word = 2;
   static constexpr int kScaleLog2 = 0;
-  __device__ static uint32_t ld16(const H *p) {
-    return (uint32_t)__ldg(reinterpret_cast<const unsigned short *>(p));
+  template <int POL> __device__ static uint32_t ld16(const H *p) {
+    return (uint32_t)ld_pol<POL>(reinterpret_cast<const unsigned short *>(p));
   }
   // node x0 - 1 in the high half, node x0 + V in the low half
-  __device__ static uint32_t left_word(const H *p) { return ld16(p) << 16; }
-  __device__ static uint32_t right_word(const H *p) { return ld16(p); }
+  template <int POL> __device__ static uint32_t left_word(const H *p) { return ld16<POL>(p) << 16; }
+  template <int POL> __device__ static uint32_t right_word(const H *p) { return ld16<POL>(p); }
   template <int W> __device__ static void shift_in_left(Words<W> &v, uint32_t l) {
 #pragma unroll
     for (int k = W - 1; k > 0; k--) v.w[k] = join16(v.w[k - 1], v.w[k]);
@@ -166,7 +166,8 @@ template <int V> __device__ __forceinline__ void ld_flags(const uint8_t *p, uint
 // other nodes of a vector (boundary-list nodes, solid nodes) are computed but
 // not stored, since the boundary-node kernel writes them.
 template <int LAT, int CM, typename S, int W, bool PACKED>
-__device__ __forceinline__ void vec_collide_store(const KArgs &a, Words<W> (&v)[Lat<LAT>::Q],
+__device__ __forceinline__ void vec_collide_store(const KArgs &a, S *dst,
+                                                  Words<W> (&v)[Lat<LAT>::Q],
                                                   const uint32_t (&fl)[(W * VecS<S>::per_word + 3) / 4],
                                                   unsigned n0, bool valid) {
   using L = Lat<LAT>;
@@ -201,8 +202,9 @@ __device__ __forceinline__ void vec_collide_store(const KArgs &a, Words<W> (&v)[
     const float g0 = (flag(2 * p) & FL_NOG) ? 0.f : 1.f;
     const float g1 = (flag(2 * p + 1) & FL_NOG) ? 0.f : 1.f;
     if constexpr (PACKED) {
-      collide_two_rate<LAT, CM, SL, (sizeof(S) > 2), float2, float>(f, make_float2(g0 * gx, g1 * gx), make_float2(g0 * gy, g1 * gy),
-                              make_float2(g0 * gz, g1 * gz), c);
+      collide_two_rate<LAT, CM, SL, even_first<S>(), float2, float>(
+          f, make_float2(g0 * gx, g1 * gx), make_float2(g0 * gy, g1 * gy),
+          make_float2(g0 * gz, g1 * gz), c);
     } else {
       float fa[Q], fb[Q];
       static_for<Q>([&](auto ic) {
@@ -223,7 +225,6 @@ __device__ __forceinline__ void vec_collide_store(const KArgs &a, Words<W> (&v)[
       else VS::put(v[i], p, f[i], sc);
     });
   });
-  S *dst = (S *)a.dst;
   if (all) {
     static_for<Q>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
@@ -244,8 +245,9 @@ __device__ __forceinline__ void vec_collide_store(const KArgs &a, Words<W> (&v)[
 // Thread t updates the vector of nodes [V t, V t + V), pulling the shifted
 // rows straight from global memory.  Every lane of the warp calls this
 // (threads past the end with t >= nt), for the shuffles.
-template <int LAT, int CM, typename S, int W, bool PACKED, bool ONCE = false>
-__device__ __forceinline__ void bulk_vec_update(const KArgs &a, unsigned t, unsigned nt) {
+template <int LAT, int CM, typename S, int W, bool PACKED, int POL = LD_NC>
+__device__ __forceinline__ void bulk_vec_update(const KArgs &a, const S *src, S *dst, unsigned t,
+                                                unsigned nt) {
   using L = Lat<LAT>;
   using VS = VecS<S>;
   constexpr int Q = L::Q, V = W * VS::per_word;
@@ -274,18 +276,17 @@ __device__ __forceinline__ void bulk_vec_update(const KArgs &a, unsigned t, unsi
   const bool lnb = lane != 0 && x0 != 0;
   const bool rnb = lane != 31 && x0 + V != nx;
   const int xl = x0 == 0 ? nx - 1 : x0 - 1, xr = x0 + V == nx ? 0 : x0 + V;
-  const S *src = (const S *)a.src;
   Words<W> v[Q];
   uint32_t edge[Q];
   static_for<Q>([&](auto ic) {
     constexpr int i = decltype(ic)::value;
     const S *row = src + (long long)i * a.fs + r[1 - L::ez(i)][1 - L::ey(i)];
-    v[i] = ld_words<W, ONCE>(row + x0);
+    v[i] = ld_words<W, POL>(row + x0);
     edge[i] = 0u;
     if constexpr (L::ex(i) == 1) {
-      if (!lnb) edge[i] = VS::left_word(row + xl);
+      if (!lnb) edge[i] = VS::template left_word<POL>(row + xl);
     } else if constexpr (L::ex(i) == -1) {
-      if (!rnb) edge[i] = VS::right_word(row + xr);
+      if (!rnb) edge[i] = VS::template right_word<POL>(row + xr);
     }
   });
   static_for<Q>([&](auto ic) {
@@ -298,9 +299,8 @@ __device__ __forceinline__ void bulk_vec_update(const KArgs &a, unsigned t, unsi
       VS::shift_in_right(v[i], rnb ? sw : edge[i]);
     }
   });
-  vec_collide_store<LAT, CM, S, W, PACKED>(a, v, fl, n0, valid);
+  vec_collide_store<LAT, CM, S, W, PACKED>(a, dst, v, fl, n0, valid);
 }
-
 
 // Registers a thread of the 2-word kernels: FP32 80 (6 blocks of 128 per SM),
 // BF16 112, FP16 128.  Measured on 128^3 / 160^3 / 192^3 lattices without
@@ -322,13 +322,14 @@ template <typename S, int W> constexpr int vec_regs() {
 // a step then starts on the nodes that the previous one wrote last, which L2
 // still holds, instead of on those it has already evicted.  128^3 without
 // solids, FP32: 50.9 -> 48.0 us per step (and 47.2 with evict-first reads,
-// ONCE); 112^3 36.1 -> 32.6 (30.9); FP16 128^3 28.8 -> 26.7 (24.7).
-template <int LAT, int CM, typename S, int W, bool PACKED, bool ONCE>
+// LD_ONCE); 112^3 36.1 -> 32.6 (30.9); FP16 128^3 28.8 -> 26.7 (24.7).
+template <int LAT, int CM, typename S, int W, bool PACKED, int POL>
 __global__ void __maxnreg__((vec_regs<S, W>()))
     k_bulk_vec(const KArgs a) {
   constexpr int V = W * VecS<S>::per_word;
   const unsigned b = a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
-  bulk_vec_update<LAT, CM, S, W, PACKED, ONCE>(a, b * blockDim.x + threadIdx.x, (unsigned)a.N / V);
+  bulk_vec_update<LAT, CM, S, W, PACKED, POL>(a, (const S *)a.src, (S *)a.dst,
+                                              b * blockDim.x + threadIdx.x, (unsigned)a.N / V);
 }
 
 // The same update for several lattices in one grid: block b belongs to the
@@ -347,7 +348,7 @@ __global__ void __maxnreg__((vec_regs<S, W>()))
     constexpr int k = decltype(kc)::value;
     if (k < g.n && b >= g.block_start[k] && b < g.block_start[k + 1])
       bulk_vec_update<LAT, CM, S, W, PACKED>(
-          g.a[k],
+          g.a[k], (const S *)g.a[k].src, (S *)g.a[k].dst,
           (unsigned)(g.a[k].rev ? g.block_start[k + 1] - 1 - b : b - g.block_start[k]) * blockDim.x +
               threadIdx.x,
           (unsigned)g.a[k].N / V);
