@@ -111,6 +111,9 @@ struct lbm_ctx {
   // pre-pass run there, concurrently with the bulk sweep on `st`
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // the face kernel's stream (made with the first non-periodic domain)
+  cudaStream_t fst = nullptr;
+  cudaEvent_t ev_face = nullptr;
   // bumped by every call that changes what a step's launches read (their
   // arguments, buffers or state): a batch's captured graph is then stale
   unsigned long long gen = 0;
@@ -1407,8 +1410,15 @@ lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
     Timed tm(ctx, TK_LIST, ctx->list_count >= 0 ? ctx->list_count : 0, ctx->aux);
     sweep(ctx, OP_LIST_SWEEP, a, ctx->aux);
   }
-  // nodes next to non-periodic domain faces
-  if (ctx->nface) sweep(ctx, OP_FACE_SWEEP, a, ctx->aux);
+  // nodes next to non-periodic domain faces: after the band nodes' forces under
+  // IBM, beside the boundary nodes otherwise (their own stream)
+  if (ctx->nface && ibm) {
+    sweep(ctx, OP_FACE_SWEEP, a, ctx->aux);
+  } else if (ctx->nface) {
+    CK(cudaStreamWaitEvent(ctx->fst, ctx->ev_fork, 0));
+    sweep(ctx, OP_FACE_SWEEP, a, ctx->fst);
+    CK(cudaEventRecord(ctx->ev_face, ctx->fst));
+  }
   ss.a = a;
   ss.ibm = ibm;
   ss.moving = moving;
@@ -1429,6 +1439,7 @@ lbm_status step_end(lbm_ctx *ctx, const StepState &ss) {
   // join
   CK(cudaEventRecord(ctx->ev_join, ctx->aux));
   CK(cudaStreamWaitEvent(ctx->st, ctx->ev_join, 0));
+  if (ctx->nface && !ibm) CK(cudaStreamWaitEvent(ctx->st, ctx->ev_face, 0));
   ctx->cur = nxt;
   ctx->prev_local = false;
   if (!ibm && moving && !free_)
@@ -1658,6 +1669,9 @@ void run_query(lbm_ctx *ctx, KArgs a) {
   }
 }
 
+// bytes of a field per piece copied while the rest is computed
+constexpr size_t kQueryPiece = 3 << 20;
+
 enum QueryKind { Q_RHO, Q_U, Q_S, Q_STRESS, Q_F, Q_EPS };
 
 // The field into host memory: enqueued on the context's stream, then (wait)
@@ -1680,8 +1694,42 @@ lbm_status query(lbm_ctx *ctx, QueryKind kind, double *host, size_t n, bool wait
   case Q_EPS: a.out_eps = ctx->qbuf; break;
   case Q_F: a.out_f = ctx->qbuf; break;
   }
-  run_query(ctx, a);
-  CK(cudaMemcpyAsync(host, ctx->qbuf, need * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
+  // Large fields in pieces of nodes, each copied on the copy stream while the
+  // next is computed (the copies of a 96^3 FP64 strain rate take 212 us, its
+  // FP64 arithmetic about 150).  The boundary and face nodes, anywhere in the
+  // lattice, are written before or with the first piece.
+  // Only into page-locked memory: copies into pageable memory hold the host.
+  int pieces = ctx->prev_local ? 1 : (int)std::min<size_t>(6, need * sizeof(double) / kQueryPiece);
+  if (pieces > 1) {
+    cudaPointerAttributes at{};
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) cudaGetLastError();
+    CK(cudaStreamIsCapturing(ctx->st, &cap));
+    if (at.type != cudaMemoryTypeHost || cap != cudaStreamCaptureStatusNone) pieces = 1;
+  }
+  if (pieces < 2) {
+    run_query(ctx, a);
+    CK(cudaMemcpyAsync(host, ctx->qbuf, need * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
+  } else {
+    TRY(ensure_copy_stream(ctx));
+    a.src = ctx->f[1 - ctx->cur];
+    a.local_gather = 0;
+    if (ctx->nface) sweep(ctx, OP_FACE_QUERY, a);
+    const size_t pitch = (size_t)ctx->N * sizeof(double);
+    for (int k = 0; k < pieces; k++) {
+      a.query_n0 = ctx->N * k / pieces;
+      a.query_n1 = ctx->N * (k + 1) / pieces;
+      sweep(ctx, OP_QUERY, a);
+      CK(cudaEventRecord(ctx->ev_rec, ctx->st));
+      CK(cudaStreamWaitEvent(ctx->cst, ctx->ev_rec, 0));
+      CK(cudaMemcpy2DAsync(host + a.query_n0, pitch, ctx->qbuf + a.query_n0, pitch,
+                           (size_t)(a.query_n1 - a.query_n0) * sizeof(double), comps,
+                           cudaMemcpyDeviceToHost, ctx->cst));
+    }
+    // later work on the stream (a query into the same staging) follows the copies
+    CK(cudaEventRecord(ctx->ev_cst, ctx->cst));
+    CK(cudaStreamWaitEvent(ctx->st, ctx->ev_cst, 0));
+  }
   if (wait) CK(cudaStreamSynchronize(ctx->st));
   CK(cudaGetLastError());
   return LBM_OK;
@@ -1898,6 +1946,11 @@ void lbm_destroy(lbm_ctx *ctx) {
     cudaStreamSynchronize(ctx->gst);
     cudaStreamDestroy(ctx->gst);
   }
+  if (ctx->fst) {
+    cudaStreamSynchronize(ctx->fst);
+    cudaStreamDestroy(ctx->fst);
+  }
+  if (ctx->ev_face) cudaEventDestroy(ctx->ev_face);
   if (ctx->ev_geom) cudaEventDestroy(ctx->ev_geom);
   if (ctx->ev_gfree) cudaEventDestroy(ctx->ev_gfree);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
@@ -2291,6 +2344,12 @@ lbm_status lbm_set_domain(lbm_ctx *ctx, const lbm_domain_desc *dom) {
   ctx->dom = lbm_domain_desc{};
   ctx->geom_dirty = true;
   if (!nodes.empty()) {
+    if (!ctx->fst) {
+      int lo = 0, hi = 0;
+      cudaDeviceGetStreamPriorityRange(&lo, &hi);
+      CK(cudaStreamCreateWithPriority(&ctx->fst, cudaStreamNonBlocking, hi));
+    }
+    if (!ctx->ev_face) CK(cudaEventCreateWithFlags(&ctx->ev_face, cudaEventDisableTiming));
     TRY(dalloc(ctx, (void **)&ctx->face_node, nodes.size() * sizeof(int)));
     CK(cudaMemcpy(ctx->face_node, nodes.data(), nodes.size() * sizeof(int), cudaMemcpyHostToDevice));
     ctx->nface = (int)nodes.size();

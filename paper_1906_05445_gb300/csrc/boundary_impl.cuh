@@ -223,7 +223,8 @@ __device__ __forceinline__ void list_query_node(const KArgs &a, int t) {
 // (as a launch of their own they took 46 us after a 96^3 FP64 lattice's plain
 // nodes).  U32: density and velocity of FP32 and 16-bit storage.
 template <int LAT, typename S, typename LT, bool U32>
-__global__ void __launch_bounds__(128) k_query(const KArgs a, int list_blocks) {
+__global__ void __launch_bounds__(128) k_query(const KArgs a, int list_blocks, long long n0,
+                                               long long n1) {
   const int b = (int)blockIdx.x - list_blocks;
   if (b < 0) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -232,8 +233,8 @@ __global__ void __launch_bounds__(128) k_query(const KArgs a, int list_blocks) {
     if (t < cnt) list_query_node<LAT, S, LT>(a, t);
     return;
   }
-  const long long n = (long long)b * blockDim.x + threadIdx.x;
-  if (n >= a.N) return;
+  const long long n = n0 + (long long)b * blockDim.x + threadIdx.x;
+  if (n >= n1) return;
   const uint8_t fl = a.flags[n];
   if (fl & (uint8_t)~(FL_NOG | FL_NEW)) return;
   int x, y, z;
@@ -672,12 +673,86 @@ __global__ void __launch_bounds__(128) k_refill(const KArgs a) {
   scatter<LAT, S, T>((S *)a.dst, a.fs, n, isc, f);
 }
 
+// Links through the domain faces: the rules stand at k_face.
+template <typename T> __device__ __forceinline__ T face_u(const KArgs &a, int k, int c) {
+  if constexpr (is_f32<T>()) return a.u_face_f[k][c];
+  else return (T)a.u_face[k][c];
+}
+
+// The neighbourhood of a node: wrapped coordinates either side of it, and per
+// axis the type of the face that a link leaves the domain through when it
+// comes from below (e_a = +1) or above (e_a = -1); 0 (periodic): none there.
+struct FaceNode {
+  int x[3], y[3], z[3];  // at - 1, at, at + 1
+  int lo[3], hi[3];
+};
+__device__ __forceinline__ FaceNode face_node(const KArgs &a, int x, int y, int z) {
+  FaceNode f;
+  f.x[0] = x == 0 ? a.nx - 1 : x - 1;
+  f.x[1] = x;
+  f.x[2] = x == a.nx - 1 ? 0 : x + 1;
+  f.y[0] = y == 0 ? a.ny - 1 : y - 1;
+  f.y[1] = y;
+  f.y[2] = y == a.ny - 1 ? 0 : y + 1;
+  f.z[0] = z == 0 ? a.nz - 1 : z - 1;
+  f.z[1] = z;
+  f.z[2] = z == a.nz - 1 ? 0 : z + 1;
+  f.lo[0] = x == 0 ? a.face[0] : 0;
+  f.hi[0] = x == a.nx - 1 ? a.face[1] : 0;
+  f.lo[1] = y == 0 ? a.face[2] : 0;
+  f.hi[1] = y == a.ny - 1 ? a.face[3] : 0;
+  f.lo[2] = z == 0 ? a.face[4] : 0;
+  f.hi[2] = z == a.nz - 1 ? a.face[5] : 0;
+  return f;
+}
+
+// direction i with its components along the axes of `axes` (bits) reversed
+template <int LAT> __host__ __device__ constexpr int reflect(int i, int axes) {
+  for (int k = 0; k < Lat<LAT>::Q; k++) {
+    bool same = true;
+    for (int c = 0; c < 3; c++)
+      same = same && ecomp<LAT>(c, k) == (((axes >> c) & 1) ? -ecomp<LAT>(c, i) : ecomp<LAT>(c, i));
+    if (same) return k;
+  }
+  return 0;
+}
+
+// Type of the face that link I of the node crosses along axis C (0: none).
+template <int LAT, int I, int C>
+__device__ __forceinline__ int crossed(const FaceNode &f) {
+  constexpr int e = ecomp<LAT>(C, I);
+  return e == 1 ? f.lo[C] : (e == -1 ? f.hi[C] : 0);
+}
+
+// f_I(x, t+1) of a node: plain pull, or through velocity / stress-free faces.
+// The direction is a compile-time constant, so that which axes a link may
+// cross and the direction it is reflected from are too (a run-time search per
+// direction made this kernel a fifth of the open box's step).
+template <int LAT, int I, typename S, typename T>
+__device__ __forceinline__ T face_pull(const KArgs &a, const S *src, const FaceNode &f, T isc) {
+  using L = Lat<LAT>;
+  constexpr int ex = L::ex(I), ey = L::ey(I), ez = L::ez(I);
+  const int cx = crossed<LAT, I, 0>(f), cy = crossed<LAT, I, 1>(f), cz = crossed<LAT, I, 2>(f);
+  auto at = [&](int j, int x, int y, int z) {
+    return Store<S>::ld(src + (long long)j * a.fs + x + (long long)a.nx * (y + (long long)a.ny * z), isc);
+  };
+  if (I == 0 || !(cx | cy | cz)) return at(I, f.x[1 - ex], f.y[1 - ey], f.z[1 - ez]);
+  const int vf = cx == LBM_FACE_VELOCITY ? (ex == 1 ? 0 : 1)
+               : cy == LBM_FACE_VELOCITY ? (ey == 1 ? 2 : 3)
+               : cz == LBM_FACE_VELOCITY ? (ez == 1 ? 4 : 5) : -1;
+  if (vf >= 0) {
+    const T eu = (T)ex * face_u<T>(a, vf, 0) + (T)ey * face_u<T>(a, vf, 1) + (T)ez * face_u<T>(a, vf, 2);
+    return at(L::opp(I), f.x[1], f.y[1], f.z[1]) + (T)(6.0 * L::w(I)) * eu;
+  }
+  const int j = (cx ? 1 : 0) + (cy ? 2 : 0) + (cz ? 4 : 0);
+  constexpr int r1 = reflect<LAT>(I, 1), r2 = reflect<LAT>(I, 2), r4 = reflect<LAT>(I, 4);
+  constexpr int r3 = reflect<LAT>(I, 3), r5 = reflect<LAT>(I, 5), r6 = reflect<LAT>(I, 6);
+  const int rd = j == 1 ? r1 : j == 2 ? r2 : j == 4 ? r4 : j == 3 ? r3 : j == 5 ? r5 : r6;
+  return at(rd, cx ? f.x[1] : f.x[1 - ex], cy ? f.y[1] : f.y[1 - ey], cz ? f.z[1] : f.z[1 - ez]);
+}
+
 // IBM: unforced velocity u~ = (sum f e + g/2)/rho0 at band nodes (the
 // external half force only, no IBM half force) and zero the IBM force there.
-template <int LAT, typename S, typename T>
-__device__ __forceinline__ T face_pull(const KArgs &a, const S *__restrict__ src, int x, int y,
-                                       int z, int i, T isc);
-
 template <int LAT, typename S, typename T, int POL>
 __device__ __forceinline__ void band_velocity(const KArgs &a, const S *src, int t) {
   using L = Lat<LAT>;
@@ -690,9 +765,13 @@ __device__ __forceinline__ void band_velocity(const KArgs &a, const S *src, int 
   const T isc = kisc<T>(a);
   if (a.local_gather)
     gather_local<LAT, S, T>(src, a.fs, n, isc, f);
-  else if (fl & FL_FACE)  // next to a velocity or stress-free domain face
-    for (int i = 0; i < L::Q; i++) f[i] = face_pull<LAT, S, T>(a, src, x, y, z, i, isc);
-  else
+  else if (fl & FL_FACE) {  // next to a velocity or stress-free domain face
+    const FaceNode fn = face_node(a, x, y, z);
+    static_for<L::Q>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      f[i] = face_pull<LAT, i, S, T>(a, src, fn, isc);
+    });
+  } else
     gather_pull<LAT, S, T, POL>(src, a.fs, x, y, z, a.nx, a.ny, a.nz, isc, f);
   T j[3] = {0, 0, 0};
   static_for<L::Q>([&](auto ic) {
@@ -783,78 +862,6 @@ __global__ void __launch_bounds__(128) k_zy_seed(const KArgs a) {
 // A velocity face decides a link that crosses two faces, then an outflow
 // face, then free slip.
 
-// bit 2a: the low face of axis a is crossed, bit 2a + 1: the high face
-template <int LAT>
-__device__ __forceinline__ int face_cross(const KArgs &a, int x, int y, int z, int i) {
-  using L = Lat<LAT>;
-  const int sx = x - L::ex(i), sy = y - L::ey(i), sz = z - L::ez(i);
-  int m = 0;
-  if (sx < 0 && a.face[0]) m |= 1;
-  if (sx >= a.nx && a.face[1]) m |= 2;
-  if (sy < 0 && a.face[2]) m |= 4;
-  if (sy >= a.ny && a.face[3]) m |= 8;
-  if (L::D == 3) {
-    if (sz < 0 && a.face[4]) m |= 16;
-    if (sz >= a.nz && a.face[5]) m |= 32;
-  }
-  return m;
-}
-
-__device__ __forceinline__ int face_of_type(const KArgs &a, int m, int type) {
-  for (int k = 0; k < 6; k++)
-    if (((m >> k) & 1) && a.face[k] == type) return k;
-  return -1;
-}
-
-template <typename T> __device__ __forceinline__ T face_u(const KArgs &a, int k, int c) {
-  if constexpr (is_f32<T>()) return a.u_face_f[k][c];
-  else return (T)a.u_face[k][c];
-}
-
-// f_i(x, t+1) of a link that leaves through velocity / stress-free faces
-template <int LAT, typename S, typename T>
-__device__ __forceinline__ T face_wall(const KArgs &a, const S *__restrict__ src, int x, int y,
-                                       int z, int i, int m, T isc) {
-  using L = Lat<LAT>;
-  const long long fs = a.fs;
-  const int vf = face_of_type(a, m, LBM_FACE_VELOCITY);
-  if (vf >= 0) {
-    const long long n = x + (long long)a.nx * (y + (long long)a.ny * z);
-    const T eu = (T)L::ex(i) * face_u<T>(a, vf, 0) + (T)L::ey(i) * face_u<T>(a, vf, 1) +
-                 (T)L::ez(i) * face_u<T>(a, vf, 2);
-    return Store<S>::ld(src + (long long)L::opp(i) * fs + n, isc) + (T)(6.0 * L::w(i)) * eu;
-  }
-  int r[3] = {L::ex(i), L::ey(i), L::ez(i)};
-  int p[3] = {x - r[0], y - r[1], z - r[2]};
-  const int at[3] = {x, y, z};
-#pragma unroll
-  for (int c = 0; c < 3; c++)
-    if ((m >> (2 * c)) & 3) {
-      r[c] = -r[c];
-      p[c] = at[c];
-    }
-  int j = 0;
-#pragma unroll
-  for (int k = 1; k < L::Q; k++)
-    if (L::ex(k) == r[0] && L::ey(k) == r[1] && L::ez(k) == r[2]) j = k;
-  const long long ns = wrap(p[0], a.nx) +
-                       (long long)a.nx * (wrap(p[1], a.ny) + (long long)a.ny * wrap(p[2], a.nz));
-  return Store<S>::ld(src + (long long)j * fs + ns, isc);
-}
-
-// f_i(x, t+1) of a node: plain pull, or through velocity / stress-free faces
-template <int LAT, typename S, typename T>
-__device__ __forceinline__ T face_pull(const KArgs &a, const S *__restrict__ src, int x, int y,
-                                       int z, int i, T isc) {
-  using L = Lat<LAT>;
-  const int m = face_cross<LAT>(a, x, y, z, i);
-  if (m) return face_wall<LAT, S, T>(a, src, x, y, z, i, m, isc);
-  const long long ns = wrap(x - L::ex(i), a.nx) +
-                       (long long)a.nx * (wrap(y - L::ey(i), a.ny) +
-                                          (long long)a.ny * wrap(z - L::ez(i), a.nz));
-  return Store<S>::ld(src + (long long)i * a.fs + ns, isc);
-}
-
 // index of a node of the outflow face in the outlet arrays
 __device__ __forceinline__ int outlet_index(const KArgs &a, int x, int y, int z) {
   const int ax = a.out_face >> 1;
@@ -894,31 +901,30 @@ __global__ void __launch_bounds__(128) k_face(const KArgs a) {
     if (!out) return;
     gather_local<LAT, S, T>(src, a.fs, n, isc, f);
   } else {
-    const int ax = a.out_face >> 1, sg = (a.out_face & 1) ? 1 : -1;
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      const int m = face_cross<LAT>(a, x, y, z, i);
-      if (m == 0) {
-        const long long ns = wrap(x - L::ex(i), a.nx) +
-                             (long long)a.nx * (wrap(y - L::ey(i), a.ny) +
-                                                (long long)a.ny * wrap(z - L::ez(i), a.nz));
-        f[i] = Store<S>::ld(src + (long long)i * a.fs + ns, isc);
-      } else if (face_of_type(a, m, LBM_FACE_VELOCITY) < 0 &&
-                 face_of_type(a, m, LBM_FACE_CONVECTIVE) >= 0) {
-        if (MODE == 1) {
-          f[i] = (T)keep[(long long)i * A + oi];  // f_i(x, t), kept by the last step
-        } else {
-          const int xi = x - (ax == 0 ? sg : 0), yi = y - (ax == 1 ? sg : 0),
-                    zi = z - (ax == 2 ? sg : 0);
-          const T vin = face_pull<LAT, S, T>(a, src, xi, yi, zi, i, isc);
-          T U = (T)keep[(long long)Q * A + oi];
-          if (U < (T)0) U = (T)0;
-          f[i] = ((T)keep[(long long)i * A + oi] + U * vin) / ((T)1 + U);
+    const FaceNode fn = face_node(a, x, y, z);
+    static_for<Q>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      if (out) {
+        // the outflow rule, on links that cross it and no velocity face
+        const int cx = crossed<LAT, i, 0>(fn), cy = crossed<LAT, i, 1>(fn), cz = crossed<LAT, i, 2>(fn);
+        const bool vel = cx == LBM_FACE_VELOCITY || cy == LBM_FACE_VELOCITY || cz == LBM_FACE_VELOCITY;
+        if (!vel && (cx == LBM_FACE_CONVECTIVE || cy == LBM_FACE_CONVECTIVE || cz == LBM_FACE_CONVECTIVE)) {
+          if (MODE == 1) {
+            f[i] = (T)keep[(long long)i * A + oi];  // f_i(x, t), kept by the last step
+          } else {
+            const int ax = a.out_face >> 1, sg = (a.out_face & 1) ? 1 : -1;
+            const FaceNode in = face_node(a, x - (ax == 0 ? sg : 0), y - (ax == 1 ? sg : 0),
+                                          z - (ax == 2 ? sg : 0));
+            const T vin = face_pull<LAT, i, S, T>(a, src, in, isc);
+            T U = (T)keep[(long long)Q * A + oi];
+            if (U < (T)0) U = (T)0;
+            f[i] = ((T)keep[(long long)i * A + oi] + U * vin) / ((T)1 + U);
+          }
+          return;
         }
-      } else {
-        f[i] = face_wall<LAT, S, T>(a, src, x, y, z, i, m, isc);
       }
-    }
+      f[i] = face_pull<LAT, i, S, T>(a, src, fn, isc);
+    });
   }
   if (MODE != 1 && out) {
     // this step's pre-collision populations and outward velocity, read by
@@ -1187,15 +1193,17 @@ void launch_one(SweepOp op, const KArgs &a, cudaStream_t st) {
     }
     break;
   case OP_QUERY: {
-    const int lb = a.list_cap > 0 ? div_up(a.list_cap, 128) : 0;
-    const int grid = lb + div_up(a.N, 128);
+    // plain nodes query_n0 .. query_n1 - 1; the boundary nodes with the first
+    const long long n1 = a.query_n1 > 0 ? a.query_n1 : a.N;
+    const int lb = a.list_cap > 0 && a.query_n0 == 0 ? div_up(a.list_cap, 128) : 0;
+    const int grid = lb + div_up(n1 - a.query_n0, 128);
     if constexpr (std::is_same<T, float>::value) {
       if (!a.out_S && !a.out_stress && !a.out_eps && !a.out_f) {
-        k_query<LAT, S, T, true><<<grid, 128, 0, st>>>(a, lb);
+        k_query<LAT, S, T, true><<<grid, 128, 0, st>>>(a, lb, a.query_n0, n1);
         break;
       }
     }
-    k_query<LAT, S, T, false><<<grid, 128, 0, st>>>(a, lb);
+    k_query<LAT, S, T, false><<<grid, 128, 0, st>>>(a, lb, a.query_n0, n1);
     break;
   }
   case OP_LIST_SWEEP:
