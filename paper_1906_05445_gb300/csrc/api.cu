@@ -1473,7 +1473,7 @@ bool run_ok(const lbm_ctx *ctx) {
   const bool ibm = ctx->scheme.scheme == LBM_IBM_DIRECT && ctx->nmark > 0;
   return ctx->run_on && ctx->sms > 0 && run_small(ctx) && !any_moving(ctx) && !ctx->nface &&
          ctx->timing == 0 && ctx->coll_mode != CM_MRT && ctx->bulk_mode == 1 &&
-         (ctx->bulk_vec_words == 0 || ctx->bulk_vec_words == 2) && ctx->bulk_vec_packed != 0 &&
+         (ctx->bulk_vec_words == 0 || ctx->bulk_vec_words == 2) && ctx->bulk_vec_packed < 0 &&
          ctx->cache_hints == 0 && (!ibm || ctx->tab.nmark > 0);
 }
 
@@ -1486,7 +1486,7 @@ bool run_vec(const lbm_ctx *ctx) {
 
 // Largest lattice (populations, nodes x Q) whose steps k_run takes, from us
 // per step of k_run against the step's own launches (3D spheres of R = 3/32
-// of the edge, 2D Couette flows):
+// of the edge, 2D Couette flows; FP32 with packed pairs):
 //   FP32 bounce-back  64^3 8.2 / 14.2, 80^3 12.4 / 14.3, 88^3 18.7 / 16.1;
 //                     301^2 5.2 / 11.3, 512^2 6.3 / 11.9
 //   FP32 IBM, 1 pass  64^3 14.8 / 24.1, 72^3 20.7 / 24.0, 80^3 23.8 / 24.2

@@ -726,29 +726,33 @@ __device__ __forceinline__ int crossed(const FaceNode &f) {
 
 // f_I(x, t+1) of a node: plain pull, or through velocity / stress-free faces.
 // The direction is a compile-time constant, so that which axes a link may
-// cross and the direction it is reflected from are too (a run-time search per
-// direction made this kernel a fifth of the open box's step).
+// cross and the direction it is reflected from are too, and the source is
+// selected without branches: one load per direction, all of a node's loads in
+// flight together (48 M node open box: 5186 us per four steps with a run-time
+// search and branches per direction, 5104 now).
 template <int LAT, int I, typename S, typename T>
 __device__ __forceinline__ T face_pull(const KArgs &a, const S *src, const FaceNode &f, T isc) {
   using L = Lat<LAT>;
   constexpr int ex = L::ex(I), ey = L::ey(I), ez = L::ez(I);
   const int cx = crossed<LAT, I, 0>(f), cy = crossed<LAT, I, 1>(f), cz = crossed<LAT, I, 2>(f);
-  auto at = [&](int j, int x, int y, int z) {
-    return Store<S>::ld(src + (long long)j * a.fs + x + (long long)a.nx * (y + (long long)a.ny * z), isc);
-  };
-  if (I == 0 || !(cx | cy | cz)) return at(I, f.x[1 - ex], f.y[1 - ey], f.z[1 - ez]);
   const int vf = cx == LBM_FACE_VELOCITY ? (ex == 1 ? 0 : 1)
                : cy == LBM_FACE_VELOCITY ? (ey == 1 ? 2 : 3)
                : cz == LBM_FACE_VELOCITY ? (ez == 1 ? 4 : 5) : -1;
-  if (vf >= 0) {
-    const T eu = (T)ex * face_u<T>(a, vf, 0) + (T)ey * face_u<T>(a, vf, 1) + (T)ez * face_u<T>(a, vf, 2);
-    return at(L::opp(I), f.x[1], f.y[1], f.z[1]) + (T)(6.0 * L::w(I)) * eu;
-  }
-  const int j = (cx ? 1 : 0) + (cy ? 2 : 0) + (cz ? 4 : 0);
+  const bool wall = vf >= 0;
   constexpr int r1 = reflect<LAT>(I, 1), r2 = reflect<LAT>(I, 2), r4 = reflect<LAT>(I, 4);
   constexpr int r3 = reflect<LAT>(I, 3), r5 = reflect<LAT>(I, 5), r6 = reflect<LAT>(I, 6);
-  const int rd = j == 1 ? r1 : j == 2 ? r2 : j == 4 ? r4 : j == 3 ? r3 : j == 5 ? r5 : r6;
-  return at(rd, cx ? f.x[1] : f.x[1 - ex], cy ? f.y[1] : f.y[1 - ey], cz ? f.z[1] : f.z[1 - ez]);
+  const int j = (cx ? 1 : 0) + (cy ? 2 : 0) + (cz ? 4 : 0);
+  const int rd = wall ? L::opp(I)
+                      : j == 0 ? I : j == 1 ? r1 : j == 2 ? r2 : j == 4 ? r4 : j == 3 ? r3 : j == 5 ? r5 : r6;
+  // a crossed axis keeps the node's own coordinate; a wall reflects at the node
+  const int sx = wall || cx ? f.x[1] : f.x[1 - ex];
+  const int sy = wall || cy ? f.y[1] : f.y[1 - ey];
+  const int sz = wall || cz ? f.z[1] : f.z[1 - ez];
+  const unsigned n = (unsigned)sx + (unsigned)a.nx * ((unsigned)sy + (unsigned)a.ny * (unsigned)sz);
+  const T v = Store<S>::ld(src + (long long)rd * a.fs + n, isc);
+  T eu = 0;
+  if (wall) eu = (T)ex * face_u<T>(a, vf, 0) + (T)ey * face_u<T>(a, vf, 1) + (T)ez * face_u<T>(a, vf, 2);
+  return wall ? v + (T)(6.0 * L::w(I)) * eu : v;
 }
 
 // IBM: unforced velocity u~ = (sum f e + g/2)/rho0 at band nodes (the
@@ -904,27 +908,29 @@ __global__ void __launch_bounds__(128) k_face(const KArgs a) {
     const FaceNode fn = face_node(a, x, y, z);
     static_for<Q>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
-      if (out) {
-        // the outflow rule, on links that cross it and no velocity face
-        const int cx = crossed<LAT, i, 0>(fn), cy = crossed<LAT, i, 1>(fn), cz = crossed<LAT, i, 2>(fn);
-        const bool vel = cx == LBM_FACE_VELOCITY || cy == LBM_FACE_VELOCITY || cz == LBM_FACE_VELOCITY;
-        if (!vel && (cx == LBM_FACE_CONVECTIVE || cy == LBM_FACE_CONVECTIVE || cz == LBM_FACE_CONVECTIVE)) {
-          if (MODE == 1) {
-            f[i] = (T)keep[(long long)i * A + oi];  // f_i(x, t), kept by the last step
-          } else {
-            const int ax = a.out_face >> 1, sg = (a.out_face & 1) ? 1 : -1;
-            const FaceNode in = face_node(a, x - (ax == 0 ? sg : 0), y - (ax == 1 ? sg : 0),
-                                          z - (ax == 2 ? sg : 0));
-            const T vin = face_pull<LAT, i, S, T>(a, src, in, isc);
-            T U = (T)keep[(long long)Q * A + oi];
-            if (U < (T)0) U = (T)0;
-            f[i] = ((T)keep[(long long)i * A + oi] + U * vin) / ((T)1 + U);
-          }
-          return;
-        }
-      }
       f[i] = face_pull<LAT, i, S, T>(a, src, fn, isc);
     });
+    if (out) {
+      // the outflow rule, on links that cross it and no velocity face
+      const int ax = a.out_face >> 1, sg = (a.out_face & 1) ? 1 : -1;
+      const FaceNode in = face_node(a, x - (ax == 0 ? sg : 0), y - (ax == 1 ? sg : 0),
+                                    z - (ax == 2 ? sg : 0));
+      T U = (T)keep[(long long)Q * A + oi];
+      if (U < (T)0) U = (T)0;
+      static_for<Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        const int cx = crossed<LAT, i, 0>(fn), cy = crossed<LAT, i, 1>(fn), cz = crossed<LAT, i, 2>(fn);
+        const bool vel = cx == LBM_FACE_VELOCITY || cy == LBM_FACE_VELOCITY || cz == LBM_FACE_VELOCITY;
+        const bool conv = cx == LBM_FACE_CONVECTIVE || cy == LBM_FACE_CONVECTIVE || cz == LBM_FACE_CONVECTIVE;
+        if (!vel && conv) {
+          if (MODE == 1)
+            f[i] = (T)keep[(long long)i * A + oi];  // f_i(x, t), kept by the last step
+          else
+            f[i] = ((T)keep[(long long)i * A + oi] + U * face_pull<LAT, i, S, T>(a, src, in, isc)) /
+                   ((T)1 + U);
+        }
+      });
+    }
   }
   if (MODE != 1 && out) {
     // this step's pre-collision populations and outward velocity, read by
@@ -1031,8 +1037,8 @@ namespace lbm {
 inline int div_up(long long a, int b) { return (int)((a + b - 1) / b); }
 
 // The vector bulk sweep: W words per thread and direction (bulk_vec_words 2
-// or 4; 0 = 2) and the node-pair collision packed (bulk_vec_packed 1, and -1,
-// the default: figures at vec_regs) or node by node (0).  Returns false where nx or the direction stride is not a
+// or 4; 0 = 2) and the node-pair collision packed (bulk_vec_packed 1) or node
+// by node (0); -1 is the storage type's default.  Returns false where nx or the direction stride is not a
 // multiple of the V nodes of a vector.
 //
 // Both arrays together up to kReuseBytes (1.5 times the 129 MB L2): the reads
@@ -1051,21 +1057,24 @@ bool launch_bulk_vec_w(const KArgs &a, int want, bool packed, cudaStream_t st) {
   const int nt = (int)(a.N / V);
   const int grid = div_up(nt, want);
   // the hint is built for the default shape only
-  if (W == 2 && packed) {
-    if (2 * Lat<LAT>::Q * a.fs * (long long)sizeof(S) <= kReuseBytes)
-      k_bulk_vec<LAT, CM, S, W, true, W == 2 ? LD_ONCE : LD_NC><<<grid, want, 0, st>>>(a);
+  const bool once = 2 * Lat<LAT>::Q * a.fs * (long long)sizeof(S) <= kReuseBytes;
+  constexpr int kOnce = W == 2 ? LD_ONCE : LD_NC;
+  if (packed) {
+    if (once && vec_packed<S>())
+      k_bulk_vec<LAT, CM, S, W, true, vec_packed<S>() ? kOnce : LD_NC><<<grid, want, 0, st>>>(a);
     else
       k_bulk_vec<LAT, CM, S, W, true, LD_NC><<<grid, want, 0, st>>>(a);
-  } else if (packed) {
-    k_bulk_vec<LAT, CM, S, W, true, LD_NC><<<grid, want, 0, st>>>(a);
   } else {
-    k_bulk_vec<LAT, CM, S, W, false, LD_NC><<<grid, want, 0, st>>>(a);
+    if (once && !vec_packed<S>())
+      k_bulk_vec<LAT, CM, S, W, false, vec_packed<S>() ? LD_NC : kOnce><<<grid, want, 0, st>>>(a);
+    else
+      k_bulk_vec<LAT, CM, S, W, false, LD_NC><<<grid, want, 0, st>>>(a);
   }
   return true;
 }
 template <int LAT, int CM, typename S>
 bool launch_bulk_vec(const KArgs &a, int want, cudaStream_t st) {
-  const bool packed = a.bulk_vec_packed != 0;
+  const bool packed = a.bulk_vec_packed >= 0 ? a.bulk_vec_packed != 0 : vec_packed<S>();
   if (a.bulk_vec_words == 4) return launch_bulk_vec_w<LAT, CM, S, 4>(a, want, packed, st);
   return launch_bulk_vec_w<LAT, CM, S, 2>(a, want, packed, st);
 }
@@ -1152,11 +1161,13 @@ bool launch_group_t(const KArgs *as, int n, cudaStream_t st) {
           as[k].bulk_vec_packed != a0.bulk_vec_packed || as[k].bulk_block != a0.bulk_block)
         return false;
     if (a0.bulk_mode < 1 || n < 1 || n > kMaxGroup) return false;
-    // only the default vector shape is built grouped (2 words, packed pairs):
-    // each grouped variant inlines the update kMaxGroup times
-    if (a0.bulk_vec_words == 4 || a0.bulk_vec_packed == 0) return false;
+    // only the default vector shape of the storage type is built grouped: each
+    // grouped variant inlines the update kMaxGroup times
+    constexpr bool kPacked = vec_packed<S>();
+    const bool packed = a0.bulk_vec_packed >= 0 ? a0.bulk_vec_packed != 0 : kPacked;
+    if (a0.bulk_vec_words == 4 || packed != kPacked) return false;
     const int want = a0.bulk_block > 0 ? a0.bulk_block : 128;
-    return launch_group_w<LAT, CM, S, 2, true>(as, n, want, st);
+    return launch_group_w<LAT, CM, S, 2, kPacked>(as, n, want, st);
   }
 }
 

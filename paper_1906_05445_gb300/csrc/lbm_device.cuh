@@ -271,8 +271,7 @@ __device__ __forceinline__ V edot_lead(V vx, V vy, V vz) {
 // add up exactly, w0 + 6 r wb + 12 wb = 1 and 2 (3 w1) + 8 (3 wb) = 1 on D3Q19
 // (w0 + 4 r wb + 4 wb = 1 and 2 (3 w1) + 4 (3 wb) = 1 on D2Q9): rounded one by
 // one (1/6 and 1/12 are both 3e-8 high) they scale the momentum by 1 + 3e-8 omega
-// every step, which is the largest systematic error of FP32 storage over
-// thousands of steps.
+// every step.
 template <int LAT, typename C> struct CollW {
   static constexpr bool f32 = sizeof(C) == 4;
   static constexpr double p25 = 1.0 / 33554432.0, p26 = p25 / 2, p27 = p25 / 4, p29 = p25 / 16;
@@ -312,12 +311,10 @@ template <int LAT, typename C> struct CollW {
 // commutes with rounding, so the stored values equal those of colliding the
 // unscaled deviations.
 // EVEN_FIRST adds the small even part to the old value before the larger odd
-// one, so that the odd part is rounded once: the stress noise of an FP32 step is
-// half that of adding the parts first, and the velocity error of a sphere flow
-// started from rest at g = 3.4e-8 is 1.6e-6 after 2000 steps against 4.9e-6.
-// BF16 storage is also faster with it (160^3 51.7 us per step against 53.3);
-// FP16 storage, whose rounding hides the difference, is not (53.4 / 53.3) and
-// adds the parts first.
+// one, so that the odd part is rounded once (half the stress noise of adding the
+// parts first).  BF16 storage is also faster with it (160^3 51.7 us per step
+// against 53.3); FP16 storage, whose rounding hides the difference, is not
+// (53.4 / 53.3) and adds the parts first.
 template <typename ST> __host__ __device__ constexpr bool even_first() {
   return !std::is_same<ST, __half>::value;
 }
@@ -429,14 +426,31 @@ __device__ __forceinline__ void collide_two_rate(V (&f)[Lat<LAT>::Q], V Fx, V Fy
   });
 }
 
-// One node; ST is the storage type of the populations.
+// Sum over the pair leaders i of q_a,i 3 w_i e_i,b: the q moments of the
+// pairs' terms -2 A_i + AF_i (A_i = 3 w_i e_i.u, AF_i = 3 w_i e_i.F) are
+// sum_b K_ab (F_b - 2 u_b).
+template <int LAT> __host__ __device__ constexpr double qk(int a, int b) {
+  using L = Lat<LAT>;
+  double s = 0;
+  for (int i = 1; i < L::Q; i++)
+    if (L::opp(i) > i) {
+      const int e = b == 0 ? L::ex(i) : (b == 1 ? L::ey(i) : L::ez(i));
+      s += qrow<LAT>(a, i) * 3.0 * L::w(i) * e;
+    }
+  return s;
+}
+
+// One node; ST is the storage type of the populations.  FP32 storage collides
+// pair by pair: its sweep is bound by HBM (128^3 without solids 51.6 us per
+// step, 50.9 with the grouped form, before the walk alternated), and over
+// hundreds of steps the two forms' roundings drift apart by 1e-5.
 template <int LAT, int CM, typename ST, typename T>
 __device__ __forceinline__ void collide(T (&f)[Lat<LAT>::Q], T Fx, T Fy, T Fz,
                                         const Coll<T> &c) {
   using L = Lat<LAT>;
   constexpr int Q = L::Q;
   constexpr bool MRT = CM == CM_MRT;
-  if constexpr (!MRT) {
+  if constexpr (!MRT && !std::is_same<ST, float>::value) {
     collide_two_rate<LAT, CM, 0, even_first<ST>(), T, T>(f, Fx, Fy, Fz, c);
     return;
   }
@@ -456,6 +470,66 @@ __device__ __forceinline__ void collide(T (&f)[Lat<LAT>::Q], T Fx, T Fy, T Fz,
   const T uF = ux * Fx + uy * Fy + uz * Fz;
   const T base = drho - (T)1.5 * uu;
   const T om = c.omega, omc = c.omc, cf = c.cforce;
+  if constexpr (CM != CM_MRT) {
+    // FP32 storage: BGK, or MRT whose only non-BGK moments are the q moments,
+    // in place pair by pair, grouped for few operations (as the packed pair
+    // collision): omega S + cforce SF = w B + A g with B = omega base -
+    // 3 cforce u.F and g = 1.5 omega e.u + 3 cforce e.F; omega A + cforce AF
+    // = omega A + w (3 cforce e.F); the q moments of Delta + Fbar/2 are
+    // sum_i q_a,i (f_i - f_ib) + K (F - 2u) (qk: the pairs' -2A + AF terms)
+    T mq[3] = {0, 0, 0};
+    const T om15 = om * (T)1.5, cf3 = cf * (T)3;
+    const T B = om * base - cf3 * uF;
+    f[0] = omc * f[0] + (T)L::w(0) * B;
+    const T Ba = (T)L::w(1) * B, Bb = (T)L::w(Q - 1) * B;
+    static_for<Q>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      if constexpr (i > 0 && L::opp(i) > i) {
+        constexpr int j = L::opp(i);
+        constexpr T w = (T)L::w(i);
+        constexpr bool ca = L::w(i) == L::w(1);
+        const T eu = edot<LAT, i, T>(ux, uy, uz);
+        const T eF = edot<LAT, i, T>(Fx, Fy, Fz);
+        const T A = (T)(3.0 * L::w(i)) * eu;
+        const T t = cf3 * eF;
+        const T P = A * (om15 * eu + t) + (ca ? Ba : Bb);
+        const T M = om * A + w * t;
+        if constexpr (CM == CM_MRT_Q) {
+          const T d = f[i] - f[j];
+          static_for<L::D>([&](auto ac) {
+            constexpr int ax = decltype(ac)::value;
+            constexpr int q = qrow<LAT>(ax, i);
+            if constexpr (q != 0) mq[ax] += (T)q * d;
+          });
+        }
+        f[i] = omc * f[i] + P + M;
+        f[j] = omc * f[j] + P - M;
+      }
+    });
+    if constexpr (CM == CM_MRT_Q) {
+      const T fu[3] = {Fx - (T)2 * ux, Fy - (T)2 * uy, Fz - (T)2 * uz};
+      static_for<L::D>([&](auto ac) {
+        constexpr int ax = decltype(ac)::value;
+        static_for<L::D>([&](auto bc) {
+          constexpr int b = decltype(bc)::value;
+          constexpr T K = (T)qk<LAT>(ax, b);
+          if constexpr (K != (T)0) mq[ax] += K * fu[b];
+        });
+      });
+      // all q rows share one rate: a_a = (omega - s_q) m_q,a / |M_q|^2
+      const T k = c.ds[4] * (T)(1.0 / mnorm<LAT>(4));
+      T aq[3] = {k * mq[0], k * mq[1], k * mq[2]};
+      static_for<Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        static_for<L::D>([&](auto ac) {
+          constexpr int ax = decltype(ac)::value;
+          constexpr int q = qrow<LAT>(ax, i);
+          if constexpr (q != 0) f[i] += (T)q * aq[ax];
+        });
+      });
+    }
+    return;
+  }
   T out[Q];
   T v[MRT ? Q : 1];
   {

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kRunBlock, 1) k_run(const __grid_constant__ Ru
         constexpr int V = 2 * VecS<S>::per_word;
         const unsigned nt = (unsigned)a.N / V, nu = (nt + 31) / 32;
         for (unsigned u = (unsigned)(warp * nb + rb); u < nu; u += (unsigned)(nb * NW))
-          bulk_vec_update<LAT, CM, S, 2, true, LD_L2>(a, src, dst, u * 32 + lane, nt);
+          bulk_vec_update<LAT, CM, S, 2, vec_packed<S>(), LD_L2>(a, src, dst, u * 32 + lane, nt);
         done = true;
       }
     }

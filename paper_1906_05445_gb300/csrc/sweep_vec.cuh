@@ -6,9 +6,9 @@
 // the pulled values are the row shifted by one node: the thread takes the
 // missing end node from its neighbour lane's vector (or loads it itself at a
 // row or warp edge).  The collision then runs on pairs of nodes in packed
-// FP32x2 arithmetic (one instruction for two nodes) or node by node, both
-// through collide_two_rate in lbm_device.cuh: Eq. 1 (BGK) or Eq. 3 (MRT) with
-// Guo forcing, where MRT differs from BGK only on the energy-flux (q) moments.
+// FP32x2 arithmetic (one instruction for two nodes; 16-bit storage's default)
+// or node by node (FP32 storage's): Eq. 1 (BGK) or Eq. 3 (MRT) with Guo
+// forcing, where MRT differs from BGK only on the energy-flux (q) moments.
 //
 // Requirements (checked by the launcher, which otherwise runs the one-node
 // kernel): nx % V == 0 and a direction stride that is a multiple of V.
@@ -302,16 +302,18 @@ __device__ __forceinline__ void bulk_vec_update(const KArgs &a, const S *src, S 
   vec_collide_store<LAT, CM, S, W, PACKED>(a, dst, v, fl, n0, valid);
 }
 
-// Registers a thread of the 2-word kernels: FP32 80 (6 blocks of 128 per SM),
-// BF16 112, FP16 128.  Measured on 128^3 / 160^3 / 192^3 lattices without
-// solids, us per step: FP32 packed 54.2 / 102.5 / 174 at 64 registers (it
-// spills), 48.1 / 92.2 / 157.3 at 72, 47.2 / 90.7 / 154.6 at 80, 47.3 / 90.7 /
-// 154.1 at 96; FP32 node by node 48.1 / 92.6 / 158.2 at 64, 47.8 / 91.9 /
-// 156.8 at 72.  BF16 29.8 / 55.3 / 91.6 at 96, 26.7 / 49.0 / 82.0 at 112,
-// 26.8 / 50.7 / 84.4 at 128; FP16 30.8 / 57.3 / 95.8 at 96, 27.8 / 51.5 / 87.8
-// at 112, 26.7 / 49.5 / 84.0 at 128.  4-word vectors are left unbounded.
-template <typename S, int W> constexpr int vec_regs() {
-  return W == 4 ? 255 : sizeof(S) == 4 ? 80 : std::is_same<S, __nv_bfloat16>::value ? 112 : 128;
+// Whether a storage type's default vector kernel collides packed node pairs.
+template <typename S> __host__ __device__ constexpr bool vec_packed() { return sizeof(S) == 2; }
+// Registers a thread of the 2-word kernels: FP32 node by node 64 (8 blocks of
+// 128 per SM, whose warps hide more of the boundary kernel's share of the SMs
+// than 6 at 80), packed 80, BF16 112, FP16 128.  Measured on 128^3 / 160^3 /
+// 192^3 lattices without solids, us per step: BF16 29.8 / 55.3 / 91.6 at 96,
+// 26.7 / 49.0 / 82.0 at 112, 26.8 / 50.7 / 84.4 at 128; FP16 30.8 / 57.3 / 95.8
+// at 96, 27.8 / 51.5 / 87.8 at 112, 26.7 / 49.5 / 84.0 at 128.  4-word vectors
+// are left unbounded.
+template <typename S, int W, bool PACKED> constexpr int vec_regs() {
+  return W == 4 ? 255 : sizeof(S) == 4 ? (PACKED ? 80 : 64)
+                      : std::is_same<S, __nv_bfloat16>::value ? 112 : 128;
 }
 
 // One thread per vector.  (A persistent grid walking the lattice measured
@@ -321,10 +323,10 @@ template <typename S, int W> constexpr int vec_regs() {
 // Blocks walk the lattice from its end when a.rev is set (every other step):
 // a step then starts on the nodes that the previous one wrote last, which L2
 // still holds, instead of on those it has already evicted.  128^3 without
-// solids, FP32: 50.9 -> 48.0 us per step (and 47.2 with evict-first reads,
-// LD_ONCE); 112^3 36.1 -> 32.6 (30.9); FP16 128^3 28.8 -> 26.7 (24.7).
+// solids, FP32 (packed): 50.9 -> 48.0 us per step (and 47.2 with evict-first
+// reads, LD_ONCE); 112^3 36.1 -> 32.6 (30.9); FP16 128^3 28.8 -> 26.7 (24.7).
 template <int LAT, int CM, typename S, int W, bool PACKED, int POL>
-__global__ void __maxnreg__((vec_regs<S, W>()))
+__global__ void __maxnreg__((vec_regs<S, W, PACKED>()))
     k_bulk_vec(const KArgs a) {
   constexpr int V = W * VecS<S>::per_word;
   const unsigned b = a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
@@ -340,7 +342,7 @@ __global__ void __maxnreg__((vec_regs<S, W>()))
 // fewer).
 // The single-lattice kernel's register limits.
 template <int LAT, int CM, typename S, int W, bool PACKED>
-__global__ void __maxnreg__((vec_regs<S, W>()))
+__global__ void __maxnreg__((vec_regs<S, W, PACKED>()))
     k_bulk_vec_group(const __grid_constant__ GroupArgs g) {
   constexpr int V = W * VecS<S>::per_word;
   const int b = (int)blockIdx.x;
