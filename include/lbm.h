@@ -71,8 +71,8 @@ enum {
  * from twice the resolution).  Measured:
  *  - fixed sphere, R = 3.75 in a 40^3 periodic box, tau = 0.6, g = 3.4e-8
  *    (flow speed ~1e-4), 2000 steps: FP16 meets it under IBM (0.05-0.8%) but
- *    not under quadratic Bouzidi (24%); BF16 meets it under neither (IBM
- *    3-19% from run to run, Bouzidi 366%);
+ *    not under quadratic Bouzidi (33%); BF16 meets it under neither (IBM
+ *    up to 32%, Bouzidi 181%);
  *  - sphere translating at U = 0.01 (R = 8, 20000 steps): FP16 meets it
  *    under both schemes (4.8% / 0.46%); BF16 under IBM only (9.7%), not
  *    under Bouzidi with refilling (216%).
