@@ -2740,9 +2740,9 @@ void drop_graph(lbm_batch *b) {
 bool graphable(const lbm_ctx *c) { return (!any_moving(c) || dev_motion(c)) && !run_ok(c); }
 
 // All nsteps of the active lattices that k_run takes, up to kMaxRun of one
-// kind per launch (eight lattices of edges 24..64, alternately bounce-back and
-// IBM: 12 + 26 us per step in two launches, 52 in one whose threads hold both
-// kinds' constants, 45 as graph replays).
+// kind per launch.  Eight lattices of edges 24..64, alternately bounce-back and
+// IBM: 40.6 us per step (12.6 + 28.3 in two launches) against 45.9 as graph
+// replays; in one launch whose threads hold both kinds' constants 52.
 lbm_status batch_run(lbm_batch *b, int nsteps) {
   const int n = (int)b->ctx.size();
   std::vector<char> done(n, 0);
