@@ -399,8 +399,10 @@ __global__ void __launch_bounds__(kRunBlock, 1) k_run(const __grid_constant__ Ru
           dF = (it == 0 ? mi.Ud : dF) - sum;
           Fm = it == 0 ? dF : Fm + dF;
           if (!last) ((T *)a.tab.dFT)[(size_t)((it & 1) * 3 + lane) * nm + mi.m] = (T)dF;
-          else ((T *)a.tab.FdV)[lane * nm + mi.m] = (T)(Fm * a.tab.dV[mi.m]);
         }
+        // all three components (z is zero in 2D): the band nodes gather three
+        if (last && mi.m >= 0 && lane < 3)
+          ((T *)a.tab.FdV)[lane * nm + mi.m] = (T)(Fm * a.tab.dV[mi.m]);
         run_arrive(r.bar);
         if (last) {
           // the solids' reaction while the other blocks arrive

@@ -1,0 +1,58 @@
+"""Where the multi-step launch of small lattices (k_run) meets the rest of the
+library: geometry changed between launches.  Every case is compared with the
+same steps as launches of their own (LBM_RUN=0).
+"""
+import numpy as np
+import pytest
+
+from paper_1906_05445_gb300 import workloads as W
+
+from .parity import rel_l2
+
+pytestmark = pytest.mark.gpu
+
+DISC = [W.Solid(W.CYLINDER_Z, (15.7, 16.2, 0.0), 6.0, omega=(0.0, 0.0, 0.002))]
+
+
+def _disc(precision, iters=1, scheme=W.IBM):
+    return W.Problem("disc", W.D2Q9, 33, 32, 1, 0.7, W.MRT, precision, (1e-4, -2e-4, 0.0),
+                     DISC, scheme, 0, ibm_iters=iters)
+
+
+def _poison():
+    """Leave small blocks of device memory that the next allocations may reuse
+    full of NaN: the populations of lattices that held nothing else."""
+    from paper_1906_05445_gb300 import lbm
+    lats = []
+    for n in [4, 8, 12, 16, 24] * 16:
+        g = lbm.Lattice(W.D2Q9, n, n, 1, 0.7, precision=W.FP32)
+        g.set_f(np.full((9, 1, n, n), np.nan))
+        lats.append(g)
+    for g in lats:
+        g.close()
+
+
+@pytest.mark.parametrize("iters", [1, 3])
+@pytest.mark.parametrize("precision,tol", [(W.FP64, 1e-13), (W.FP32, 2e-6)])
+def test_markers_changed_between_launches_2d(monkeypatch, precision, tol, iters):
+    """New IBM tables straight into a multi-step launch, without an initial
+    collision: the unused z component of the markers' forces reads as zero.
+    Both runs sum the same few hundred terms in another order."""
+    from paper_1906_05445_gb300 import lbm
+    out = []
+    for run in ("0", "1"):
+        monkeypatch.setenv("LBM_RUN", run)
+        g = lbm.Lattice.from_problem(_disc(precision, iters))
+        g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        g.step(4)
+        # more markers: larger tables, in memory that held something else
+        g.set_scheme(W.IBM, iters, 0.0, 6.0)
+        g.set_solid_motion(0, centre=(15.9, 16.1, 0.0), omega=(0.0, 0.0, 0.001))
+        _poison()
+        g.step(9)
+        out.append((g.velocity(), g.solid_mask(), g.force_torque(0)))
+        g.close()
+    assert np.isfinite(out[1][0]).all()
+    assert rel_l2(out[1][0], out[0][0], out[0][1]) <= tol
+    for a, b in zip(out[0][2], out[1][2]):
+        assert np.abs(a - b).max() <= 20 * tol * np.abs(out[0][2][0]).max()
