@@ -73,6 +73,9 @@ using namespace lbm;
 namespace {
 
 constexpr int kHistCap = 4096;          // force records kept (steps)
+// slots of their ring: one more than is handed out, for the record that a
+// multi-step launch clears ahead of the step after it
+constexpr int kHistSlots = kHistCap + 1;
 constexpr double kFp16Scale = (double)(1 << kFp16ScaleLog2);  // FP16 storage keeps (f - w) * 2^10
 constexpr int kGeomMargin = 7;          // box margin around a moving solid
 
@@ -1321,7 +1324,7 @@ lbm_status init_collide(lbm_ctx *ctx) {
   TRY(ensure_geometry(ctx));
   const int prev = 1 - ctx->cur;
   ctx->zero_slot = -1;
-  ctx->slot = (ctx->slot + 1) % kHistCap;
+  ctx->slot = (ctx->slot + 1) % kHistSlots;
   double *acc = force_slot(ctx, ctx->slot);
   CK(cudaMemsetAsync(acc, 0, sizeof(double) * kMaxSolids * 6, ctx->st));
   ibm_prepass(ctx, ctx->f[prev], true, true, acc, ctx->st);
@@ -1389,7 +1392,7 @@ lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
     a.dst = ctx->f[cur];
     sweep(ctx, OP_REFILL, a);
   }
-  ctx->slot = (ctx->slot + 1) % kHistCap;
+  ctx->slot = (ctx->slot + 1) % kHistSlots;
   ctx->zero_slot = -1;
   double *acc = force_slot(ctx, ctx->slot);
   a = base_args(ctx);
@@ -1538,12 +1541,12 @@ lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
     r.cur = c->cur;
     r.nsteps = nsteps;
     r.slot0 = c->slot;
-    r.hist_cap = kHistCap;
+    r.hist_cap = kHistSlots;
     r.hist = c->hist;
     r.bar = c->run_bar;
     r.iters = std::max(1, c->scheme.ibm_iters);
     r.vec = vec ? 1 : 0;
-    const int first = (c->slot + 1) % kHistCap;
+    const int first = (c->slot + 1) % kHistSlots;
     // the record the launch starts with: left zeroed by the launch before
     // (never relied on in a capture, whose replays find their own sums there)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1556,8 +1559,8 @@ lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
   CK(launch_run(g, ctx->d.lattice, ctx->coll_mode, ctx->d.precision, st));
   for (int k = 0; k < n; k++) {
     lbm_ctx *c = ctxs[k];
-    c->slot = (c->slot + nsteps) % kHistCap;
-    c->zero_slot = (c->slot + 1) % kHistCap;
+    c->slot = (c->slot + nsteps) % kHistSlots;
+    c->zero_slot = (c->slot + 1) % kHistSlots;
     c->cur = (c->cur + nsteps) & 1;
     c->prev_local = false;
     c->records = std::min<long long>(c->records + nsteps, kHistCap);
@@ -1905,7 +1908,7 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
       (s = dalloc(ctx, (void **)&ctx->flags, padN)) != LBM_OK ||
       (s = dalloc(ctx, (void **)&ctx->sid, 2 * padN)) != LBM_OK ||
       (s = dalloc(ctx, (void **)&ctx->counts, 16 * sizeof(int))) != LBM_OK ||
-      (s = dalloc(ctx, (void **)&ctx->hist, sizeof(double) * kHistCap * kMaxSolids * 6)) != LBM_OK ||
+      (s = dalloc(ctx, (void **)&ctx->hist, sizeof(double) * kHistSlots * kMaxSolids * 6)) != LBM_OK ||
       (s = dalloc(ctx, (void **)&ctx->run_bar, 2 * sizeof(unsigned))) != LBM_OK ||
       (s = dalloc(ctx, (void **)&ctx->red2, 2 * sizeof(double))) != LBM_OK) {
     lbm_destroy(ctx);
@@ -1915,7 +1918,7 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
   cudaMemsetAsync(ctx->sid, 0, 2 * padN, ctx->st);
   cudaMemsetAsync(ctx->counts, 0, 16 * sizeof(int), ctx->st);
   cudaMemsetAsync(ctx->run_bar, 0, 2 * sizeof(unsigned), ctx->st);
-  cudaMemsetAsync(ctx->hist, 0, sizeof(double) * kHistCap * kMaxSolids * 6, ctx->st);
+  cudaMemsetAsync(ctx->hist, 0, sizeof(double) * kHistSlots * kMaxSolids * 6, ctx->st);
   // rest state f = w as a pre-collision state, collided on first use
   KArgs a = base_args(ctx);
   a.dst = ctx->f[1];
@@ -2274,11 +2277,11 @@ lbm_status lbm_get_force_history(lbm_ctx *ctx, int id, double *host_out, size_t 
   if (!ctx || id < 0 || id >= (int)ctx->solids.size() || !n) return LBM_ERR_ARG;
   TRY(prepare(ctx));
   const long long have = std::min<long long>(ctx->records, (long long)max_steps);
-  std::vector<double> all((size_t)kHistCap * kMaxSolids * 6);
+  std::vector<double> all((size_t)kHistSlots * kMaxSolids * 6);
   CK(cudaMemcpyAsync(all.data(), ctx->hist, all.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
   CK(cudaStreamSynchronize(ctx->st));
   for (long long k = 0; k < have; k++) {
-    const int slot = (int)(((ctx->slot - (have - 1 - k)) % kHistCap + kHistCap) % kHistCap);
+    const int slot = (int)(((ctx->slot - (have - 1 - k)) % kHistSlots + kHistSlots) % kHistSlots);
     if (host_out) memcpy(host_out + 6 * k, &all[((size_t)slot * kMaxSolids + id) * 6], 6 * sizeof(double));
   }
   *n = (size_t)have;
@@ -2550,7 +2553,7 @@ lbm_status lbm_load(lbm_ctx *ctx, const void *host_buf, size_t size) {
   if (!ctx->need_collide && ctx->scheme.scheme == LBM_IBM_DIRECT) {
     // the IBM force of the current time is recomputed from the restored state
     ctx->zero_slot = -1;
-    ctx->slot = (ctx->slot + 1) % kHistCap;
+    ctx->slot = (ctx->slot + 1) % kHistSlots;
     double *acc = force_slot(ctx, ctx->slot);
     CK(cudaMemsetAsync(acc, 0, sizeof(double) * kMaxSolids * 6, ctx->st));
     ibm_prepass(ctx, ctx->f[1], ctx->prev_local, true, acc, ctx->st);
@@ -2702,7 +2705,7 @@ lbm_status autotune(lbm_ctx *ctx, void *scratch) {
   KArgs a = base_args(ctx);
   a.src = ctx->f[ctx->cur];
   a.dst = scratch;
-  a.force_acc = force_slot(ctx, (ctx->slot + kHistCap / 2) % kHistCap);
+  a.force_acc = force_slot(ctx, (ctx->slot + kHistCap / 2) % kHistSlots);
   float best = 1e30f;
   int best_b = ctx->bulk_block;
   for (int c : cand_bulk) {
@@ -2818,7 +2821,7 @@ lbm_status capture(lbm_batch *b) {
     // the first step reads it there (the current record is copied there
     // before the first replay, below)
     if (c->scheme.scheme == LBM_IBM_DIRECT && dev_motion(c))
-      c->motion_slot = (c->slot + 2) % kHistCap;
+      c->motion_slot = (c->slot + 2) % kHistSlots;
     cudaStreamWaitEvent(c->st, b->ev_origin, 0);
     st = step_once(c);
     if (st == LBM_OK) st = step_once(c);
@@ -2835,7 +2838,7 @@ lbm_status capture(lbm_batch *b) {
     lbm_ctx *c = b->ctx[i];
     c->motion_slot = -1;
     if (c->scheme.scheme == LBM_IBM_DIRECT && dev_motion(c))
-      cudaMemcpyAsync(force_slot(c, (saved[i].slot + 2) % kHistCap), force_slot(c, saved[i].slot),
+      cudaMemcpyAsync(force_slot(c, (saved[i].slot + 2) % kHistSlots), force_slot(c, saved[i].slot),
                       sizeof(double) * kMaxSolids * 6, cudaMemcpyDeviceToDevice, c->st);
     b->pair_launches[i] = c->launches - saved[i].launches;
     b->graph_slot[i] = c->slot;  // after two captured steps

@@ -56,3 +56,22 @@ def test_markers_changed_between_launches_2d(monkeypatch, precision, tol, iters)
     assert rel_l2(out[1][0], out[0][0], out[0][1]) <= tol
     for a, b in zip(out[0][2], out[1][2]):
         assert np.abs(a - b).max() <= 20 * tol * np.abs(out[0][2][0]).max()
+
+
+def test_whole_force_history_of_a_full_ring(monkeypatch):
+    """Once more steps ran than records are kept, the history still holds the
+    last 4096 steps, the oldest included."""
+    from paper_1906_05445_gb300 import lbm
+    hist = []
+    for run in ("0", "1"):
+        monkeypatch.setenv("LBM_RUN", run)
+        g = lbm.Lattice.from_problem(_disc(W.FP64, scheme=W.BOUZIDI_QUAD))
+        g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        g.step(2100)
+        g.step(2110)
+        hist.append(g.force_history(0))
+        g.close()
+    assert hist[0].shape == hist[1].shape == (4096, 6)
+    # FP64 sums of the same parts in another order
+    assert np.abs(hist[0] - hist[1]).max() <= 1e-12 * max(1.0, np.abs(hist[0]).max())
+    assert np.abs(hist[1][0, :2]).min() > 1e-8
