@@ -1522,6 +1522,9 @@ lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
     w[k] = (double)c->N * c->Q;
     sum += w[k];
   }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(st, &cap));
+  const bool capturing = cap != cudaStreamCaptureStatusNone;
   int at = 0;
   for (int k = 0; k < n; k++) {
     lbm_ctx *c = ctxs[k];
@@ -1549,9 +1552,7 @@ lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
     const int first = (c->slot + 1) % kHistSlots;
     // the record the launch starts with: left zeroed by the launch before
     // (never relied on in a capture, whose replays find their own sums there)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(st, &cap));
-    if (c->zero_slot != first || cap != cudaStreamCaptureStatusNone)
+    if (c->zero_slot != first || capturing)
       CK(cudaMemsetAsync(force_slot(c, first), 0, sizeof(double) * kMaxSolids * 6, st));
   }
   g.block_start[n] = at;
@@ -1560,7 +1561,8 @@ lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
   for (int k = 0; k < n; k++) {
     lbm_ctx *c = ctxs[k];
     c->slot = (c->slot + nsteps) % kHistSlots;
-    c->zero_slot = (c->slot + 1) % kHistSlots;
+    // a captured launch has not run: nothing is zeroed yet
+    c->zero_slot = capturing ? -1 : (c->slot + 1) % kHistSlots;
     c->cur = (c->cur + nsteps) & 1;
     c->prev_local = false;
     c->records = std::min<long long>(c->records + nsteps, kHistCap);

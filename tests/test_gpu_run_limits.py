@@ -75,3 +75,26 @@ def test_whole_force_history_of_a_full_ring(monkeypatch):
     # FP64 sums of the same parts in another order
     assert np.abs(hist[0] - hist[1]).max() <= 1e-12 * max(1.0, np.abs(hist[0]).max())
     assert np.abs(hist[1][0, :2]).min() > 1e-8
+
+
+def test_captured_launch_clears_no_record_by_itself(monkeypatch):
+    """Steps captured into a graph that is never launched leave every record
+    as it was: the next launch clears its own first one."""
+    import torch
+    from paper_1906_05445_gb300 import lbm
+    out = []
+    for run in ("0", "1"):
+        monkeypatch.setenv("LBM_RUN", run)
+        s = torch.cuda.Stream()
+        g = lbm.Lattice.from_problem(_disc(W.FP64, scheme=W.BOUZIDI_QUAD), stream=s.cuda_stream)
+        g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        g.step(4200)  # every slot of the ring holds a record
+        g.sync()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s, capture_error_mode="thread_local"):
+            g.step(2)
+        g.step(3)
+        out.append(g.force_history(0, 3))
+        g.close()
+        del graph
+    assert np.abs(out[0] - out[1]).max() <= 1e-12 * max(1.0, np.abs(out[0]).max())
