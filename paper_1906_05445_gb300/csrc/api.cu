@@ -1506,12 +1506,9 @@ bool run_small(const lbm_ctx *ctx) {
   return v <= (f64 ? 2400000 : 17000000);
 }
 
-// nsteps steps of the lattices in `ctxs` (run_ok, same lattice, collision and
-// precision, all or none with IBM tables, at most kMaxRun) in one launch on `st`, which follows their own
-// streams' earlier work and precedes their later work (the caller's order).
-lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
+// One launch of k_run: nsteps steps of the lattices in `ctxs` on `st`.
+lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
   lbm_ctx *ctx = ctxs[0];
-  if (nsteps < 1) return LBM_OK;
   RunArgs<kMaxRun> g;
   memset(&g, 0, sizeof(g));
   g.n = n;
@@ -1570,6 +1567,22 @@ lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
     c->launches++;
     c->bulk_kernel = run_vec(c) ? BK_VEC : BK_NODE;
   }
+  return LBM_OK;
+}
+
+// Steps per launch: a launch holds the SMs it runs on to its end, and other
+// streams wait for them.  At the largest lattices that k_run takes (about 110 us
+// per step) 256 steps are 28 ms; a launch and its set-up, a few us, are under
+// 1% of 256 of the shortest steps.
+constexpr int kRunSteps = 256;
+
+// nsteps steps of the lattices in `ctxs` (run_ok, same lattice, collision and
+// precision, all or none with IBM tables, at most kMaxRun) on `st`, which follows
+// their own streams' earlier work and precedes their later work (the caller's
+// order).
+lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
+  for (int done = 0; done < nsteps; done += kRunSteps)
+    TRY(run_launch(ctxs, n, std::min(kRunSteps, nsteps - done), st));
   return LBM_OK;
 }
 

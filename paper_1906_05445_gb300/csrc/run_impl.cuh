@@ -3,8 +3,8 @@
 // A small lattice's step is a chain of short kernels on two streams: with the
 // launches, the fork and the join between them it took 11-17 us per step for
 // the 64^2 and 301^2 Couette flows and 47-75 us with five IBM forcing
-// iterations at 48^3, against 1-6 us of work.  k_run takes all the steps of a
-// call in one cooperative launch: the lattice's blocks (one per SM at most)
+// iterations at 48^3, against 1-6 us of work.  k_run takes the steps of a
+// call (up to 256 at a time) in one cooperative launch: the lattice's blocks (one per SM at most)
 // keep stepping, with a barrier over them wherever one phase reads what
 // another wrote:
 //   bounce-back or no solids: boundary nodes and plain nodes read f*(t) and
@@ -22,9 +22,10 @@ namespace lbm {
 
 // Barrier over the nb blocks of a lattice, in two halves, so that work the
 // other blocks do not wait for runs in between.  ctr counts arrivals since the
-// launch began (target: nb per barrier so far).  run_wait is false when the
-// barrier was not reached within a second: the kernel then records it and
-// returns.
+// launch began (target: nb per barrier so far), both modulo 2^32: they are never
+// further apart than a barrier's blocks, so their difference has a sign.
+// run_wait is false when the barrier was not reached within a second: the kernel
+// then records it and returns.
 __device__ __forceinline__ void run_arrive(unsigned *ctr) {
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -38,7 +39,7 @@ __device__ __forceinline__ bool run_wait(unsigned *ctr, unsigned target, int *er
     unsigned long long t0 = 0, now;
     for (unsigned spin = 0;; spin++) {
       asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-      if (v >= target) break;
+      if ((int)(v - target) >= 0) break;
       if ((spin & 255u) == 255u) {
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
         if (t0 == 0) t0 = now;

@@ -98,3 +98,25 @@ def test_captured_launch_clears_no_record_by_itself(monkeypatch):
         g.close()
         del graph
     assert np.abs(out[0] - out[1]).max() <= 1e-12 * max(1.0, np.abs(out[0]).max())
+
+
+@pytest.mark.parametrize("scheme", [W.BOUZIDI_QUAD, W.IBM])
+def test_long_calls_run_in_launches_of_bounded_length(monkeypatch, scheme):
+    """A call of many steps is split: 600 steps are three launches, with the
+    results of the same steps in short calls."""
+    from paper_1906_05445_gb300 import lbm
+    monkeypatch.setenv("LBM_RUN", "1")
+    out = []
+    for calls in ((600,), (100,) * 6):
+        g = lbm.Lattice.from_problem(_disc(W.FP32, 2, scheme=scheme))
+        g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        g.step(2)
+        n0 = g.info().kernel_launches
+        for k in calls:
+            g.step(k)
+        out.append((g.info().kernel_launches - n0, g.get_f(), g.force_history(0)))
+        g.close()
+    assert out[0][0] == 3 and out[1][0] == 6
+    assert np.array_equal(out[0][1], out[1][1])
+    # FP64 sums of the same parts in another order
+    assert np.abs(out[0][2] - out[1][2]).max() <= 1e-12 * max(1.0, np.abs(out[0][2]).max())
