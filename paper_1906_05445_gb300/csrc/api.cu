@@ -217,7 +217,7 @@ struct lbm_ctx {
   unsigned *run_bar = nullptr;  // k_run's barrier counters (zero between launches)
   int zero_slot = -1;           // the record a k_run launch left zeroed for the step after it
   bool run_on = true;           // LBM_RUN=0: every step as launches of its own
-  int sms = 0;
+  int sms = 0;                  // blocks of a k_run launch at most: the SMs, or LBM_RUN_SMS
   int slot = 0;
   long long records = 0;
   // queries / residual
@@ -1507,7 +1507,10 @@ bool run_small(const lbm_ctx *ctx) {
 }
 
 // One launch of k_run: nsteps steps of the lattices in `ctxs` on `st`.
-lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
+// *refused: the blocks do not fit beside each other on the SMs that the stream
+// may use (a green context, a limited client), or cooperative launches are not
+// supported there; nothing was stepped.
+lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st, bool *refused) {
   lbm_ctx *ctx = ctxs[0];
   RunArgs<kMaxRun> g;
   memset(&g, 0, sizeof(g));
@@ -1554,7 +1557,14 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) 
   }
   g.block_start[n] = at;
   for (int k = n; k < kMaxRun; k++) g.block_start[k + 1] = at;
-  CK(launch_run(g, ctx->d.lattice, ctx->coll_mode, ctx->d.precision, st));
+  const cudaError_t e = launch_run(g, ctx->d.lattice, ctx->coll_mode, ctx->d.precision, st);
+  *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+             e == cudaErrorNotSupported;
+  if (*refused) {
+    cudaGetLastError();
+    return LBM_OK;
+  }
+  CK(e);
   for (int k = 0; k < n; k++) {
     lbm_ctx *c = ctxs[k];
     c->slot = (c->slot + nsteps) % kHistSlots;
@@ -1576,13 +1586,22 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) 
 // 1% of 256 of the shortest steps.
 constexpr int kRunSteps = 256;
 
-// nsteps steps of the lattices in `ctxs` (run_ok, same lattice, collision and
-// precision, all or none with IBM tables, at most kMaxRun) on `st`, which follows
-// their own streams' earlier work and precedes their later work (the caller's
-// order).
-lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st) {
-  for (int done = 0; done < nsteps; done += kRunSteps)
-    TRY(run_launch(ctxs, n, std::min(kRunSteps, nsteps - done), st));
+// Up to nsteps steps of the lattices in `ctxs` (run_ok, same lattice, collision
+// and precision, all or none with IBM tables, at most kMaxRun) on `st`, which
+// follows their own streams' earlier work and precedes their later work (the
+// caller's order).  *ran: the steps done; fewer than nsteps where a launch was
+// refused, and these lattices then step with launches of their own.
+lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st, int *ran) {
+  for (*ran = 0; *ran < nsteps;) {
+    const int k = std::min(kRunSteps, nsteps - *ran);
+    bool refused = false;
+    TRY(run_launch(ctxs, n, k, st, &refused));
+    if (refused) {
+      for (int i = 0; i < n; i++) ctxs[i]->run_on = false;
+      break;
+    }
+    *ran += k;
+  }
   return LBM_OK;
 }
 
@@ -1597,8 +1616,9 @@ lbm_status step_once(lbm_ctx *ctx) {
 // constants) is then not shared by any other step, and two lattices stepped in
 // turn on their own streams could not overlap (64^3 pair: 34 us against 30).
 lbm_status step_many(lbm_ctx *ctx, int nsteps) {
-  if (nsteps >= 2 && run_ok(ctx)) return run_steps(&ctx, 1, nsteps, ctx->st);
-  for (int k = 0; k < nsteps; k++) TRY(step_once(ctx));
+  int done = 0;
+  if (nsteps >= 2 && run_ok(ctx)) TRY(run_steps(&ctx, 1, nsteps, ctx->st, &done));
+  for (; done < nsteps; done++) TRY(step_once(ctx));
   return LBM_OK;
 }
 
@@ -1885,7 +1905,9 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
       return LBM_ERR_CUDA;
     }
   }
-  if (cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess)
+  int coop = 0;
+  if (cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device) != cudaSuccess || !coop)
     ctx->sms = 0;
   ctx->ssz = d.precision == LBM_FP64 ? 8 : d.precision == LBM_FP32 ? 4 : 2;
   ctx->tsz = d.precision == LBM_FP64 ? 8 : 4;
@@ -1910,6 +1932,8 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
     if (const char *e = getenv("LBM_GEOM_PREFETCH")) ctx->geom_prefetch = atoi(e) != 0;
     if (const char *e = getenv("LBM_VEC_PACKED")) ctx->bulk_vec_packed = atoi(e);
     if (const char *e = getenv("LBM_RUN")) ctx->run_on = atoi(e) != 0;
+    if (const char *e = getenv("LBM_RUN_SMS"))
+      if (ctx->sms > 0 && atoi(e) > 0) ctx->sms = atoi(e);
     if (const char *e = getenv("LBM_IBM_TABLES")) ctx->ibm_tables = atoi(e) != 0;
     if (const char *e = getenv("LBM_IBM_CLUSTER")) ctx->ibm_cluster_on = atoi(e) != 0;
     if (const char *e = getenv("LBM_MRT_GENERAL"))
@@ -2761,7 +2785,8 @@ bool graphable(const lbm_ctx *c) { return (!any_moving(c) || dev_motion(c)) && !
 // kind per launch.  Eight lattices of edges 24..64, alternately bounce-back and
 // IBM: 40.6 us per step (12.6 + 28.3 in two launches) against 45.9 as graph
 // replays; in one launch whose threads hold both kinds' constants 52.
-lbm_status batch_run(lbm_batch *b, int nsteps) {
+// ran: set for the lattices stepped here; the others are left to the graph.
+lbm_status batch_run(lbm_batch *b, int nsteps, std::vector<char> &ran) {
   const int n = (int)b->ctx.size();
   std::vector<char> done(n, 0);
   for (int i = 0; i < n; i++) {
@@ -2782,12 +2807,17 @@ lbm_status batch_run(lbm_batch *b, int nsteps) {
       BCK(cudaEventRecord(b->ev_done[idx[k]], grp[k]->st));
       BCK(cudaStreamWaitEvent(b->origin, b->ev_done[idx[k]], 0));
     }
-    const lbm_status s = run_steps(grp, m, nsteps, b->origin);
+    int steps = 0;
+    lbm_status s = run_steps(grp, m, nsteps, b->origin, &steps);
     if (s != LBM_OK) return bfail(b, s, lbm_last_error(grp[0]));
     BCK(cudaEventRecord(b->ev_origin, b->origin));
+    for (int k = 0; k < m; k++) BCK(cudaStreamWaitEvent(grp[k]->st, b->ev_origin, 0));
+    if (steps == 0) continue;
     for (int k = 0; k < m; k++) {
-      BCK(cudaStreamWaitEvent(grp[k]->st, b->ev_origin, 0));
+      for (int j = steps; j < nsteps; j++)
+        if ((s = step_once(grp[k])) != LBM_OK) return bfail(b, s, lbm_last_error(grp[k]));
       b->steps_done[idx[k]] += nsteps;
+      ran[idx[k]] = 1;
     }
     b->graph_launches++;
   }
@@ -2940,8 +2970,7 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
   // small lattices first, all their steps at once
   std::vector<char> ran(n, 0);
   if (nsteps >= 2) {
-    for (int i = 0; i < n; i++) ran[i] = b->active[i] && run_ok(b->ctx[i]);
-    const lbm_status s = batch_run(b, nsteps);
+    const lbm_status s = batch_run(b, nsteps, ran);
     if (s != LBM_OK) return s;
   }
   bool rest = false;

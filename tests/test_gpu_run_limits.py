@@ -120,3 +120,36 @@ def test_long_calls_run_in_launches_of_bounded_length(monkeypatch, scheme):
     assert np.array_equal(out[0][1], out[1][1])
     # FP64 sums of the same parts in another order
     assert np.abs(out[0][2] - out[1][2]).max() <= 1e-12 * max(1.0, np.abs(out[0][2]).max())
+
+
+@pytest.mark.parametrize("scheme", [W.BOUZIDI_QUAD, W.IBM])
+def test_refused_launch_steps_with_launches(monkeypatch, scheme):
+    """More blocks than the device holds at once (LBM_RUN_SMS above its SMs, as
+    on a stream with fewer SMs): the runtime refuses the cooperative launch on
+    the host, and the lattice steps with launches of its own, alone and in a
+    batch."""
+    from paper_1906_05445_gb300 import lbm
+    p = _disc(W.FP64, scheme=scheme).with_(nx=192, ny=190)
+    out = []
+    for run, sms in (("0", ""), ("1", "1200")):
+        monkeypatch.setenv("LBM_RUN", run)
+        if sms:
+            monkeypatch.setenv("LBM_RUN_SMS", sms)
+        lats = [lbm.Lattice.from_problem(p) for _ in range(2)]
+        for g in lats:
+            g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        b = lbm.Batch(lats, autotune=False)
+        b.step(6)
+        b.close()
+        lats[0].step(5)
+        n0 = lats[0].info().kernel_launches
+        lats[0].step(3)
+        assert lats[0].info().kernel_launches - n0 >= 6
+        out.append([(g.get_f(), g.force_torque(0)) for g in lats])
+        for g in lats:
+            g.sync()
+            g.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a[0], b[0])
+        for x, y in zip(a[1], b[1]):
+            assert np.abs(x - y).max() <= 1e-12 * max(1.0, np.abs(x).max())
