@@ -153,3 +153,55 @@ def test_refused_launch_steps_with_launches(monkeypatch, scheme):
         assert np.array_equal(a[0], b[0])
         for x, y in zip(a[1], b[1]):
             assert np.abs(x - y).max() <= 1e-12 * max(1.0, np.abs(x).max())
+
+
+SPHERE = [W.Solid(W.SPHERE, (8.3, 9.1, 7.7), 3.2, omega=(0.002, 0.0, -0.001))]
+ROUTES = [("0", ""), ("1", ""), ("1", "1"), ("1", "5"), ("1", "40")]
+
+
+def _routes(monkeypatch, lattice, shape, solids, precision, scheme, iters=1, density=1.0):
+    """Launches, and multi-step launches on one block (every boundary node and
+    marker of the lattice in turn), a few and many blocks (one group of boundary
+    nodes per block, one marker per warp)."""
+    from paper_1906_05445_gb300 import lbm
+    p = W.Problem("routes", lattice, *shape, 0.7, W.MRT, precision, (1e-4, -2e-4, 0.0), solids,
+                  scheme, 0, ibm_iters=iters, marker_density=density)
+    out = []
+    for run, sms in ROUTES:
+        monkeypatch.setenv("LBM_RUN", run)
+        if sms:
+            monkeypatch.setenv("LBM_RUN_SMS", sms)
+        g = lbm.Lattice.from_problem(p)
+        g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        g.step(1)
+        g.step(6)
+        out.append((g.get_f(), g.velocity(), g.force_history(0), g.solid_mask()))
+        g.sync()
+        g.close()
+    return out
+
+
+@pytest.mark.parametrize("precision", [W.FP64, W.FP32, W.FP32_BF16, W.FP32_FP16])
+@pytest.mark.parametrize("scheme", [W.BOUZIDI_QUAD, W.ZHAO_YONG])
+@pytest.mark.parametrize("lattice,shape,solids", [(W.D3Q19, (20, 17, 16), SPHERE),
+                                                  (W.D2Q9, (33, 32, 1), DISC)])
+def test_blocks_of_a_launch_do_not_show(monkeypatch, lattice, shape, solids, precision, scheme):
+    a, *rest = _routes(monkeypatch, lattice, shape, solids, precision, scheme)
+    for b in rest:
+        assert np.array_equal(a[0], b[0])
+        # FP64 sums of the same parts in another order
+        assert np.abs(a[2] - b[2]).max() <= 1e-12 * max(1.0, np.abs(a[2]).max())
+
+
+@pytest.mark.parametrize("precision,tol", [(W.FP64, 1e-13), (W.FP32, 2e-6)])
+@pytest.mark.parametrize("iters,density", [(1, 1.0), (5, 1.0), (2, 5.0)])
+@pytest.mark.parametrize("lattice,shape,solids", [(W.D3Q19, (20, 17, 16), SPHERE),
+                                                  (W.D2Q9, (33, 32, 1), DISC)])
+def test_blocks_of_an_ibm_launch(monkeypatch, lattice, shape, solids, precision, tol, iters,
+                                 density):
+    """At density 5 a node's row holds more markers than its group has threads
+    for.  The same sums in another order, a few hundred roundings deep."""
+    a, *rest = _routes(monkeypatch, lattice, shape, solids, precision, W.IBM, iters, density)
+    for b in rest:
+        assert rel_l2(b[1], a[1], a[3]) <= tol
+        assert np.abs(a[2] - b[2]).max() <= 20 * tol * np.abs(a[2]).max()
