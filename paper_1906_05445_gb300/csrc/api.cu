@@ -96,6 +96,29 @@ const double PI = 3.14159265358979323846;
 
 }  // namespace
 
+namespace {
+
+// The stepping calls (lbm_step, lbm_run_to_steady, lbm_step_multi) of the
+// process's lattices, in order.  Lattices stepped in turn on streams of their
+// own, by one thread or several, run side by side, and a multi-step launch holds
+// its SMs to its end: each lattice then takes a share of them (run_share).
+struct StepMark {
+  int device = -1;
+  cudaStream_t st = nullptr;
+  unsigned long long last = 0;  // the clock at the last stepping call
+};
+struct StepMarks {
+  std::mutex mu;
+  std::vector<StepMark *> live;  // of every context
+  unsigned long long clock = 0;
+};
+StepMarks &step_marks() {
+  static StepMarks *m = new StepMarks;  // contexts may outlive static objects
+  return *m;
+}
+
+}  // namespace
+
 struct lbm_ctx {
   lbm_lattice_desc d;
   int Q = 0, D = 0;
@@ -216,7 +239,8 @@ struct lbm_ctx {
   double *hist = nullptr;
   unsigned *run_bar = nullptr;  // k_run's barrier counters (zero between launches)
   int zero_slot = -1;           // the record a k_run launch left zeroed for the step after it
-  bool run_on = true;           // LBM_RUN=0: every step as launches of its own
+  bool run_on = true;           // LBM_RUN=0, or refused: every step as launches of its own
+  StepMark mark;
   int sms = 0;                  // blocks of a k_run launch at most: the SMs, or LBM_RUN_SMS
   int slot = 0;
   long long records = 0;
@@ -944,7 +968,7 @@ lbm_status tab_alloc(lbm_ctx *ctx, void **p, size_t bytes) {
   return LBM_OK;
 }
 
-bool run_small(const lbm_ctx *ctx);
+bool run_small(const lbm_ctx *ctx, int share);
 
 // The row and coupling tables of IBM solids at rest, after the geometry and
 // the stencils are built: for lattices whose steps k_run takes, and for the
@@ -957,7 +981,7 @@ lbm_status build_tables(lbm_ctx *ctx) {
   const bool small = ctx->d.nx < 8 || ctx->d.ny < 8 || (ctx->D == 3 && ctx->d.nz < 8);
   if (ctx->scheme.scheme != LBM_IBM_DIRECT || ctx->nmark == 0 || any_moving(ctx) || small ||
       ctx->list_count <= 0 || ctx->ibm_cluster_on || !ctx->ibm_tables ||
-      (ctx->scheme.ibm_iters <= 1 && !run_small(ctx)))
+      (ctx->scheme.ibm_iters <= 1 && !run_small(ctx, 1)))
     return LBM_OK;
   const int nm = ctx->nmark, nl = ctx->list_count;
   const bool iterate = ctx->scheme.ibm_iters > 1;
@@ -1467,17 +1491,40 @@ lbm_status step_end(lbm_ctx *ctx, const StepState &ss) {
 
 // ---- several steps in one launch (run_impl.cuh)
 
-bool run_small(const lbm_ctx *ctx);
+bool run_small(const lbm_ctx *ctx, int share);
 
-// Whether a lattice's steps can run in k_run: solids at rest (IBM: with
-// tables), a periodic box, the default kernels, untimed, and small enough
-// that launches and phase latencies, not bandwidth, set its step.
-bool run_ok(const lbm_ctx *ctx) {
+// Whether a lattice's steps can run in k_run, on one of `share` parts of the SMs:
+// solids at rest (IBM: with tables), a periodic box, the default kernels,
+// untimed, and small enough that launches and phase latencies, not bandwidth,
+// set its step.
+bool run_ok(const lbm_ctx *ctx, int share) {
   const bool ibm = ctx->scheme.scheme == LBM_IBM_DIRECT && ctx->nmark > 0;
-  return ctx->run_on && ctx->sms > 0 && run_small(ctx) && !any_moving(ctx) && !ctx->nface &&
-         ctx->timing == 0 && ctx->coll_mode != CM_MRT && ctx->bulk_mode == 1 &&
+  return ctx->run_on && ctx->sms >= share && run_small(ctx, share) && !any_moving(ctx) &&
+         !ctx->nface && ctx->timing == 0 && ctx->coll_mode != CM_MRT && ctx->bulk_mode == 1 &&
          (ctx->bulk_vec_words == 0 || ctx->bulk_vec_words == 2) && ctx->bulk_vec_packed < 0 &&
          ctx->cache_hints == 0 && (!ibm || ctx->tab.nmark > 0);
+}
+
+// Marks a stepping call of the lattice and returns the number of streams that
+// step side by side: its own, and every other one on the device that stepped
+// since this lattice's last call.  Only the time of a step depends on it.
+// us per step of all, two / four lattices on streams of their own, 20 steps a call:
+// with all SMs for each (one after the other), with shares, as launches:
+//   FP32 64^3 bounce-back 18.8 / 37.8, 14.6 / 24.2 (launches), 16.8 / 24.2;
+//   FP32 64^3 IBM 32.0 / 64.5, 25.8 / 39.8 (launches), 27.0 / 39.8;
+//   FP32 80^3 IBM, 5 passes 75 / 147, 54 / 97 (launches), 61 / 97;
+//   301^2 FP32 10.6 / 21.1, 6.4 / 8.2, 12.8 / 23.9; 64^2 FP64 17.8 / 35.4, 11.9 / 12.1, 15.2 / 23.8.
+int run_share(lbm_ctx *ctx) {
+  StepMarks &m = step_marks();
+  std::lock_guard<std::mutex> lk(m.mu);
+  std::vector<cudaStream_t> others;
+  for (const StepMark *o : m.live)
+    if (o->device == ctx->device && o->st != ctx->st && o->last > ctx->mark.last &&
+        std::find(others.begin(), others.end(), o->st) == others.end())
+      others.push_back(o->st);
+  ctx->mark.st = ctx->st;
+  ctx->mark.last = ++m.clock;
+  return 1 + (int)others.size();
 }
 
 // nodes per vector of the 2-word kernels, 0 where the one-node update runs
@@ -1497,20 +1544,25 @@ bool run_vec(const lbm_ctx *ctx) {
 //   FP16 bounce-back  80^3 11.0 / 14.4, 88^3 14.2 / 14.2; IBM 72^3 22.1 / 22.7
 //   FP64 bounce-back  48^3 41.9 / 51.9, 56^3 60.8 / 59.7; 512^2 34.4 / 41.1
 //   FP64 IBM, 1       32^3 27.7 / 30.9, 41^3 38.2 / 37.2; 5: 48^3 67 / 79, 64^3 110 / 111
-// Beyond, the one block per SM keeps too few loads in flight for the sweep.
-bool run_small(const lbm_ctx *ctx) {
+// Beyond, the one block per SM keeps too few loads in flight for the sweep.  On
+// a share of the SMs the limits shrink with it (half the SMs: 64^3 bounce-back
+// 14.2 / 14.7, 72^3 17.7 / 15.7; IBM 40^3 13.2 / 20.3, 56^3 21.2 / 20.7; five passes
+// 80^3 44.0 / 46.8; a quarter: 40^3 9.2 / 10.9, 48^3 12.4 / 11.6).
+bool run_small(const lbm_ctx *ctx, int share) {
   const bool f64 = ctx->d.precision == LBM_FP64;
-  const long long v = ctx->N * ctx->Q;
+  const long long v = ctx->N * ctx->Q * share;
   if (ctx->scheme.scheme != LBM_IBM_DIRECT || ctx->nmark == 0) return v <= (f64 ? 2400000 : 10000000);
   if (ctx->scheme.ibm_iters <= 1) return v <= (f64 ? 700000 : 7200000);
   return v <= (f64 ? 2400000 : 17000000);
 }
 
-// One launch of k_run: nsteps steps of the lattices in `ctxs` on `st`.
+// One launch of k_run: nsteps steps of the lattices in `ctxs` on `st`, on one of
+// `share` parts of the SMs.
 // *refused: the blocks do not fit beside each other on the SMs that the stream
 // may use (a green context, a limited client), or cooperative launches are not
 // supported there; nothing was stepped.
-lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st, bool *refused) {
+lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaStream_t st,
+                      bool *refused) {
   lbm_ctx *ctx = ctxs[0];
   RunArgs<kMaxRun> g;
   memset(&g, 0, sizeof(g));
@@ -1532,9 +1584,10 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st, 
     const int V = !vec ? 1 : c->d.precision == LBM_FP32 ? 2 : 4;
     // no more blocks than warps of nodes and groups of boundary nodes
     const long long warps = (c->N / V + 31) / 32 + std::max(0, c->list_count) / 16;
-    const long long share =
-        n == 1 ? c->sms : std::max<long long>(4, (long long)(w[k] / sum * (c->sms - 4 * n)) + 4);
-    const int nb = (int)std::max<long long>(1, std::min(share, warps));
+    const int sms = c->sms / share;
+    const long long most =
+        n == 1 ? sms : std::max<long long>(4, (long long)(w[k] / sum * (sms - 4 * n)) + 4);
+    const int nb = (int)std::max<long long>(1, std::min(most, warps));
     g.block_start[k] = at;
     at += nb;
     RunLat &r = g.l[k];
@@ -1591,11 +1644,11 @@ constexpr int kRunSteps = 256;
 // follows their own streams' earlier work and precedes their later work (the
 // caller's order).  *ran: the steps done; fewer than nsteps where a launch was
 // refused, and these lattices then step with launches of their own.
-lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, cudaStream_t st, int *ran) {
+lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaStream_t st, int *ran) {
   for (*ran = 0; *ran < nsteps;) {
     const int k = std::min(kRunSteps, nsteps - *ran);
     bool refused = false;
-    TRY(run_launch(ctxs, n, k, st, &refused));
+    TRY(run_launch(ctxs, n, k, share, st, &refused));
     if (refused) {
       for (int i = 0; i < n; i++) ctxs[i]->run_on = false;
       break;
@@ -1617,7 +1670,8 @@ lbm_status step_once(lbm_ctx *ctx) {
 // turn on their own streams could not overlap (64^3 pair: 34 us against 30).
 lbm_status step_many(lbm_ctx *ctx, int nsteps) {
   int done = 0;
-  if (nsteps >= 2 && run_ok(ctx)) TRY(run_steps(&ctx, 1, nsteps, ctx->st, &done));
+  const int share = run_share(ctx);
+  if (nsteps >= 2 && run_ok(ctx, share)) TRY(run_steps(&ctx, 1, nsteps, share, ctx->st, &done));
   for (; done < nsteps; done++) TRY(step_once(ctx));
   return LBM_OK;
 }
@@ -1889,6 +1943,12 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
     return LBM_ERR_CUDA;
   }
   {
+    StepMarks &m = step_marks();
+    std::lock_guard<std::mutex> lk(m.mu);
+    ctx->mark = {ctx->device, ctx->st, m.clock};
+    m.live.push_back(&ctx->mark);
+  }
+  {
     int lo = 0, hi = 0;
     cudaDeviceGetStreamPriorityRange(&lo, &hi);
     // high priority: the boundary and IBM kernels start with the bulk sweep
@@ -1977,6 +2037,11 @@ lbm_status lbm_create(lbm_ctx **out, const lbm_lattice_desc *desc, void *cuda_st
 
 void lbm_destroy(lbm_ctx *ctx) {
   if (!ctx) return;
+  {
+    StepMarks &m = step_marks();
+    std::lock_guard<std::mutex> lk(m.mu);
+    m.live.erase(std::remove(m.live.begin(), m.live.end(), &ctx->mark), m.live.end());
+  }
   cudaStreamSynchronize(ctx->st);
   if (ctx->aux) {
     cudaStreamSynchronize(ctx->aux);
@@ -2195,6 +2260,7 @@ lbm_status lbm_step_multi(lbm_ctx *const *ctxs, int n, int nsteps) {
       if (ctxs[j] == ctxs[i]) return fail(ctxs[i], LBM_ERR_ARG, "a lattice appears twice");
   }
   for (int i = 0; i < n; i++) TRY(prepare(ctxs[i]));
+  for (int i = 0; i < n; i++) run_share(ctxs[i]);
   // lattices that can share a bulk launch: same lattice, collision and storage
   std::vector<std::vector<int>> groups;
   for (int i = 0; i < n; i++) {
@@ -2777,7 +2843,7 @@ void drop_graph(lbm_batch *b) {
 // with a prescribed motion move on the host, which prefetches their next
 // geometry: those lattices step directly.
 // Small lattices run their steps in k_run, outside the graph.
-bool graphable(const lbm_ctx *c) { return (!any_moving(c) || dev_motion(c)) && !run_ok(c); }
+bool graphable(const lbm_ctx *c) { return (!any_moving(c) || dev_motion(c)) && !run_ok(c, 1); }
 
 // All nsteps of the active lattices that k_run takes, up to kMaxRun of one
 // kind per launch.  Eight lattices of edges 24..64, alternately bounce-back and
@@ -2788,12 +2854,12 @@ lbm_status batch_run(lbm_batch *b, int nsteps, std::vector<char> &ran) {
   const int n = (int)b->ctx.size();
   std::vector<char> done(n, 0);
   for (int i = 0; i < n; i++) {
-    if (!b->active[i] || done[i] || !run_ok(b->ctx[i])) continue;
+    if (!b->active[i] || done[i] || !run_ok(b->ctx[i], 1)) continue;
     lbm_ctx *grp[kMaxRun];
     int idx[kMaxRun], m = 0;
     for (int j = i; j < n && m < kMaxRun; j++) {
       const lbm_ctx *c = b->ctx[j], *c0 = b->ctx[i];
-      if (!b->active[j] || done[j] || !run_ok(c) || c->d.lattice != c0->d.lattice ||
+      if (!b->active[j] || done[j] || !run_ok(c, 1) || c->d.lattice != c0->d.lattice ||
           c->coll_mode != c0->coll_mode || c->d.precision != c0->d.precision ||
           (c->tab.nmark > 0) != (c0->tab.nmark > 0))
         continue;
@@ -2806,7 +2872,7 @@ lbm_status batch_run(lbm_batch *b, int nsteps, std::vector<char> &ran) {
       BCK(cudaStreamWaitEvent(b->origin, b->ev_done[idx[k]], 0));
     }
     int steps = 0;
-    lbm_status s = run_steps(grp, m, nsteps, b->origin, &steps);
+    lbm_status s = run_steps(grp, m, nsteps, 1, b->origin, &steps);
     if (s != LBM_OK) return bfail(b, s, lbm_last_error(grp[0]));
     BCK(cudaEventRecord(b->ev_origin, b->origin));
     for (int k = 0; k < m; k++) BCK(cudaStreamWaitEvent(grp[k]->st, b->ev_origin, 0));

@@ -205,3 +205,42 @@ def test_blocks_of_an_ibm_launch(monkeypatch, lattice, shape, solids, precision,
     for b in rest:
         assert rel_l2(b[1], a[1], a[3]) <= tol
         assert np.abs(a[2] - b[2]).max() <= 20 * tol * np.abs(a[2]).max()
+
+
+def test_lattices_on_streams_of_their_own_share_the_sms(monkeypatch):
+    """Stepped in turn, lattices on streams of their own take a share of the SMs
+    each, and launches of their own where the share is too small for them; one
+    stepped alone has them all again.  The fields do not depend on it."""
+    import torch
+    from paper_1906_05445_gb300 import lbm
+    p = W.Problem("share", W.D3Q19, 36, 36, 36, 0.7, W.MRT, W.FP64, (1e-4, -2e-4, 0.0), SPHERE,
+                  W.BOUZIDI_QUAD, 0)
+    monkeypatch.setenv("LBM_RUN", "0")
+    ref = lbm.Lattice.from_problem(p)
+    ref.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+    ref.step(16)
+    monkeypatch.setenv("LBM_RUN", "1")
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    lats = [lbm.Lattice.from_problem(p, stream=s.cuda_stream) for s in streams]
+
+    def launches(g, k):
+        n0 = g.info().kernel_launches
+        g.step(k)
+        return g.info().kernel_launches - n0
+
+    for g in lats:
+        g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        g.step(1)
+    assert all(launches(g, 3) > 1 for g in lats)  # a third of the SMs each
+    assert launches(lats[0], 2) > 1               # the others stepped since
+    assert launches(lats[0], 2) == 1              # alone
+    assert launches(lats[1], 2) > 1               # after both others
+    assert launches(lats[0], 2) == 1              # beside one other: half
+    assert launches(lats[1], 2) == 1
+    lats[0].step(6)
+    lats[1].step(8)
+    lats[2].step(12)
+    for g in lats:
+        assert np.array_equal(g.get_f(), ref.get_f())
+        g.close()
+    ref.close()
