@@ -426,11 +426,13 @@ const char *lbm_last_error(const lbm_ctx *ctx);
  * cuda_stream: lbm_batch_step and lbm_batch_run_to_steady start after the
  * work already queued there, and work queued there afterwards (an event, a
  * copy) waits for them; the contexts' queries wait for them as well.
- * Stepping captures one step pair of every lattice with static solids into
- * a CUDA graph whose per-lattice chains are independent branches, and
- * replays it: two steps of the whole batch per launch.  Lattices with
- * moving solids step directly.  Under graph replay the force history keeps
- * only the last two records per lattice (lbm_get_force_torque is exact).
+ * Stepping captures one step pair of every lattice with static solids (or
+ * free ones) into a CUDA graph whose per-lattice chains are independent
+ * branches, and replays it: two steps of the whole batch per launch.
+ * Lattices whose solids have a prescribed motion step directly.  Under graph
+ * replay the force history keeps only the last two records per lattice
+ * (lbm_get_force_torque is exact).  Where every lattice is small, the steps of
+ * a call run in multi-step launches instead, if that is estimated faster.
  * lbm_batch_run_to_steady runs every lattice to its own residual < tol
  * (checked every check_every steps, as lbm_run_to_steady), drops converged
  * lattices from the graph, and reports steps_done[i] and residual[i]. */

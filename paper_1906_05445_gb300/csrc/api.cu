@@ -1556,6 +1556,23 @@ bool run_small(const lbm_ctx *ctx, int share) {
   return v <= (f64 ? 2400000 : 17000000);
 }
 
+// Blocks of each of n lattices in one launch: in proportion to the nodes, at least
+// four each, one per SM in all, and no more than a lattice has warps of nodes and
+// groups of boundary nodes.
+void run_blocks(lbm_ctx *const *ctxs, int n, int share, int *nb) {
+  double sum = 0;
+  for (int k = 0; k < n; k++) sum += (double)ctxs[k]->N * ctxs[k]->Q;
+  for (int k = 0; k < n; k++) {
+    const lbm_ctx *c = ctxs[k];
+    const int V = !run_vec(c) ? 1 : c->d.precision == LBM_FP32 ? 2 : 4;
+    const long long warps = (c->N / V + 31) / 32 + std::max(0, c->list_count) / 16;
+    const int sms = c->sms / share;
+    const long long most =
+        n == 1 ? sms : std::max<long long>(4, (long long)((double)c->N * c->Q / sum * (sms - 4 * n)) + 4);
+    nb[k] = (int)std::max<long long>(1, std::min(most, warps));
+  }
+}
+
 // One launch of k_run: nsteps steps of the lattices in `ctxs` on `st`, on one of
 // `share` parts of the SMs.
 // *refused: the blocks do not fit beside each other on the SMs that the stream
@@ -1567,29 +1584,15 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaSt
   RunArgs<kMaxRun> g;
   memset(&g, 0, sizeof(g));
   g.n = n;
-  // blocks in proportion to the nodes, at least four each, one per SM in all
-  double w[kMaxRun], sum = 0;
-  for (int k = 0; k < n; k++) {
-    const lbm_ctx *c = ctxs[k];
-    w[k] = (double)c->N * c->Q;
-    sum += w[k];
-  }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   CK(cudaStreamIsCapturing(st, &cap));
   const bool capturing = cap != cudaStreamCaptureStatusNone;
-  int at = 0;
+  int at = 0, blocks[kMaxRun];
+  run_blocks(ctxs, n, share, blocks);
   for (int k = 0; k < n; k++) {
     lbm_ctx *c = ctxs[k];
-    const bool vec = run_vec(c);
-    const int V = !vec ? 1 : c->d.precision == LBM_FP32 ? 2 : 4;
-    // no more blocks than warps of nodes and groups of boundary nodes
-    const long long warps = (c->N / V + 31) / 32 + std::max(0, c->list_count) / 16;
-    const int sms = c->sms / share;
-    const long long most =
-        n == 1 ? sms : std::max<long long>(4, (long long)(w[k] / sum * (sms - 4 * n)) + 4);
-    const int nb = (int)std::max<long long>(1, std::min(most, warps));
     g.block_start[k] = at;
-    at += nb;
+    at += blocks[k];
     RunLat &r = g.l[k];
     r.a = base_args(c);
     r.f[0] = c->f[0];
@@ -1601,7 +1604,7 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaSt
     r.hist = c->hist;
     r.bar = c->run_bar;
     r.iters = std::max(1, c->scheme.ibm_iters);
-    r.vec = vec ? 1 : 0;
+    r.vec = run_vec(c) ? 1 : 0;
     const int first = (c->slot + 1) % kHistSlots;
     // the record the launch starts with: left zeroed by the launch before
     // (never relied on in a capture, whose replays find their own sums there)
@@ -2842,48 +2845,112 @@ void drop_graph(lbm_batch *b) {
 // solids, or solids that move on the device (a free solid present).  Solids
 // with a prescribed motion move on the host, which prefetches their next
 // geometry: those lattices step directly.
-// Small lattices run their steps in k_run, outside the graph.
-bool graphable(const lbm_ctx *c) { return (!any_moving(c) || dev_motion(c)) && !run_ok(c, 1); }
+bool graphable(const lbm_ctx *c) { return !any_moving(c) || dev_motion(c); }
 
-// All nsteps of the active lattices that k_run takes, up to kMaxRun of one
-// kind per launch.  Eight lattices of edges 24..64, alternately bounce-back and
-// IBM: 40.6 us per step (12.6 + 28.3 in two launches) against 45.9 as graph
-// replays; in one launch whose threads hold both kinds' constants 52.
-// ran: set for the lattices stepped here; the others are left to the graph.
-lbm_status batch_run(lbm_batch *b, int nsteps, std::vector<char> &ran) {
+// Launches of k_run for the active lattices of a batch: up to kMaxRun of one kind
+// each, one launch after the other.  Empty where a lattice does not run in it.
+std::vector<std::vector<int>> run_groups(const lbm_batch *b) {
   const int n = (int)b->ctx.size();
-  std::vector<char> done(n, 0);
+  std::vector<std::vector<int>> out;
   for (int i = 0; i < n; i++) {
-    if (!b->active[i] || done[i] || !run_ok(b->ctx[i], 1)) continue;
-    lbm_ctx *grp[kMaxRun];
-    int idx[kMaxRun], m = 0;
-    for (int j = i; j < n && m < kMaxRun; j++) {
-      const lbm_ctx *c = b->ctx[j], *c0 = b->ctx[i];
-      if (!b->active[j] || done[j] || !run_ok(c, 1) || c->d.lattice != c0->d.lattice ||
-          c->coll_mode != c0->coll_mode || c->d.precision != c0->d.precision ||
-          (c->tab.nmark > 0) != (c0->tab.nmark > 0))
-        continue;
-      grp[m] = b->ctx[j];
-      idx[m++] = j;
-      done[j] = 1;
+    if (!b->active[i]) continue;
+    const lbm_ctx *c = b->ctx[i];
+    if (!run_ok(c, 1)) return {};
+    bool placed = false;
+    for (auto &g : out) {
+      const lbm_ctx *o = b->ctx[g[0]];
+      if ((int)g.size() < kMaxRun && c->d.lattice == o->d.lattice && c->coll_mode == o->coll_mode &&
+          c->d.precision == o->d.precision && (c->tab.nmark > 0) == (o->tab.nmark > 0)) {
+        g.push_back(i);
+        placed = true;
+        break;
+      }
     }
+    if (!placed) out.push_back({i});
+  }
+  return out;
+}
+
+// Whether a batch's steps run in k_run or as graph replays, from estimates of the
+// us per step of both.  k_run's launches follow each other and hold the SMs, so a
+// lattice outside it (large, or moving) would wait for them: such batches are all
+// graph (128^3 with a 64^3 IBM lattice 60.8 us per step against 68.3).  A replay
+// steps all lattices side by side at about 4 us of launches each.  Measured, k_run
+// / graph, n lattices of one kind, then grid-convergence batches (edges 24 ...,
+// alternately bounce-back and IBM):
+//   FP32 bounce-back  8 x 24^3 6.6 / 34.6, 8 x 48^3 27.6 / 45.0, 8 x 56^3 48.9 / 45.9;
+//                     2 x 56^3 11.9 / 14.7, 4 x 64^3 32.4 / 30.4
+//   FP32 IBM, 1 pass  4 x 40^3 20.4 / 22.3, 4 x 56^3 32.7 / 28.4, 2 x 48^3 19.9 / 17.6
+//   FP32 IBM, 5       8 x 48^3 50.0 / 63.6, 8 x 56^3 81.4 / 75.4
+//   FP64 bounce-back  8 x 32^3 84.6 / 87.4, 64^2 9.2 / 13.6, 8 x 64^2 13.3 / 40.2
+//   FP64 IBM          4 x 32^3 80.5 / 53.6 (1 pass), 8 x 24^3 112 / 72 (5): graph
+//   convergence       5 (24-56) 31.8 / 27.9, 8 (24-64) 42.8 / 52.6, 10 53.3 / 65.4
+// The estimates are fits to 114 such batches; p counts populations in millions, an
+// FP64 one as 11.
+double run_us(const lbm_batch *b, const std::vector<int> &group) {
+  const int n = (int)group.size();
+  lbm_ctx *c[kMaxRun];
+  int nb[kMaxRun], iters = 1;
+  for (int k = 0; k < n; k++) c[k] = b->ctx[group[k]];
+  run_blocks(c, n, 1, nb);
+  const bool f64 = c[0]->d.precision == LBM_FP64, ibm = c[0]->tab.nmark > 0;
+  double p = 0;
+  bool groups = false, rounds = false;  // more boundary-node groups / markers than at once
+  for (int k = 0; k < n; k++) {
+    p += 1e-6 * c[k]->N * c[k]->Q * (f64 ? 11 : 1);
+    groups |= c[k]->list_count > (long long)nb[k] * (kRunBlock / c[k]->Q);
+    rounds |= c[k]->tab.nmark > nb[k] * (kRunBlock / 32);
+    iters = std::max(iters, c[k]->scheme.ibm_iters);
+  }
+  const double over = std::max(0.0, p - 10);
+  if (f64) return ibm ? INFINITY : 12 + 1.25 * p;
+  if (!ibm) return 4.2 + 1.25 * p + 0.6 * over + (groups ? 7 : 0);
+  return 12.3 + 2.1 * (iters - 1) + 0.9 * std::max(0.0, p - 2) + 0.8 * over + (groups ? 6.5 : 0) +
+         (rounds ? 2.5 * iters : 0);
+}
+double graph_us(const lbm_batch *b) {
+  double p = 0;
+  int n = 0, iters = 1;
+  bool f64 = false, ibm = false;
+  for (size_t i = 0; i < b->ctx.size(); i++) {
+    if (!b->active[i]) continue;
+    const lbm_ctx *c = b->ctx[i];
+    n++;
+    p += 1e-6 * c->N * c->Q * (c->d.precision == LBM_FP64 ? 11 : 1);
+    f64 |= c->d.precision == LBM_FP64;
+    if (c->tab.nmark > 0) {
+      ibm = true;
+      iters = std::max(iters, c->scheme.ibm_iters);
+    }
+  }
+  const double launches = (ibm ? 5 : 3) + 4.1 * std::min(n, 5) + 5.5 * std::max(0, n - 5);
+  const double work = (f64 ? 14 : ibm ? 10 : 6) + (ibm ? 1.45 : 1.3) * p;
+  return std::max({(ibm ? 12.0 : 8.0) + 2 * n, launches, work}) + 2.9 * (iters - 1);
+}
+
+// All nsteps of a batch in k_run.  In one launch whose threads hold both kinds'
+// constants, eight lattices of edges 24..64 took 52 us per step (12.6 + 28.3 in two).
+lbm_status batch_run(lbm_batch *b, const std::vector<std::vector<int>> &groups, int nsteps) {
+  for (const auto &g : groups) {
+    const int m = (int)g.size();
+    lbm_ctx *grp[kMaxRun];
     for (int k = 0; k < m; k++) {
-      BCK(cudaEventRecord(b->ev_done[idx[k]], grp[k]->st));
-      BCK(cudaStreamWaitEvent(b->origin, b->ev_done[idx[k]], 0));
+      grp[k] = b->ctx[g[k]];
+      BCK(cudaEventRecord(b->ev_done[g[k]], grp[k]->st));
+      BCK(cudaStreamWaitEvent(b->origin, b->ev_done[g[k]], 0));
     }
     int steps = 0;
     lbm_status s = run_steps(grp, m, nsteps, 1, b->origin, &steps);
     if (s != LBM_OK) return bfail(b, s, lbm_last_error(grp[0]));
     BCK(cudaEventRecord(b->ev_origin, b->origin));
-    for (int k = 0; k < m; k++) BCK(cudaStreamWaitEvent(grp[k]->st, b->ev_origin, 0));
-    if (steps == 0) continue;
     for (int k = 0; k < m; k++) {
+      BCK(cudaStreamWaitEvent(grp[k]->st, b->ev_origin, 0));
+      // refused: with launches, here; the next call takes the graph
       for (int j = steps; j < nsteps; j++)
         if ((s = step_once(grp[k])) != LBM_OK) return bfail(b, s, lbm_last_error(grp[k]));
-      b->steps_done[idx[k]] += nsteps;
-      ran[idx[k]] = 1;
+      b->steps_done[g[k]] += nsteps;
     }
-    b->graph_launches++;
+    if (steps > 0) b->graph_launches++;
   }
   return LBM_OK;
 }
@@ -3031,15 +3098,13 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
       lbm_status s = prepare(b->ctx[i]);
       if (s != LBM_OK) return bfail(b, s, lbm_last_error(b->ctx[i]));
     }
-  // small lattices first, all their steps at once
-  std::vector<char> ran(n, 0);
   if (nsteps >= 2) {
-    const lbm_status s = batch_run(b, nsteps, ran);
-    if (s != LBM_OK) return s;
+    const auto groups = run_groups(b);
+    double us = 0;
+    for (const auto &g : groups) us += run_us(b, g);
+    if (!groups.empty() && us <= graph_us(b)) return batch_run(b, groups, nsteps);
   }
-  bool rest = false;
-  for (int i = 0; i < n; i++) rest |= b->active[i] && !ran[i];
-  int done = rest ? 0 : nsteps;
+  int done = 0;
   while (done < nsteps) {
     const bool pair = nsteps - done >= 2;
     bool any_static = false;
@@ -3068,7 +3133,7 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
       }
       // lattices outside the graph (solids with a prescribed motion) step directly
       for (int i = 0; i < n; i++) {
-        if (!b->active[i] || b->in_graph[i] || ran[i]) continue;
+        if (!b->active[i] || b->in_graph[i]) continue;
         for (int k = 0; k < 2; k++) {
           lbm_status s = step_once(b->ctx[i]);
           if (s != LBM_OK) return bfail(b, s, lbm_last_error(b->ctx[i]));
@@ -3078,7 +3143,7 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
       done += 2;
     } else {
       for (int i = 0; i < n; i++) {
-        if (!b->active[i] || ran[i]) continue;
+        if (!b->active[i]) continue;
         lbm_status s = step_once(b->ctx[i]);
         if (s != LBM_OK) return bfail(b, s, lbm_last_error(b->ctx[i]));
         b->steps_done[i] += 1;

@@ -185,6 +185,7 @@ bool launch_bulk_group(const KArgs *as, int n, int lattice, int collision, int p
 // Many steps of small lattices in one launch (run_impl.cuh): lattice k runs on
 // blocks block_start[k] .. block_start[k + 1] - 1.
 constexpr int kMaxRun = 8;
+constexpr int kRunBlock = 512;  // threads per block
 struct RunLat {
   KArgs a;         // src, dst and force_acc are set per step from the fields below
   void *f[2];      // the two distribution arrays

@@ -56,8 +56,6 @@ __device__ __forceinline__ bool run_wait(unsigned *ctr, unsigned target, int *er
   return *ok != 0;
 }
 
-constexpr int kRunBlock = 512;
-
 // What a thread of a boundary-node group reads again every step: its node,
 // direction and cut link do not change while the solids rest, so the record
 // stays in registers and a step's populations are one memory latency away.

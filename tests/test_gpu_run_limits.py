@@ -244,3 +244,30 @@ def test_lattices_on_streams_of_their_own_share_the_sms(monkeypatch):
         assert np.array_equal(g.get_f(), ref.get_f())
         g.close()
     ref.close()
+
+
+def test_batch_takes_one_route_for_all(monkeypatch):
+    """A batch of small lattices runs in multi-step launches; with a lattice among
+    them that does not (here: a moving solid), all step by graph replays or
+    launches.  Both give the populations of the lattices stepped alone."""
+    from paper_1906_05445_gb300 import lbm
+    monkeypatch.setenv("LBM_RUN", "1")
+    small = [W.Problem("b", W.D3Q19, n, 17, 16, 0.7, W.MRT, W.FP32, (1e-4, -2e-4, 0.0), SPHERE,
+                       W.BOUZIDI_QUAD, 0) for n in (20, 24, 31)]
+    moving = W.translating_sphere(36, 20, 20, 4.3, seed=23, u=0.05, tau=0.7,
+                                  scheme=W.BOUZIDI_QUAD, precision=W.FP32)
+    for extra, launches in (([], [1, 2]), ([moving], [4, 7])):
+        alone = [lbm.Lattice.from_problem(p) for p in small + extra]
+        mixed = [lbm.Lattice.from_problem(p) for p in small + extra]
+        b = lbm.Batch(mixed, autotune=False)
+        for k, n in zip((9, 6), launches):
+            b.step(k)
+            for g in alone:
+                g.step(k)
+            assert b.info(0)[2] == n
+        for a, m in zip(alone, mixed):
+            assert np.array_equal(a.get_f(), m.get_f())
+            assert m.info().steps == 15
+        b.close()
+        for g in alone + mixed:
+            g.close()
