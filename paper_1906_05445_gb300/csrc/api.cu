@@ -241,6 +241,7 @@ struct lbm_ctx {
   int zero_slot = -1;           // the record a k_run launch left zeroed for the step after it
   bool run_on = true;           // LBM_RUN=0, or refused: every step as launches of its own
   StepMark mark;
+  long long beside = 0;  // bytes of the populations of lattices stepping beside this one
   int sms = 0;                  // blocks of a k_run launch at most: the SMs, or LBM_RUN_SMS
   int slot = 0;
   long long records = 0;
@@ -422,6 +423,7 @@ KArgs base_args(lbm_ctx *ctx) {
   a.bulk_mode = ctx->bulk_mode;
   a.bulk_vec_words = ctx->bulk_vec_words;
   a.bulk_vec_packed = ctx->bulk_vec_packed;
+  a.beside = ctx->beside;
   a.ibm = ctx->scheme.scheme == LBM_IBM_DIRECT ? 1 : 0;
   a.tab = ctx->tab;
   a.zy_pre = ctx->scheme.scheme == LBM_ZHAO_YONG ? ctx->zy_pre : nullptr;
@@ -1661,6 +1663,9 @@ lbm_status run_steps(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaStr
   return LBM_OK;
 }
 
+// bytes of a lattice's two population arrays
+long long pop_bytes(const lbm_ctx *ctx) { return 2LL * ctx->Q * ctx->fs * (long long)ctx->ssz; }
+
 lbm_status step_once(lbm_ctx *ctx) {
   StepState ss;
   TRY(step_begin(ctx, ss));
@@ -1674,6 +1679,7 @@ lbm_status step_once(lbm_ctx *ctx) {
 lbm_status step_many(lbm_ctx *ctx, int nsteps) {
   int done = 0;
   const int share = run_share(ctx);
+  ctx->beside = (share - 1) * pop_bytes(ctx);  // taken to be alike
   if (nsteps >= 2 && run_ok(ctx, share)) TRY(run_steps(&ctx, 1, nsteps, share, ctx->st, &done));
   for (; done < nsteps; done++) TRY(step_once(ctx));
   return LBM_OK;
@@ -2263,7 +2269,12 @@ lbm_status lbm_step_multi(lbm_ctx *const *ctxs, int n, int nsteps) {
       if (ctxs[j] == ctxs[i]) return fail(ctxs[i], LBM_ERR_ARG, "a lattice appears twice");
   }
   for (int i = 0; i < n; i++) TRY(prepare(ctxs[i]));
-  for (int i = 0; i < n; i++) run_share(ctxs[i]);
+  long long bytes = 0;
+  for (int i = 0; i < n; i++) bytes += pop_bytes(ctxs[i]);
+  for (int i = 0; i < n; i++) {
+    run_share(ctxs[i]);
+    ctxs[i]->beside = bytes - pop_bytes(ctxs[i]);
+  }
   // lattices that can share a bulk launch: same lattice, collision and storage
   std::vector<std::vector<int>> groups;
   for (int i = 0; i < n; i++) {
@@ -3104,6 +3115,9 @@ lbm_status batch_advance(lbm_batch *b, int nsteps) {
     for (const auto &g : groups) us += run_us(b, g);
     if (!groups.empty() && us <= graph_us(b)) return batch_run(b, groups, nsteps);
   }
+  long long bytes = 0;
+  for (int i = 0; i < n; i++) bytes += b->active[i] ? pop_bytes(b->ctx[i]) : 0;
+  for (int i = 0; i < n; i++) b->ctx[i]->beside = bytes - (b->active[i] ? pop_bytes(b->ctx[i]) : 0);
   int done = 0;
   while (done < nsteps) {
     const bool pair = nsteps - done >= 2;
@@ -3243,6 +3257,7 @@ void lbm_batch_destroy(lbm_batch *b) {
     if (i < b->own_st.size() && b->own_st[i]) {
       cudaStreamSynchronize(b->own_st[i]);
       b->ctx[i]->st = b->user_st[i];
+      b->ctx[i]->beside = 0;
       cudaStreamDestroy(b->own_st[i]);
     }
     if (i < b->ev_done.size() && b->ev_done[i]) cudaEventDestroy(b->ev_done[i]);

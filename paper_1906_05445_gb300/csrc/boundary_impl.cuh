@@ -1043,13 +1043,19 @@ inline int div_up(long long a, int b) { return (int)((a + b - 1) / b); }
 //
 // Both arrays together up to kReuseBytes (1.5 times the 129 MB L2): the reads
 // are evict-first, so that L2 keeps what the step writes, which the next step
-// reads.  us per step without / with it, lattices without solids: FP32 96^3
-// (134 MB) 20.6 / 18.5, 112^3 (213 MB) 32.6 / 30.9, 128^3 (319 MB) 48.0 / 47.2,
-// 160^3 (623 MB) 92.5 / 93.2; FP16 112^3 (107 MB) 18.5 / 16.5, 128^3 (159 MB)
-// 26.7 / 24.7, 192^3 (538 MB) 84.0 / 84.6.  The line lies below the sizes that
-// gain little alone: two 128^3 FP32 lattices stepped side by side on their own
-// streams lose 4% with it (100.0 -> 104.0 us per step of both).
+// reads.  us per step without / with it, lattices without solids: FP32 84^3
+// (90 MB) 14.5 / 12.9, 96^3 (134 MB) 21.7 / 19.0, 104^3 (171 MB) 27.4 / 25.4,
+// 112^3 (213 MB) 33.6 / 32.5, 128^3 (319 MB) 48.6 / 47.7, 144^3 (454 MB) 68.4 / 70.3;
+// FP16 112^3 (107 MB) 19.1 / 17.7, 128^3 (159 MB) 29.0 / 26.6, 160^3 (311 MB)
+// 52.9 / 51.9.  The line lies below the sizes that gain little alone and lose side
+// by side: two 112^3 FP32 lattices 66.9 / 71.5.
+// With other lattices stepping beside it (a batch, other streams) L2 is theirs
+// too: up to kReuseBeside together.  Batches with the hint in every lattice / none:
+// FP32 8 x 80^3 (623 MB) 100.5 / 92.3, 8 x 72^3 with spheres (454 MB) 77.2 / 74.1,
+// 4 x 96^3 (538 MB) 89.2 / 83.9, 8 x 64^3 IBM (319 MB) 70.0 / 68.1, 2 x 96^3
+// (269 MB) 43.3 / 43.1; FP16 8 x 80^3 (311 MB) 60.0 / 62.4.
 constexpr long long kReuseBytes = 192LL << 20;
+constexpr long long kReuseBeside = 300LL << 20;
 template <int LAT, int CM, typename S, int W>
 bool launch_bulk_vec_w(const KArgs &a, int want, bool packed, cudaStream_t st) {
   constexpr int V = W * VecS<S>::per_word;
@@ -1057,7 +1063,8 @@ bool launch_bulk_vec_w(const KArgs &a, int want, bool packed, cudaStream_t st) {
   const int nt = (int)(a.N / V);
   const int grid = div_up(nt, want);
   // the hint is built for the default shape only
-  const bool once = 2 * Lat<LAT>::Q * a.fs * (long long)sizeof(S) <= kReuseBytes;
+  const long long bytes = 2 * Lat<LAT>::Q * a.fs * (long long)sizeof(S);
+  const bool once = bytes <= kReuseBytes && bytes + a.beside <= kReuseBeside;
   constexpr int kOnce = W == 2 ? LD_ONCE : LD_NC;
   if (packed) {
     if (once && vec_packed<S>())

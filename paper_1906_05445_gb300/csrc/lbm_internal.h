@@ -112,6 +112,7 @@ struct KArgs {
                        // 2 vectors fed by bulk copies of row segments (each where nx and
                        // the direction stride allow, else the next simpler one)
   int bulk_vec_words;  // vector sweep: 32-bit words per thread and direction (2 or 4; 0 = 2)
+  long long beside;    // bytes of the populations of lattices stepping beside this one
   int bulk_vec_packed; // vector sweep: 1 packed FP32x2 collision of node pairs, 0 node by
                        // node, -1 by storage type
   int rev;             // bulk sweep: blocks walk the lattice from its end
