@@ -979,7 +979,7 @@ bool run_small(const lbm_ctx *ctx, int share);
 // kernel: two 128^3 lattices 98.9 us per step against 101.4 with the band
 // nodes gathering beside the sweep.  Axes of at least 8 nodes: two stencils then meet at
 // one periodic shift only, and a node lies in a stencil once.
-lbm_status build_tables(lbm_ctx *ctx) {
+lbm_status fill_tables(lbm_ctx *ctx) {
   const bool small = ctx->d.nx < 8 || ctx->d.ny < 8 || (ctx->D == 3 && ctx->d.nz < 8);
   if (ctx->scheme.scheme != LBM_IBM_DIRECT || ctx->nmark == 0 || any_moving(ctx) || small ||
       ctx->list_count <= 0 || ctx->ibm_cluster_on || !ctx->ibm_tables ||
@@ -1031,6 +1031,15 @@ lbm_status build_tables(lbm_ctx *ctx) {
   tb.mw = mw;
   tb.nmark = nm;
   ctx->tab = tb;
+  return LBM_OK;
+}
+
+// Without memory for them the markers scatter, as on a large lattice.
+lbm_status build_tables(lbm_ctx *ctx) {
+  const lbm_status s = fill_tables(ctx);
+  if (s != LBM_ERR_OOM) return s;
+  free_tables(ctx);
+  ctx->err.clear();
   return LBM_OK;
 }
 

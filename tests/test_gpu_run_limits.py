@@ -271,3 +271,37 @@ def test_batch_takes_one_route_for_all(monkeypatch):
         b.close()
         for g in alone + mixed:
             g.close()
+
+
+@pytest.mark.parametrize("iters", [1, 3])
+def test_no_memory_for_the_tables(monkeypatch, iters):
+    """Where the markers' tables find no memory, the lattice steps without them,
+    as with LBM_IBM_TABLES=0."""
+    from paper_1906_05445_gb300 import lbm
+    p = _disc(W.FP64, iters)
+
+    def run(allowed):
+        lbm.debug_fail_allocations_after(allowed)
+        g = None
+        try:
+            g = lbm.Lattice.from_problem(p)
+            g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+            g.step(5)
+            lbm.debug_fail_allocations_after(-1)
+            return g.velocity(), g.solid_mask(), g.force_torque(0)
+        except lbm.LbmError as e:
+            assert "OOM" in str(e)
+        finally:
+            lbm.debug_fail_allocations_after(-1)
+            if g is not None:
+                g.close()
+
+    monkeypatch.setenv("LBM_IBM_TABLES", "0")
+    need = next(k for k in range(200) if run(k) is not None)
+    ref = run(need)
+    monkeypatch.setenv("LBM_IBM_TABLES", "1")
+    assert run(need - 1) is None
+    for extra in (0, 1, 4, 9):
+        got = run(need + extra)
+        assert rel_l2(got[0], ref[0], ref[1]) <= 1e-13
+        assert np.abs(got[2][0] - ref[2][0]).max() <= 2e-12 * np.abs(ref[2][0]).max()
