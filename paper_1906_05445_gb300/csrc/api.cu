@@ -76,6 +76,7 @@ constexpr int kHistCap = 4096;          // force records kept (steps)
 // slots of their ring: one more than is handed out, for the record that a
 // multi-step launch clears ahead of the step after it
 constexpr int kHistSlots = kHistCap + 1;
+constexpr int kTabMem = 15;  // buffers of the IBM tables
 constexpr double kFp16Scale = (double)(1 << kFp16ScaleLog2);  // FP16 storage keeps (f - w) * 2^10
 constexpr int kGeomMargin = 7;          // box margin around a moving solid
 
@@ -226,7 +227,11 @@ struct lbm_ctx {
   int nmark = 0;
   // tables of markers at rest (ibm_device.cuh): tab.nmark 0 without them
   IbmTab tab{};
-  std::vector<void *> tab_mem;
+  // their memory, kept from one geometry to the next (kTabMem buffers)
+  struct TabMem {
+    void *p = nullptr;
+    size_t bytes = 0;
+  } tab_mem[kTabMem];
   int mk_start[kMaxSolids + 1] = {0};  // markers of solid k: mk_start[k] .. mk_start[k+1] - 1
   // the forcing loop in one cluster per solid (see ibm.cu), taken with
   // LBM_IBM_CLUSTER=1 where it fits the device (decided when the markers are
@@ -959,14 +964,27 @@ void ibm_prepare(lbm_ctx *ctx, cudaStream_t s);
 IbmArgs ibm_args(lbm_ctx *ctx, double *acc);
 
 void free_tables(lbm_ctx *ctx) {
-  for (void *p : ctx->tab_mem) dfree(ctx, p);
-  ctx->tab_mem.clear();
+  for (auto &m : ctx->tab_mem) {
+    dfree(ctx, m.p);
+    ctx->dev_bytes -= m.bytes;
+    m = {};
+  }
   ctx->tab = IbmTab{};
 }
 
-lbm_status tab_alloc(lbm_ctx *ctx, void **p, size_t bytes) {
-  TRY(dalloc(ctx, p, std::max<size_t>(bytes, 8)));
-  ctx->tab_mem.push_back(*p);
+// Buffer `k` of at least `bytes`, with room for the next geometry's.
+template <typename P> lbm_status tab_alloc(lbm_ctx *ctx, int k, P **p, size_t bytes) {
+  auto &m = ctx->tab_mem[k];
+  bytes = std::max<size_t>(bytes, 8);
+  if (m.bytes < bytes) {
+    dfree(ctx, m.p);
+    ctx->dev_bytes -= m.bytes;
+    m = {};
+    const size_t want = bytes + bytes / 8 + 64;
+    TRY(dalloc(ctx, &m.p, want));
+    m.bytes = want;
+  }
+  *p = (P *)m.p;
   return LBM_OK;
 }
 
@@ -993,33 +1011,46 @@ lbm_status fill_tables(lbm_ctx *ctx) {
   tb.dV = ctx->mk_dV;
   tb.msid = ctx->mk_sid;
   tb.Fm = ctx->mk_F;
-  IbmArgs ib = ibm_args(ctx, nullptr);
-  int *nrow = nullptr, *ncol = nullptr, *mrow = nullptr, *mcol = nullptr;
-  void *nw = nullptr, *mw = nullptr;
+  const IbmArgs ib = ibm_args(ctx, nullptr);
+  TabCells cells = tab_cells(ib);
+  const size_t ncell = (size_t)cells.nc[0] * cells.nc[1] * cells.nc[2];
+  int *nrow = nullptr, *ncol = nullptr, *mrow = nullptr, *mcol = nullptr, *tmp = nullptr;
+  char *nw = nullptr, *mw = nullptr, *dFT = nullptr, *FdV = nullptr;
   double *Ud = nullptr, *arm = nullptr;
-  TRY(tab_alloc(ctx, (void **)&nrow, sizeof(int) * ((size_t)nl + 1)));
-  TRY(tab_alloc(ctx, (void **)&mrow, sizeof(int) * ((size_t)nm + 1)));
-  TRY(tab_alloc(ctx, (void **)&Ud, sizeof(double) * 3 * nm));
-  TRY(tab_alloc(ctx, (void **)&arm, sizeof(double) * 3 * nm));
-  TRY(tab_alloc(ctx, (void **)&tb.dF, sizeof(double) * 3 * nm));
-  TRY(tab_alloc(ctx, &tb.dFT, ctx->tsz * 6 * nm));
-  TRY(tab_alloc(ctx, &tb.FdV, ctx->tsz * 3 * nm));
+  TRY(tab_alloc(ctx, 0, &nrow, sizeof(int) * ((size_t)nl + 1)));
+  TRY(tab_alloc(ctx, 1, &mrow, sizeof(int) * ((size_t)nm + 1)));
+  TRY(tab_alloc(ctx, 2, &Ud, sizeof(double) * 3 * nm));
+  TRY(tab_alloc(ctx, 3, &arm, sizeof(double) * 3 * nm));
+  TRY(tab_alloc(ctx, 4, &tb.dF, sizeof(double) * 3 * nm));
+  TRY(tab_alloc(ctx, 5, &dFT, ctx->tsz * 6 * nm));
+  TRY(tab_alloc(ctx, 6, &FdV, ctx->tsz * 3 * nm));
+  TRY(tab_alloc(ctx, 7, &cells.start, sizeof(int) * (2 * ncell + 1)));
+  cells.cur = cells.start + ncell + 1;
+  TRY(tab_alloc(ctx, 8, &cells.mk, sizeof(int) * (size_t)nm));
+  TRY(tab_alloc(ctx, 9, &cells.phi, sizeof(double) * 12 * nm));
   launch_tab_desired(ib, Ud, arm, ctx->st);
-  launch_tab_nodes(ib, ctx->list_node, nl, nrow, nullptr, nullptr, ctx->d.precision, ctx->st);
-  if (iterate) launch_tab_markers(ib, mrow, nullptr, nullptr, ctx->d.precision, ctx->st);
-  int ne = 0, me = 0;
-  CK(cudaMemcpyAsync(&ne, nrow + nl, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-  if (iterate) CK(cudaMemcpyAsync(&me, mrow + nm, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-  CK(cudaStreamSynchronize(ctx->st));
-  TRY(tab_alloc(ctx, (void **)&ncol, sizeof(int) * (size_t)ne));
-  TRY(tab_alloc(ctx, &nw, ctx->tsz * (size_t)ne));
-  launch_tab_nodes(ib, ctx->list_node, nl, nrow, ncol, nw, ctx->d.precision, ctx->st);
+  launch_tab_cells(ib, cells, ctx->st);
+  launch_tab_nodes(ib, cells, ctx->list_node, nl, nrow, nullptr, nullptr, nullptr, ctx->d.precision, ctx->st);
+  if (iterate) launch_tab_markers(ib, cells, mrow, nullptr, nullptr, nullptr, ctx->d.precision, ctx->st);
+  // a marker is in the rows of its stencil's nodes at most
+  const size_t ne = (size_t)nm * (ctx->D == 3 ? 64 : 16);
+  int me = 0;
   if (iterate) {
-    TRY(tab_alloc(ctx, (void **)&mcol, sizeof(int) * (size_t)me));
-    TRY(tab_alloc(ctx, &mw, ctx->tsz * (size_t)me));
-    launch_tab_markers(ib, mrow, mcol, mw, ctx->d.precision, ctx->st);
+    CK(cudaMemcpyAsync(&me, mrow + nm, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+    CK(cudaStreamSynchronize(ctx->st));
   }
-  ctx->launches += iterate ? 7 : 4;
+  TRY(tab_alloc(ctx, 10, &ncol, sizeof(int) * ne));
+  TRY(tab_alloc(ctx, 11, &nw, ctx->tsz * ne));
+  TRY(tab_alloc(ctx, 12, &tmp, sizeof(int) * std::max(ne, (size_t)me)));
+  launch_tab_nodes(ib, cells, ctx->list_node, nl, nrow, tmp, ncol, nw, ctx->d.precision, ctx->st);
+  if (iterate) {
+    TRY(tab_alloc(ctx, 13, &mcol, sizeof(int) * (size_t)me));
+    TRY(tab_alloc(ctx, 14, &mw, ctx->tsz * (size_t)me));
+    launch_tab_markers(ib, cells, mrow, tmp, mcol, mw, ctx->d.precision, ctx->st);
+  }
+  ctx->launches += iterate ? 10 : 7;
+  tb.dFT = dFT;
+  tb.FdV = FdV;
   CK(cudaGetLastError());
   tb.Ud = Ud;
   tb.arm = arm;
@@ -1037,10 +1068,9 @@ lbm_status fill_tables(lbm_ctx *ctx) {
 // Without memory for them the markers scatter, as on a large lattice.
 lbm_status build_tables(lbm_ctx *ctx) {
   const lbm_status s = fill_tables(ctx);
-  if (s != LBM_ERR_OOM) return s;
-  free_tables(ctx);
-  ctx->err.clear();
-  return LBM_OK;
+  if (ctx->tab.nmark == 0) free_tables(ctx);
+  if (s == LBM_ERR_OOM) ctx->err.clear();
+  return s == LBM_ERR_OOM ? LBM_OK : s;
 }
 
 lbm_status read_counts(lbm_ctx *ctx, int out[16]) {
@@ -1053,7 +1083,7 @@ lbm_status read_counts(lbm_ctx *ctx, int out[16]) {
 // boundary nodes and links first, size the lists exactly, then build.
 lbm_status rebuild_full(lbm_ctx *ctx) {
   if (ctx) ctx->gen++;
-  free_tables(ctx);
+  ctx->tab = IbmTab{};  // their memory stays for the next ones
   free_spare(ctx);  // capacities may change; the next moving step prefetches again
   TRY(motion_pull(ctx));
   if (!ctx->restore_geometry)

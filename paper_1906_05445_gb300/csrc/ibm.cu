@@ -9,6 +9,10 @@
 // block in FP64.
 #include <cooperative_groups.h>
 
+#include <string.h>
+
+#include <algorithm>
+
 #include "ibm_device.cuh"
 
 namespace cg = cooperative_groups;
@@ -191,8 +195,78 @@ __global__ void __launch_bounds__(128) k_fused(const IbmArgs a) {
 
 // ---------------------------------------------------------------- tables
 // Built once per geometry of solids at rest (ibm_device.cuh says what they
-// are for) by exhaustive search, a warp per row: the rows come out in marker
-// order without sorting or atomics.  COUNT: row lengths only.
+// are for), a warp per row, which looks at the markers of the cells around it:
+// searching them all took 108 of the 113 ms that the geometry of a sphere of
+// R = 60 with five passes takes (45 k markers).  The row's markers are then put in
+// marker order by rank, so that sums over it repeat bit for bit.  COUNT: row
+// lengths only.
+
+__device__ __forceinline__ int cell_axis(const TabCells &c, int a, int v) {
+  return min(v >> c.shift, c.nc[a] - 1);
+}
+
+// the cells that hold v - 3 (wrapped) and v, and with `up` v + 3: cells are at
+// least 4 nodes wide, so no other cell meets the stretch between them
+__device__ __forceinline__ int cells_near(const TabCells &c, int a, int v, int n, bool up, int (&out)[3]) {
+  int k = 0;
+  out[k++] = cell_axis(c, a, wrap(v, n));
+  const int lo = cell_axis(c, a, wrap(v - 3, n));
+  if (lo != out[0]) out[k++] = lo;
+  if (up) {
+    const int hi = cell_axis(c, a, wrap(v + 3, n));
+    if (hi != out[0] && hi != lo) out[k++] = hi;
+  }
+  return k;
+}
+
+__global__ void __launch_bounds__(128) k_cell_markers(const IbmArgs a, const TabCells c, bool place) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= a.nmark) return;
+  const int4 b = a.mk_base[m];
+  const int cell = cell_axis(c, 0, wrap(b.x, a.nx)) +
+                   c.nc[0] * (cell_axis(c, 1, wrap(b.y, a.ny)) +
+                              c.nc[1] * (a.dim == 3 ? cell_axis(c, 2, wrap(b.z, a.nz)) : 0));
+  if (!place) {
+    atomicAdd(c.start + cell, 1);
+    const Stencil<double> s = stencil_of<double>(a, marker(a, m));
+    for (int k = 0; k < 4; k++) {
+      c.phi[12 * (long long)m + k] = phi_k<double>(a.kernel, s.dx + k);
+      c.phi[12 * (long long)m + 4 + k] = phi_k<double>(a.kernel, s.dy + k);
+      c.phi[12 * (long long)m + 8 + k] = a.dim == 3 ? phi_k<double>(a.kernel, s.dz + k) : 0.0;
+    }
+  } else {
+    c.mk[c.start[cell] + atomicAdd(c.cur + cell, 1)] = m;
+  }
+}
+
+// Every marker of the cells near (x, y, z), a lane each: f(marker or -1).
+template <typename F>
+__device__ __forceinline__ void near_markers(const IbmArgs &a, const TabCells &c, int x, int y, int z,
+                                             bool up, int lane, F f) {
+  int cx[3], cy[3], cz[3] = {0, 0, 0};
+  const int kx = cells_near(c, 0, x, a.nx, up, cx), ky = cells_near(c, 1, y, a.ny, up, cy);
+  const int kz = a.dim == 3 ? cells_near(c, 2, z, a.nz, up, cz) : 1;
+  for (int k = 0; k < kz; k++)
+    for (int j = 0; j < ky; j++)
+      for (int i = 0; i < kx; i++) {
+        const int cell = cx[i] + c.nc[0] * (cy[j] + c.nc[1] * cz[k]);
+        const int end = c.start[cell + 1];
+        for (int q = c.start[cell]; q < end; q += 32) f(q + lane < end ? c.mk[q + lane] : -1);
+      }
+}
+
+// A row's entries tmp[row .. row + n - 1] in rising order to col, and f of each.
+template <typename F>
+__device__ __forceinline__ void rank_row(const int *tmp, int *col, int row, int n, int lane, F f) {
+  __syncwarp();
+  for (int e = lane; e < n; e += 32) {
+    const int m = tmp[row + e];
+    int r = row;
+    for (int j = 0; j < n; j++) r += tmp[row + j] < m;
+    col[r] = m;
+    f(r, m);
+  }
+}
 
 // whether node (x, y, z) lies in the stencil of base b, and its point
 __device__ __forceinline__ int stencil_index(const IbmArgs &a, int4 b, int x, int y, int z) {
@@ -202,27 +276,29 @@ __device__ __forceinline__ int stencil_index(const IbmArgs &a, int4 b, int x, in
 }
 
 template <typename T, bool COUNT>
-__global__ void __launch_bounds__(128) k_tab_nodes(const IbmArgs a, const int *list_node, int nlist,
-                                                   int *row, int *col, T *wt) {
+__global__ void __launch_bounds__(128) k_tab_nodes(const IbmArgs a, const TabCells c, const int *list_node,
+                                                   int nlist, int *row, int *tmp, int *col, T *wt) {
   const int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (t >= nlist) return;
   const int n = list_node[t];
   const int x = n % a.nx, y = (n / a.nx) % a.ny, z = n / (a.nx * a.ny);
   const int npts = a.dim == 3 ? 64 : 16;
-  int at = COUNT ? 0 : row[t];
-  for (int m0 = 0; m0 < a.nmark; m0 += 32) {
-    const int m = m0 + lane;
-    const int p = m < a.nmark ? stencil_index(a, a.mk_base[m], x, y, z) : -1;
-    const unsigned hit = __ballot_sync(0xffffffffu, p >= 0);
-    if (!COUNT && p >= 0) {
-      const int e = at + __popc(hit & ((1u << lane) - 1u));
-      col[e] = m;
-      wt[e] = ((const T *)a.mk_wts)[(long long)m * npts + p];
-    }
+  const int first = COUNT ? 0 : row[t];
+  int at = first;
+  near_markers(a, c, x, y, z, false, lane, [&](int m) {
+    const bool in = m >= 0 && stencil_index(a, a.mk_base[m], x, y, z) >= 0;
+    const unsigned hit = __ballot_sync(0xffffffffu, in);
+    if (!COUNT && in) tmp[at + __popc(hit & ((1u << lane) - 1u))] = m;
     at += __popc(hit);
+  });
+  if (COUNT) {
+    if (lane == 0) row[t] = at;
+  } else {
+    rank_row(tmp, col, first, at - first, lane, [&](int e, int m) {
+      wt[e] = ((const T *)a.mk_wts)[(long long)m * npts + stencil_index(a, a.mk_base[m], x, y, z)];
+    });
   }
-  if (COUNT && lane == 0) row[t] = at;
 }
 
 // separation of two stencil bases on an axis of n >= 8 nodes, or 8 when the
@@ -232,73 +308,79 @@ __device__ __forceinline__ int base_shift(int b0, int b1, int n) {
   return d <= 3 ? d : (n - d <= 3 ? d - n : 8);
 }
 
-// sum_k phi(x0 + k) phi(x1 + k - d): node k of the first stencil is node k - d
-// of the second, whose base lies d nodes further
-template <typename T>
-__device__ __forceinline__ T overlap(int kernel, T x0, T x1, int d) {
-  T s = (T)0;
-  for (int k = 0; k < 4; k++) {
-    const int q = k - d;
-    if (q >= 0 && q < 4) s += phi_k<T>(kernel, x0 + (T)k) * phi_k<T>(kernel, x1 + (T)q);
-  }
+// sum_k phi0(k) phi1(k - d): node k of the first stencil is node k - d of the
+// second, whose base lies d nodes further
+__device__ __forceinline__ double overlap(const double *p0, const double *p1, int d) {
+  double s = 0;
+  for (int k = max(0, d); k < min(4, 4 + d); k++) s += p0[k] * p1[k - d];
   return s;
 }
 
 template <typename T, bool COUNT>
-__global__ void __launch_bounds__(128) k_tab_markers(const IbmArgs a, int *row, int *col, T *wt) {
+__global__ void __launch_bounds__(128) k_tab_markers(const IbmArgs a, const TabCells c, int *row,
+                                                     int *tmp, int *col, T *wt) {
   const int m = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (m >= a.nmark) return;
   const int4 b = a.mk_base[m];
-  const Stencil<T> s0 = stencil_of<T>(a, marker(a, m));
-  int at = COUNT ? 0 : row[m];
-  for (int k0 = 0; k0 < a.nmark; k0 += 32) {
-    const int k = k0 + lane;
-    int dx = 8, dy = 8, dz = 8;
-    if (k < a.nmark) {
-      const int4 c = a.mk_base[k];
-      dx = base_shift(b.x, c.x, a.nx);
-      dy = base_shift(b.y, c.y, a.ny);
-      dz = a.dim == 3 ? base_shift(b.z, c.z, a.nz) : 0;
-    }
-    const bool meet = dx < 8 && dy < 8 && dz < 8;
+  const int first = COUNT ? 0 : row[m];
+  int at = first;
+  auto shifts = [&](int k, int (&d)[3]) {
+    const int4 o = a.mk_base[k];
+    d[0] = base_shift(b.x, o.x, a.nx);
+    d[1] = base_shift(b.y, o.y, a.ny);
+    d[2] = a.dim == 3 ? base_shift(b.z, o.z, a.nz) : 0;
+    return d[0] < 8 && d[1] < 8 && d[2] < 8;
+  };
+  near_markers(a, c, b.x, b.y, b.z, true, lane, [&](int k) {
+    int d[3];
+    const bool meet = k >= 0 && shifts(k, d);
     const unsigned hit = __ballot_sync(0xffffffffu, meet);
-    if (!COUNT && meet) {
-      const int e = at + __popc(hit & ((1u << lane) - 1u));
-      const Stencil<T> s1 = stencil_of<T>(a, marker(a, k));
-      T w = overlap<T>(a.kernel, s0.dx, s1.dx, dx) * overlap<T>(a.kernel, s0.dy, s1.dy, dy);
-      if (a.dim == 3) w *= overlap<T>(a.kernel, s0.dz, s1.dz, dz);
-      col[e] = k;
-      wt[e] = w * (T)a.dV[k];
-    }
+    if (!COUNT && meet) tmp[at + __popc(hit & ((1u << lane) - 1u))] = k;
     at += __popc(hit);
+  });
+  if (COUNT) {
+    if (lane == 0) row[m] = at;
+  } else {
+    // the coefficients in FP64, rounded once
+    const double *p0 = c.phi + 12 * (long long)m;
+    rank_row(tmp, col, first, at - first, lane, [&](int e, int k) {
+      int d[3];
+      shifts(k, d);
+      const double *p1 = c.phi + 12 * (long long)k;
+      double w = overlap(p0, p1, d[0]) * overlap(p0 + 4, p1 + 4, d[1]);
+      if (a.dim == 3) w *= overlap(p0 + 8, p1 + 8, d[2]);
+      wt[e] = (T)(w * a.dV[k]);
+    });
   }
-  if (COUNT && lane == 0) row[m] = at;
 }
 
 // exclusive prefix sum of n counts in place, the total in v[n] (one block)
 __global__ void __launch_bounds__(1024) k_tab_scan(int *v, int n) {
-  __shared__ int sh[1024];
-  const int t = threadIdx.x;
+  __shared__ int sh[32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int per = (n + 1023) / 1024;
   const int i0 = min(n, t * per), i1 = min(n, i0 + per);
   int s = 0;
   for (int i = i0; i < i1; i++) s += v[i];
-  sh[t] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const int add = t >= o ? sh[t - o] : 0;
-    __syncthreads();
-    sh[t] += add;
-    __syncthreads();
+  int sum = s;  // inclusive over the warp, then the warps before it added
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, sum, o);
+    if (lane >= o) sum += up;
   }
-  int at = sh[t] - s;
+  if (lane == 31) sh[warp] = sum;
+  __syncthreads();
+  int w = lane < warp ? sh[lane] : 0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  int at = w + sum - s;
   for (int i = i0; i < i1; i++) {
     const int c = v[i];
     v[i] = at;
     at += c;
   }
-  if (t == 1023) v[n] = sh[1023];
+  if (t == 1023) v[n] = at;
 }
 
 // desired velocity and lever arm of every marker (solids at rest)
@@ -625,29 +707,50 @@ void launch_ibm_cluster(const IbmArgs &a, const IbmClusterArgs &cl, int precisio
     launch_cluster_t<float>(a, cl, smem, st);
 }
 
-void launch_tab_nodes(const IbmArgs &a, const int *list_node, int nlist, int *row, int *col,
-                      void *wt, int precision, cudaStream_t st) {
-  const int grid = (nlist + 3) / 4;
-  if (!col) {
-    k_tab_nodes<float, true><<<grid, 128, 0, st>>>(a, list_node, nlist, row, nullptr, nullptr);
-    k_tab_scan<<<1, 1024, 0, st>>>(row, nlist);
-  } else if (precision == LBM_FP64) {
-    k_tab_nodes<double, false><<<grid, 128, 0, st>>>(a, list_node, nlist, row, col, (double *)wt);
-  } else {
-    k_tab_nodes<float, false><<<grid, 128, 0, st>>>(a, list_node, nlist, row, col, (float *)wt);
+// As few cells as still hold a few markers each, so that they cost no more to
+// clear and scan than the markers themselves.
+TabCells tab_cells(const IbmArgs &a) {
+  TabCells c;
+  memset(&c, 0, sizeof(c));
+  for (c.shift = 2;; c.shift++) {
+    c.nc[0] = std::max(1, a.nx >> c.shift);
+    c.nc[1] = std::max(1, a.ny >> c.shift);
+    c.nc[2] = a.dim == 3 ? std::max(1, a.nz >> c.shift) : 1;
+    if ((double)c.nc[0] * c.nc[1] * c.nc[2] <= std::max(4096.0, 4.0 * a.nmark)) return c;
   }
 }
 
-void launch_tab_markers(const IbmArgs &a, int *row, int *col, void *wt, int precision,
-                        cudaStream_t st) {
+void launch_tab_cells(const IbmArgs &a, const TabCells &c, cudaStream_t st) {
+  const int n = c.nc[0] * c.nc[1] * c.nc[2], grid = (a.nmark + 127) / 128;
+  cudaMemsetAsync(c.start, 0, sizeof(int) * (2 * (size_t)n + 1), st);
+  k_cell_markers<<<grid, 128, 0, st>>>(a, c, false);
+  k_tab_scan<<<1, 1024, 0, st>>>(c.start, n);
+  k_cell_markers<<<grid, 128, 0, st>>>(a, c, true);
+}
+
+void launch_tab_nodes(const IbmArgs &a, const TabCells &c, const int *list_node, int nlist, int *row,
+                      int *tmp, int *col, void *wt, int precision, cudaStream_t st) {
+  const int grid = (nlist + 3) / 4;
+  if (!col) {
+    k_tab_nodes<float, true><<<grid, 128, 0, st>>>(a, c, list_node, nlist, row, tmp, nullptr, nullptr);
+    k_tab_scan<<<1, 1024, 0, st>>>(row, nlist);
+  } else if (precision == LBM_FP64) {
+    k_tab_nodes<double, false><<<grid, 128, 0, st>>>(a, c, list_node, nlist, row, tmp, col, (double *)wt);
+  } else {
+    k_tab_nodes<float, false><<<grid, 128, 0, st>>>(a, c, list_node, nlist, row, tmp, col, (float *)wt);
+  }
+}
+
+void launch_tab_markers(const IbmArgs &a, const TabCells &c, int *row, int *tmp, int *col, void *wt,
+                        int precision, cudaStream_t st) {
   const int grid = (a.nmark + 3) / 4;
   if (!col) {
-    k_tab_markers<float, true><<<grid, 128, 0, st>>>(a, row, nullptr, nullptr);
+    k_tab_markers<float, true><<<grid, 128, 0, st>>>(a, c, row, tmp, nullptr, nullptr);
     k_tab_scan<<<1, 1024, 0, st>>>(row, a.nmark);
   } else if (precision == LBM_FP64) {
-    k_tab_markers<double, false><<<grid, 128, 0, st>>>(a, row, col, (double *)wt);
+    k_tab_markers<double, false><<<grid, 128, 0, st>>>(a, c, row, tmp, col, (double *)wt);
   } else {
-    k_tab_markers<float, false><<<grid, 128, 0, st>>>(a, row, col, (float *)wt);
+    k_tab_markers<float, false><<<grid, 128, 0, st>>>(a, c, row, tmp, col, (float *)wt);
   }
 }
 

@@ -313,12 +313,24 @@ void launch_ibm_fused(const IbmArgs &a, int precision, cudaStream_t st);
 void launch_ibm_interp(const IbmArgs &a, int precision, cudaStream_t st);
 void launch_ibm_spread(const IbmArgs &a, int precision, cudaStream_t st);
 
+// Markers of solids at rest by cell: cell (x, y, z) >> shift, the last one of an
+// axis wider, holds the markers whose stencil begins in it.
+struct TabCells {
+  int nc[3];         // cells per axis
+  int shift;         // cells of 2^shift >= 4 nodes
+  int *start, *cur;  // [cells + 1] first entry of a cell, then [cells] entries placed
+  int *mk;           // [nmark] markers by cell
+  double *phi;       // [nmark][3][4] the delta function of every axis at the stencil
+};
+// the cells of a lattice with this many markers (start, cur, mk, phi unset)
+TabCells tab_cells(const IbmArgs &a);
+void launch_tab_cells(const IbmArgs &a, const TabCells &c, cudaStream_t st);
 // tables of solids at rest: without `col` the row lengths and their prefix
-// sum (row[0 .. n]), with it the entries
-void launch_tab_nodes(const IbmArgs &a, const int *list_node, int nlist, int *row, int *col,
-                      void *wt, int precision, cudaStream_t st);
-void launch_tab_markers(const IbmArgs &a, int *row, int *col, void *wt, int precision,
-                        cudaStream_t st);
+// sum (row[0 .. n]), with it the entries; tmp as long as col
+void launch_tab_nodes(const IbmArgs &a, const TabCells &c, const int *list_node, int nlist, int *row,
+                      int *tmp, int *col, void *wt, int precision, cudaStream_t st);
+void launch_tab_markers(const IbmArgs &a, const TabCells &c, int *row, int *tmp, int *col, void *wt,
+                        int precision, cudaStream_t st);
 void launch_tab_desired(const IbmArgs &a, double *Ud, double *arm, cudaStream_t st);
 // one forcing pass over the markers through the tables (a.tab): pass 0
 // interpolates u~, later ones iterate; the last keeps F dV and reduces the
