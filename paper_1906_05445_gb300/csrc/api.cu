@@ -2164,6 +2164,7 @@ lbm_status lbm_set_solid_motion(lbm_ctx *ctx, int id, const double centre[3], co
   if (!ctx || id < 0 || id >= (int)ctx->solids.size()) return LBM_ERR_ARG;
   TRY(solids_to_host(ctx, true));
   SolidHost &h = ctx->solids[id];
+  const SolidHost was = h;
   for (int a = 0; a < 3; a++) {
     if (centre) h.c[a] = h.d.centre[a] = centre[a];
     if (vel) h.d.velocity[a] = vel[a];
@@ -2173,6 +2174,19 @@ lbm_status lbm_set_solid_motion(lbm_ctx *ctx, int id, const double centre[3], co
     h.c[2] = h.d.centre[2] = 0;
     h.d.velocity[2] = 0;
     h.d.omega[0] = h.d.omega[1] = 0;
+  }
+  bool turned = ctx->scheme.scheme == LBM_IBM_DIRECT && !ctx->geom_dirty && !any_moving(ctx);
+  for (int a = 0; a < 3; a++)
+    turned = turned && h.c[a] == was.c[a] && h.d.velocity[a] == was.d.velocity[a];
+  if (turned) {
+    // IBM at rest: the markers stay, their desired velocities are new
+    if (ctx->tab.nmark > 0) {
+      launch_tab_desired(ibm_args(ctx, nullptr), const_cast<double *>(ctx->tab.Ud),
+                         const_cast<double *>(ctx->tab.arm), ctx->st);
+      ctx->launches++;
+      CK(cudaGetLastError());
+    }
+    return LBM_OK;
   }
   // wall velocities are stored with the links: rebuild
   ctx->geom_dirty = true;

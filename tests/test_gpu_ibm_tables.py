@@ -69,3 +69,29 @@ def test_tables_keep_their_memory():
         sizes[tables] = np.array(held)
     extra = sizes[True] - sizes[False]
     assert extra[0] > 0 and extra[-1] <= 1.3 * extra[0]
+
+
+@pytest.mark.parametrize("precision", [W.FP64, W.FP32])
+@pytest.mark.parametrize("iters", [1, 3])
+def test_new_rotation_keeps_the_geometry(precision, iters):
+    """A new angular velocity of an IBM solid at rest changes the markers' desired
+    velocities only: the same fields as after a rebuild of everything."""
+    from paper_1906_05445_gb300 import lbm
+    p = W.Problem("turn", W.D3Q19, 26, 19, 17, 0.7, W.MRT, precision, (1e-4, -2e-4, 0.0),
+                  CASES[2][2], W.IBM, 0, ibm_iters=iters)
+    out = []
+    for rebuild in (False, True):
+        g = lbm.Lattice.from_problem(p)
+        g.init_equilibrium(1.0, (0.01, 0.005, 0.0))
+        g.step(3)
+        for k in range(3):
+            n0 = g.info().kernel_launches
+            g.set_solid_motion(1, omega=(1e-3, 0.0, 2e-3 * k), velocity=(0.0, 0.0, 0.0))
+            if rebuild:
+                g.set_scheme(W.IBM, iters)
+            g.step(2)
+            assert (g.info().kernel_launches - n0 <= 2) != rebuild
+        out.append((g.get_f(), g.force_torque(1)))
+        g.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.abs(out[0][1][1] - out[1][1][1]).max() <= 1e-12
