@@ -76,7 +76,7 @@ constexpr int kHistCap = 4096;          // force records kept (steps)
 // slots of their ring: one more than is handed out, for the record that a
 // multi-step launch clears ahead of the step after it
 constexpr int kHistSlots = kHistCap + 1;
-constexpr int kTabMem = 15;  // buffers of the IBM tables
+constexpr int kTabMem = 2;  // buffers of the IBM tables
 constexpr double kFp16Scale = (double)(1 << kFp16ScaleLog2);  // FP16 storage keeps (f - w) * 2^10
 constexpr int kGeomMargin = 7;          // box margin around a moving solid
 
@@ -972,19 +972,28 @@ void free_tables(lbm_ctx *ctx) {
   ctx->tab = IbmTab{};
 }
 
+// Arrays of one buffer (256-byte boundaries).
+struct TabLayout {
+  size_t bytes = 0;
+  size_t add(size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) / 256 * 256;
+    return at;
+  }
+};
+
 // Buffer `k` of at least `bytes`, with room for the next geometry's.
-template <typename P> lbm_status tab_alloc(lbm_ctx *ctx, int k, P **p, size_t bytes) {
+lbm_status tab_alloc(lbm_ctx *ctx, int k, char **p, size_t bytes) {
   auto &m = ctx->tab_mem[k];
-  bytes = std::max<size_t>(bytes, 8);
   if (m.bytes < bytes) {
     dfree(ctx, m.p);
     ctx->dev_bytes -= m.bytes;
     m = {};
-    const size_t want = bytes + bytes / 8 + 64;
+    const size_t want = bytes + bytes / 8;
     TRY(dalloc(ctx, &m.p, want));
     m.bytes = want;
   }
-  *p = (P *)m.p;
+  *p = (char *)m.p;
   return LBM_OK;
 }
 
@@ -1014,49 +1023,53 @@ lbm_status fill_tables(lbm_ctx *ctx) {
   const IbmArgs ib = ibm_args(ctx, nullptr);
   TabCells cells = tab_cells(ib);
   const size_t ncell = (size_t)cells.nc[0] * cells.nc[1] * cells.nc[2];
-  int *nrow = nullptr, *ncol = nullptr, *mrow = nullptr, *mcol = nullptr, *tmp = nullptr;
-  char *nw = nullptr, *mw = nullptr, *dFT = nullptr, *FdV = nullptr;
-  double *Ud = nullptr, *arm = nullptr;
-  TRY(tab_alloc(ctx, 0, &nrow, sizeof(int) * ((size_t)nl + 1)));
-  TRY(tab_alloc(ctx, 1, &mrow, sizeof(int) * ((size_t)nm + 1)));
-  TRY(tab_alloc(ctx, 2, &Ud, sizeof(double) * 3 * nm));
-  TRY(tab_alloc(ctx, 3, &arm, sizeof(double) * 3 * nm));
-  TRY(tab_alloc(ctx, 4, &tb.dF, sizeof(double) * 3 * nm));
-  TRY(tab_alloc(ctx, 5, &dFT, ctx->tsz * 6 * nm));
-  TRY(tab_alloc(ctx, 6, &FdV, ctx->tsz * 3 * nm));
-  TRY(tab_alloc(ctx, 7, &cells.start, sizeof(int) * (2 * ncell + 1)));
+  // a marker is in the rows of its stencil's nodes at most
+  const size_t ne = (size_t)nm * (ctx->D == 3 ? 64 : 16);
+  TabLayout l;
+  const size_t o_nrow = l.add(sizeof(int) * ((size_t)nl + 1)), o_mrow = l.add(sizeof(int) * ((size_t)nm + 1));
+  const size_t o_Ud = l.add(sizeof(double) * 3 * nm), o_arm = l.add(sizeof(double) * 3 * nm);
+  const size_t o_dF = l.add(sizeof(double) * 3 * nm), o_dFT = l.add(ctx->tsz * 6 * nm);
+  const size_t o_FdV = l.add(ctx->tsz * 3 * nm), o_cells = l.add(sizeof(int) * (2 * ncell + 1));
+  const size_t o_mk = l.add(sizeof(int) * (size_t)nm), o_phi = l.add(sizeof(double) * 12 * nm);
+  const size_t o_ncol = l.add(sizeof(int) * ne), o_nw = l.add(ctx->tsz * ne), o_tmp = l.add(sizeof(int) * ne);
+  char *base = nullptr;
+  TRY(tab_alloc(ctx, 0, &base, l.bytes));
+  int *nrow = (int *)(base + o_nrow), *mrow = (int *)(base + o_mrow), *ncol = (int *)(base + o_ncol);
+  double *Ud = (double *)(base + o_Ud), *arm = (double *)(base + o_arm);
+  tb.dF = (double *)(base + o_dF);
+  tb.dFT = base + o_dFT;
+  tb.FdV = base + o_FdV;
+  cells.start = (int *)(base + o_cells);
   cells.cur = cells.start + ncell + 1;
-  TRY(tab_alloc(ctx, 8, &cells.mk, sizeof(int) * (size_t)nm));
-  TRY(tab_alloc(ctx, 9, &cells.phi, sizeof(double) * 12 * nm));
+  cells.mk = (int *)(base + o_mk);
+  cells.phi = (double *)(base + o_phi);
   launch_tab_desired(ib, Ud, arm, ctx->st);
   launch_tab_cells(ib, cells, ctx->st);
   launch_tab_nodes(ib, cells, ctx->list_node, nl, nrow, nullptr, nullptr, nullptr, ctx->d.precision, ctx->st);
-  if (iterate) launch_tab_markers(ib, cells, mrow, nullptr, nullptr, nullptr, ctx->d.precision, ctx->st);
-  // a marker is in the rows of its stencil's nodes at most
-  const size_t ne = (size_t)nm * (ctx->D == 3 ? 64 : 16);
-  int me = 0;
+  launch_tab_nodes(ib, cells, ctx->list_node, nl, nrow, (int *)(base + o_tmp), ncol, base + o_nw,
+                   ctx->d.precision, ctx->st);
+  int *mcol = nullptr;
+  char *mw = nullptr;
   if (iterate) {
-    CK(cudaMemcpyAsync(&me, mrow + nm, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+    launch_tab_markers(ib, cells, mrow, nullptr, nullptr, nullptr, ctx->d.precision, ctx->st);
+    int n = 0;
+    CK(cudaMemcpyAsync(&n, mrow + nm, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
-  }
-  TRY(tab_alloc(ctx, 10, &ncol, sizeof(int) * ne));
-  TRY(tab_alloc(ctx, 11, &nw, ctx->tsz * ne));
-  TRY(tab_alloc(ctx, 12, &tmp, sizeof(int) * std::max(ne, (size_t)me)));
-  launch_tab_nodes(ib, cells, ctx->list_node, nl, nrow, tmp, ncol, nw, ctx->d.precision, ctx->st);
-  if (iterate) {
-    TRY(tab_alloc(ctx, 13, &mcol, sizeof(int) * (size_t)me));
-    TRY(tab_alloc(ctx, 14, &mw, ctx->tsz * (size_t)me));
-    launch_tab_markers(ib, cells, mrow, tmp, mcol, mw, ctx->d.precision, ctx->st);
+    const size_t me = n;
+    TabLayout k;
+    const size_t o_mcol = k.add(sizeof(int) * me), o_mw = k.add(ctx->tsz * me), o_mtmp = k.add(sizeof(int) * me);
+    TRY(tab_alloc(ctx, 1, &base, k.bytes));
+    mcol = (int *)(base + o_mcol);
+    mw = base + o_mw;
+    launch_tab_markers(ib, cells, mrow, (int *)(base + o_mtmp), mcol, mw, ctx->d.precision, ctx->st);
   }
   ctx->launches += iterate ? 10 : 7;
-  tb.dFT = dFT;
-  tb.FdV = FdV;
   CK(cudaGetLastError());
   tb.Ud = Ud;
   tb.arm = arm;
   tb.nrow = nrow;
   tb.ncol = ncol;
-  tb.nw = nw;
+  tb.nw = (char *)ctx->tab_mem[0].p + o_nw;
   tb.mrow = mrow;
   tb.mcol = mcol;
   tb.mw = mw;
