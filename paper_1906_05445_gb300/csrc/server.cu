@@ -71,7 +71,8 @@ size_t estimate_bytes(const lbm_request &r) {
   if (r.scheme.scheme == LBM_IBM_DIRECT) {
     b += 6 * n * tsz;
     // the markers' tables: up to 64 stencil points and about 70 coupled
-    // markers per marker, a 4-byte index and a coefficient each
+    // markers per marker, two 4-byte indices and a coefficient each, 250 bytes
+    // of its own, and an eighth for the next geometry
     double markers = 0;
     const double dens = r.scheme.ibm_marker_density > 0 ? r.scheme.ibm_marker_density : 1.0;
     for (int k = 0; k < r.nsolids; k++) {
@@ -79,7 +80,8 @@ size_t estimate_bytes(const lbm_request &r) {
       markers += dens * (d.lattice == LBM_D2Q9 ? 6.3 * R
                          : r.solids[k].kind == LBM_SPHERE ? 12.6 * R * R : 6.3 * R * d.nz);
     }
-    b += (size_t)(markers * (160.0 + 140.0 * (4 + tsz)));
+    // (a request of no finite size fails when it is created)
+    if (markers < 1e12) b += (size_t)(markers * 1.125 * (250.0 + 140.0 * (8 + tsz)));
   }
   return b + b / 10 + (1u << 20) + run_bytes(r);
 }
