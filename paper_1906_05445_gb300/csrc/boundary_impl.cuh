@@ -418,7 +418,7 @@ __device__ __forceinline__ void list_group(const KArgs &a, const S *src, S *dst,
 #pragma unroll
     for (int d = 0; d < Q; d++) f[d] = sm.f[d * NG + k];
     const Coll<T> c = make_coll<LAT, T>(a);
-    collide<LAT, CM, S, T>(f, Fx, Fy, Fz, c);
+    collide<LAT, CM, S, T, true>(f, Fx, Fy, Fz, c);
     scatter<LAT, S, T>(dst, a.fs, n, isc, f);
   }
   if (force_acc) {

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kRunBlock, 1) k_run(const __grid_constant__ Ru
 #pragma unroll
           for (int d = 0; d < Q; d++) f[d] = sm.f[d * NG + kk];
           const Coll<T> c = make_coll<LAT, T>(a);
-          collide<LAT, CM, S, T>(f, kg<T>(a, 0), kg<T>(a, 1), kg<T>(a, 2), c);
+          collide<LAT, CM, S, T, true>(f, kg<T>(a, 0), kg<T>(a, 1), kg<T>(a, 2), c);
           scatter<LAT, S, T>(dst, a.fs, li.n, isc, f);
         }
       }
