@@ -414,8 +414,8 @@ const char *lbm_last_error(const lbm_ctx *ctx);
  * (workload shaped like a grid-convergence sweep: one solve per resolution).
  * lbm_batch_create takes n distinct, configured and initialised contexts
  * on one device.  It prepares them (geometry, initial collision), gives
- * each a private stream and, when autotune_blocks != 0, picks the bulk and
- * boundary-node block widths per lattice shape by timing the kernels into a
+ * each a private stream and, when autotune_blocks != 0, picks the bulk
+ * sweep's block width per lattice shape by timing the kernel into a
  * scratch buffer (the simulation state is untouched).  While in a batch the
  * contexts must be stepped only through the batch; their queries remain
  * valid, and a context reconfigured between batch calls (scheme, solids,
@@ -444,8 +444,9 @@ lbm_status lbm_batch_step(lbm_batch *batch, int nsteps);
 lbm_status lbm_batch_run_to_steady(lbm_batch *batch, double tol,
                                    int check_every, int max_steps,
                                    int64_t *steps_done, double *residual);
-/* block widths chosen for lattice i and the number of graph launches (and of
- * multi-step launches of small lattices) */
+/* threads per block of lattice i's bulk sweep (the fastest of three with
+ * autotune_blocks) and of its boundary-node kernel (fixed: 128, IBM 64), and the
+ * number of graph launches and of multi-step launches of small lattices */
 lbm_status lbm_batch_info(lbm_batch *batch, int i, int *bulk_block,
                           int *list_block, int64_t *graph_launches);
 const char *lbm_batch_last_error(const lbm_batch *batch);

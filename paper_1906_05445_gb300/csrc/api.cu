@@ -126,7 +126,6 @@ struct lbm_ctx {
   long long N = 0;
   long long fs = 0;  // direction stride of the distribution arrays (elements)
   int bulk_block = 128;
-  int list_block = 128;  // threads per block of the boundary-node kernels (reported only)
   int cache_hints = 0;
   int bulk_mode = 1;
   int bulk_kernel = -1;  // the bulk sweep kernel of the last step (BulkKernel), -1 none yet
@@ -3443,7 +3442,8 @@ lbm_status lbm_batch_run_to_steady(lbm_batch *b, double tol, int check_every, in
 lbm_status lbm_batch_info(lbm_batch *b, int i, int *bulk_block, int *list_block, int64_t *graph_launches) {
   if (!b || i < 0 || i >= (int)b->ctx.size()) return LBM_ERR_ARG;
   if (bulk_block) *bulk_block = b->ctx[i]->bulk_block;
-  if (list_block) *list_block = b->ctx[i]->list_block;
+  if (list_block)
+    *list_block = b->ctx[i]->scheme.scheme == LBM_IBM_DIRECT ? kListIbmBlock : kListBlock;
   if (graph_launches) *graph_launches = b->graph_launches;
   return LBM_OK;
 }

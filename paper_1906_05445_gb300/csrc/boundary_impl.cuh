@@ -456,7 +456,6 @@ __device__ __forceinline__ void list_group(const KArgs &a, const S *src, S *dst,
   __syncthreads();  // the next group reuses the shared arrays
 }
 
-constexpr int kListBlock = 128;
 template <int LAT, int CM, typename S, typename T>
 __global__ void __launch_bounds__(kListBlock) k_list(const KArgs a) {
   __shared__ ListSmem<T, kListBlock> sm;
@@ -513,7 +512,7 @@ __device__ __forceinline__ void ibm_list_node(const KArgs &a, const S *src, S *d
 }
 
 template <int LAT, int CM, typename S, typename T>
-__global__ void __launch_bounds__(64) k_list_ibm(const KArgs a) {
+__global__ void __launch_bounds__(kListIbmBlock) k_list_ibm(const KArgs a) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   int cnt = a.counts[0];
   if (cnt > a.list_cap) cnt = a.list_cap;
@@ -1226,7 +1225,7 @@ void launch_one(SweepOp op, const KArgs &a, cudaStream_t st) {
   }
   case OP_LIST_SWEEP:
     if (a.list_cap > 0 && a.ibm)
-      k_list_ibm<LAT, CM, S, T><<<div_up(lc, 64), 64, 0, st>>>(a);
+      k_list_ibm<LAT, CM, S, T><<<div_up(lc, kListIbmBlock), kListIbmBlock, 0, st>>>(a);
     else if (a.list_cap > 0)
       k_list<LAT, CM, S, T>
           <<<div_up(lc, kListBlock / Lat<LAT>::Q), kListBlock, 0, st>>>(a);

@@ -183,6 +183,9 @@ struct GroupArgs {
 bool launch_bulk_group(const KArgs *as, int n, int lattice, int collision, int precision,
                        cudaStream_t st);
 
+// Threads per block of the boundary-node kernels (boundary_impl.cuh).
+constexpr int kListBlock = 128, kListIbmBlock = 64;
+
 // Many steps of small lattices in one launch (run_impl.cuh): lattice k runs on
 // blocks block_start[k] .. block_start[k + 1] - 1.
 constexpr int kMaxRun = 8;

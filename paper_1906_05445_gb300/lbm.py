@@ -417,7 +417,8 @@ def step_multi(lattices: Sequence["Lattice"], nsteps: int = 1):
 
 class Batch:
     """Several lattices advanced together (one CUDA graph launch per step
-    pair, per-lattice residual checks); see lbm_batch_create."""
+    pair, or multi-step launches where all are small; per-lattice residual
+    checks); see lbm_batch_create."""
 
     def __init__(self, lattices: Sequence[Lattice], stream: Optional[int] = None,
                  autotune: bool = True):

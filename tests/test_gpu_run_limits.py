@@ -305,3 +305,14 @@ def test_no_memory_for_the_tables(monkeypatch, iters):
         got = run(need + extra)
         assert rel_l2(got[0], ref[0], ref[1]) <= 1e-13
         assert np.abs(got[2][0] - ref[2][0]).max() <= 2e-12 * np.abs(ref[2][0]).max()
+
+
+def test_batch_reports_the_boundary_kernels_width():
+    from paper_1906_05445_gb300 import lbm
+    lats = [lbm.Lattice.from_problem(_disc(W.FP32, scheme=s)) for s in (W.BOUZIDI_QUAD, W.IBM)]
+    b = lbm.Batch(lats, autotune=False)
+    b.step(2)
+    assert [b.info(i)[1] for i in range(2)] == [128, 64]
+    b.close()
+    for g in lats:
+        g.close()
