@@ -242,7 +242,8 @@ struct lbm_ctx {
   // forces
   double *hist = nullptr;
   unsigned *run_bar = nullptr;  // k_run's barrier counters (zero between launches)
-  int zero_slot = -1;           // the record a k_run launch left zeroed for the step after it
+  int zero_slot = -1;           // the record that the last launch left zeroed for the step after it
+  unsigned long long zero_in = 0;  // the stream capture which that launch is part of (0: none)
   bool run_on = true;           // LBM_RUN=0, or refused: every step as launches of its own
   StepMark mark;
   long long beside = 0;  // bytes of the populations of lattices stepping beside this one
@@ -1433,6 +1434,16 @@ struct StepState {
   int nxt = 0;
 };
 
+// The capture that work on `st` is recorded into now (0: none).  What a captured
+// launch leaves behind holds within its capture only.
+lbm_status capture_of(lbm_ctx *ctx, cudaStream_t st, unsigned long long *id) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long n = 0;
+  CK(cudaStreamGetCaptureInfo(st, &status, &n));
+  *id = status == cudaStreamCaptureStatusNone ? 0 : n;
+  return LBM_OK;
+}
+
 lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
   const bool moving = any_moving(ctx);
   const bool ibm = ctx->scheme.scheme == LBM_IBM_DIRECT;
@@ -1469,14 +1480,22 @@ lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
     a.dst = ctx->f[cur];
     sweep(ctx, OP_REFILL, a);
   }
+  unsigned long long capture = 0;
+  TRY(capture_of(ctx, ctx->st, &capture));
   ctx->slot = (ctx->slot + 1) % kHistSlots;
-  ctx->zero_slot = -1;
+  const int zeroed = ctx->zero_slot;
   double *acc = force_slot(ctx, ctx->slot);
   a = base_args(ctx);
   a.src = ctx->f[cur];
   a.dst = ctx->f[nxt];
   a.force_acc = acc;
   a.rev = cur;  // alternates from step to step
+  // the boundary kernel of a bounce-back step clears the next step's record
+  ctx->zero_slot = -1;
+  if (ctx->scheme.scheme != LBM_IBM_DIRECT && a.list_cap > 0) {
+    ctx->zero_slot = (ctx->slot + 1) % kHistSlots;
+    a.force_next = force_slot(ctx, ctx->zero_slot);
+  }
   // fork: the boundary nodes (and the IBM pre-pass that feeds them) on the
   // auxiliary stream, the bulk nodes on the main stream; they read the same
   // f*(t) and write disjoint nodes of f*(t+1)
@@ -1484,7 +1503,9 @@ lbm_status step_begin(lbm_ctx *ctx, StepState &ss) {
   CK(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
   // the IBM band-velocity kernel clears the record itself (one launch fewer
   // on the IBM lattice's critical chain); otherwise a memset does
-  if (!ibm_zeroes_record(ctx)) CK(cudaMemsetAsync(acc, 0, sizeof(double) * kMaxSolids * 6, ctx->aux));
+  if (!ibm_zeroes_record(ctx) && !(zeroed == ctx->slot && ctx->zero_in == capture))
+    CK(cudaMemsetAsync(acc, 0, sizeof(double) * kMaxSolids * 6, ctx->aux));
+  ctx->zero_in = capture;
   ibm_prepass(ctx, ctx->f[cur], false, false, acc, ctx->aux);
   {
     Timed tm(ctx, TK_LIST, ctx->list_count >= 0 ? ctx->list_count : 0, ctx->aux);
@@ -1637,9 +1658,8 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaSt
   RunArgs<kMaxRun> g;
   memset(&g, 0, sizeof(g));
   g.n = n;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  CK(cudaStreamIsCapturing(st, &cap));
-  const bool capturing = cap != cudaStreamCaptureStatusNone;
+  unsigned long long capture = 0;
+  TRY(capture_of(ctx, st, &capture));
   int at = 0, blocks[kMaxRun];
   run_blocks(ctxs, n, share, blocks);
   for (int k = 0; k < n; k++) {
@@ -1660,8 +1680,7 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaSt
     r.vec = run_vec(c) ? 1 : 0;
     const int first = (c->slot + 1) % kHistSlots;
     // the record the launch starts with: left zeroed by the launch before
-    // (never relied on in a capture, whose replays find their own sums there)
-    if (c->zero_slot != first || capturing)
+    if (c->zero_slot != first || c->zero_in != capture)
       CK(cudaMemsetAsync(force_slot(c, first), 0, sizeof(double) * kMaxSolids * 6, st));
   }
   g.block_start[n] = at;
@@ -1677,8 +1696,8 @@ lbm_status run_launch(lbm_ctx *const *ctxs, int n, int nsteps, int share, cudaSt
   for (int k = 0; k < n; k++) {
     lbm_ctx *c = ctxs[k];
     c->slot = (c->slot + nsteps) % kHistSlots;
-    // a captured launch has not run: nothing is zeroed yet
-    c->zero_slot = capturing ? -1 : (c->slot + 1) % kHistSlots;
+    c->zero_slot = (c->slot + 1) % kHistSlots;
+    c->zero_in = capture;
     c->cur = (c->cur + nsteps) & 1;
     c->prev_local = false;
     c->records = std::min<long long>(c->records + nsteps, kHistCap);

@@ -421,11 +421,14 @@ __device__ __forceinline__ void list_group(const KArgs &a, const S *src, S *dst,
     collide<LAT, CM, S, T, true>(f, Fx, Fy, Fz, c);
     scatter<LAT, S, T>(dst, a.fs, n, isc, f);
   }
-  if (force_acc) {
-    // Eq. 17: the links' parts of each node in the compile-time order of the
-    // directions (compute type), then the nodes in FP64: the sums do not
-    // depend on the order of the list beyond FP64 rounding
-    for (int q = tid; q < 6 * NG; q += NT) {
+  // Eq. 17 in the other warps meanwhile: the links' parts of each node in the
+  // compile-time order of the directions (compute type), then the nodes in FP64:
+  // the sums do not depend on the order of the list beyond FP64 rounding
+  constexpr int NC = (NG + 31) / 32 * 32, NU = NT - NC;  // threads of the warps that collide, and the others
+  static_assert(NU >= 96, "16 threads per component");
+  if (force_acc && tid >= NC) {
+    const int u = tid - NC;
+    for (int q = u; q < 6 * NG; q += NU) {
       const int c = q / NG, kk = q - c * NG;
       if (group * NG + kk >= cnt) continue;
       T v = 0;
@@ -433,11 +436,10 @@ __device__ __forceinline__ void list_group(const KArgs &a, const S *src, S *dst,
       for (int d = 1; d < Q; d++) v += sm.red[c][d * NG + kk];
       if (sm.sid0[kk] >= 0) sm.cst[c][kk] += (double)v;
     }
-    __syncthreads();
+    asm volatile("bar.sync 1, %0;" ::"n"(NU) : "memory");
     for (int s = 0; s < a.nsolids; s++) {
-      if (tid < 96) {
-        // 16 threads per component
-        const int c = tid >> 4, p = tid & 15;
+      if (u < 96) {
+        const int c = u >> 4, p = u & 15;
         double v = 0;
         bool any = false;
         for (int kk = p; kk < NG && group * NG + kk < cnt; kk += 16)
@@ -459,6 +461,9 @@ __device__ __forceinline__ void list_group(const KArgs &a, const S *src, S *dst,
 template <int LAT, int CM, typename S, typename T>
 __global__ void __launch_bounds__(kListBlock) k_list(const KArgs a) {
   __shared__ ListSmem<T, kListBlock> sm;
+  // the next step's force record starts at zero (a clearing launch in front of
+  // this kernel would lie on the step's critical path)
+  if (a.force_next && blockIdx.x == 0 && threadIdx.x < 6 * kMaxSolids) a.force_next[threadIdx.x] = 0.0;
   int cnt = a.counts[0];
   if (cnt > a.list_cap) cnt = a.list_cap;
   if ((int)blockIdx.x * (kListBlock / Lat<LAT>::Q) >= cnt) return;

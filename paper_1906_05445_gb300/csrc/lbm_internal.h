@@ -90,6 +90,7 @@ struct KArgs {
   IbmTab tab;
   // momentum exchange accumulators: [solid][6] doubles (F, T)
   double *force_acc;
+  double *force_next;  // the next step's record, cleared by k_list (or null)
   int nsolids;
   // refill
   const int *refill_node;
