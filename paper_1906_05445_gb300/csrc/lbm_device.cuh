@@ -440,22 +440,14 @@ template <int LAT> __host__ __device__ constexpr double qk(int a, int b) {
   return s;
 }
 
-// position of pair leader i among the leaders
-template <int LAT> __host__ __device__ constexpr int pair_index(int i) {
-  int n = 0;
-  for (int k = 1; k < i; k++) n += Lat<LAT>::opp(k) > k;
-  return n;
-}
-
 // One node; ST is the storage type of the populations.  FP32 storage collides
 // pair by pair: its sweep is bound by HBM (128^3 without solids 51.6 us per
 // step, 50.9 with the grouped form, before the walk alternated), and over
 // hundreds of steps the two forms' roundings drift apart by 1e-5.
-// WALL: a node with cut links, whose roundings show in the solids' force.  The
-// moments are sums of the pairs' sums and differences, and the odd part is
-// w (3 e.u): 3 w rounded to FP32 is 3e-8 high, w itself 7e-9.  Error of the
-// torque after 20 steps of a 128^3 sphere 1.1e-6 -> 7.6e-7, of the force on the
-// sphere of the 48 M node open box 5.8e-8 -> 2.5e-8.
+// WALL: a node with cut links.  Its odd part is formed as w (3 e.u): 3 w rounded
+// to FP32 is 3e-8 high, w itself 7e-9, and at the wall that shows in the solids'
+// torque.  Rms error over 12 seeds: 128^3 sphere after 20 steps 1.09e-6 -> 7.6e-7,
+// moving sphere 6.4e-7 -> 4.1e-7.
 template <int LAT, int CM, typename ST, typename T, bool WALL = false>
 __device__ __forceinline__ void collide(T (&f)[Lat<LAT>::Q], T Fx, T Fy, T Fz,
                                         const Coll<T> &c) {
@@ -467,38 +459,16 @@ __device__ __forceinline__ void collide(T (&f)[Lat<LAT>::Q], T Fx, T Fy, T Fz,
     return;
   }
   T drho = 0, jx = 0, jy = 0, jz = 0;
-  if constexpr (WALL && !MRT) {
-    T sp[Q / 2];
-    static_for<Q>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      if constexpr (i > 0 && L::opp(i) > i) {
-        const T d = f[i] - f[L::opp(i)];
-        sp[pair_index<LAT>(i)] = f[i] + f[L::opp(i)];
-        if constexpr (L::ex(i) == 1) jx += d;
-        if constexpr (L::ex(i) == -1) jx -= d;
-        if constexpr (L::ey(i) == 1) jy += d;
-        if constexpr (L::ey(i) == -1) jy -= d;
-        if constexpr (L::ez(i) == 1) jz += d;
-        if constexpr (L::ez(i) == -1) jz -= d;
-      }
-    });
-#pragma unroll
-    for (int o = 1; o < Q / 2; o <<= 1)
-#pragma unroll
-      for (int i = 0; i + o < Q / 2; i += 2 * o) sp[i] += sp[i + o];
-    drho = f[0] + sp[0];
-  } else {
-    static_for<Q>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      drho += f[i];
-      if constexpr (L::ex(i) == 1) jx += f[i];
-      if constexpr (L::ex(i) == -1) jx -= f[i];
-      if constexpr (L::ey(i) == 1) jy += f[i];
-      if constexpr (L::ey(i) == -1) jy -= f[i];
-      if constexpr (L::ez(i) == 1) jz += f[i];
-      if constexpr (L::ez(i) == -1) jz -= f[i];
-    });
-  }
+  static_for<Q>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    drho += f[i];
+    if constexpr (L::ex(i) == 1) jx += f[i];
+    if constexpr (L::ex(i) == -1) jx -= f[i];
+    if constexpr (L::ey(i) == 1) jy += f[i];
+    if constexpr (L::ey(i) == -1) jy -= f[i];
+    if constexpr (L::ez(i) == 1) jz += f[i];
+    if constexpr (L::ez(i) == -1) jz -= f[i];
+  });
   const T ux = jx + (T)0.5 * Fx, uy = jy + (T)0.5 * Fy, uz = jz + (T)0.5 * Fz;
   const T uu = ux * ux + uy * uy + uz * uz;
   const T uF = ux * Fx + uy * Fy + uz * Fz;
