@@ -1610,23 +1610,27 @@ bool run_vec(const lbm_ctx *ctx) {
 
 // Largest lattice (populations, nodes x Q) whose steps k_run takes, from us
 // per step of k_run against the step's own launches (3D spheres of R = 3/32
-// of the edge, 2D Couette flows; FP32 with packed pairs):
-//   FP32 bounce-back  64^3 8.2 / 14.2, 80^3 12.4 / 14.3, 88^3 18.7 / 16.1;
-//                     301^2 5.2 / 11.3, 512^2 6.3 / 11.9
-//   FP32 IBM, 1 pass  64^3 14.8 / 24.1, 72^3 20.7 / 24.0, 80^3 23.8 / 24.2
-//   FP32 IBM, 5       80^3 33.4 / 49.6, 96^3 47.6 / 57.4
-//   FP16 bounce-back  80^3 11.0 / 14.4, 88^3 14.2 / 14.2; IBM 72^3 22.1 / 22.7
-//   FP64 bounce-back  48^3 41.9 / 51.9, 56^3 60.8 / 59.7; 512^2 34.4 / 41.1
-//   FP64 IBM, 1       32^3 27.7 / 30.9, 41^3 38.2 / 37.2; 5: 48^3 67 / 79, 64^3 110 / 111
+// of the edge, 2D Couette flows).  A bounce-back step's launches take one of two
+// times, as the boundary kernel's blocks get to run before or behind the sweep's:
+//   FP32 bounce-back  24^3 4.9 / 8.0, 64^3 9.2 / 10.6-11.8, 72^3 11.7 / 10.6-13.7,
+//                     80^3 14.4 / 12.8-15.5, 88^3 20.8 / 18.2;
+//                     64^2 4.2 / 8.5, 512^2 6.6 / 8.7, 850^2 10.1 / 11.2, 1024^2 12.9 / 12.9
+//   FP32 IBM, 1 pass  64^3 15.8 / 21.0, 72^3 22.0 / 22.5, 80^3 25.8 / 23.6
+//   FP32 IBM, 5       80^3 36.2 / 47.5, 96^3 51.4 / 53.7
+//   BF16 bounce-back  64^3 7.4 / 9.5, 80^3 10.2 / 11.8; FP16 8.3 / 10.7, 11.1 / 11.2
+//   FP16 IBM, 1 pass  68^3 15.3 / 20.9, 72^3 22.5 / 20.9
+//   FP64 bounce-back  32^3 20.9 / 17.1-25.7, 48^3 42.1 / 41.8, 52^3 52.0 / 47.6;
+//                     64^2 9.1 / 10.6, 301^2 18.0 / 18.8, 512^2 34.5 / 32.0
+//   FP64 IBM, 1       32^3 28.3 / 29.4, 40^3 37.6 / 37.4; 5: 48^3 67.3 / 73.2, 64^3 111 / 110
 // Beyond, the one block per SM keeps too few loads in flight for the sweep.  On
 // a share of the SMs the limits shrink with it (half the SMs: 64^3 bounce-back
-// 14.2 / 14.7, 72^3 17.7 / 15.7; IBM 40^3 13.2 / 20.3, 56^3 21.2 / 20.7; five passes
-// 80^3 44.0 / 46.8; a quarter: 40^3 9.2 / 10.9, 48^3 12.4 / 11.6).
+// 14.2, 72^3 17.7; IBM 40^3 13.2, 56^3 21.2; five passes 80^3 44.0).
 bool run_small(const lbm_ctx *ctx, int share) {
   const bool f64 = ctx->d.precision == LBM_FP64;
   const long long v = ctx->N * ctx->Q * share;
   if (ctx->scheme.scheme != LBM_IBM_DIRECT || ctx->nmark == 0) return v <= (f64 ? 2400000 : 10000000);
-  if (ctx->scheme.ibm_iters <= 1) return v <= (f64 ? 700000 : 7200000);
+  if (ctx->scheme.ibm_iters <= 1)
+    return v <= (f64 ? 700000 : ctx->d.precision == LBM_FP32 ? 7200000 : 6400000);
   return v <= (f64 ? 2400000 : 17000000);
 }
 
@@ -2978,16 +2982,16 @@ std::vector<std::vector<int>> run_groups(const lbm_batch *b) {
 // us per step of both.  k_run's launches follow each other and hold the SMs, so a
 // lattice outside it (large, or moving) would wait for them: such batches are all
 // graph (128^3 with a 64^3 IBM lattice 60.8 us per step against 68.3).  A replay
-// steps all lattices side by side at about 4 us of launches each.  Measured, k_run
-// / graph, n lattices of one kind, then grid-convergence batches (edges 24 ...,
+// steps all lattices side by side at 3-5 us of launches each.  Measured, k_run /
+// graph, n lattices of one kind, then grid-convergence batches (edges 24 ...,
 // alternately bounce-back and IBM):
-//   FP32 bounce-back  8 x 24^3 6.6 / 34.6, 8 x 48^3 27.6 / 45.0, 8 x 56^3 48.9 / 45.9;
-//                     2 x 56^3 11.9 / 14.7, 4 x 64^3 32.4 / 30.4
-//   FP32 IBM, 1 pass  4 x 40^3 20.4 / 22.3, 4 x 56^3 32.7 / 28.4, 2 x 48^3 19.9 / 17.6
-//   FP32 IBM, 5       8 x 48^3 50.0 / 63.6, 8 x 56^3 81.4 / 75.4
-//   FP64 bounce-back  8 x 32^3 84.6 / 87.4, 64^2 9.2 / 13.6, 8 x 64^2 13.3 / 40.2
-//   FP64 IBM          4 x 32^3 80.5 / 53.6 (1 pass), 8 x 24^3 112 / 72 (5): graph
-//   convergence       5 (24-56) 31.8 / 27.9, 8 (24-64) 42.8 / 52.6, 10 53.3 / 65.4
+//   FP32 bounce-back  8 x 24^3 6.6 / 29.7, 8 x 48^3 27.3 / 38.0, 8 x 56^3 48.4 / 42.9;
+//                     2 x 48^3 9.2 / 11.0, 4 x 56^3 21.7 / 18.9
+//   FP32 IBM, 1 pass  4 x 40^3 21.1 / 21.8, 4 x 56^3 32.2 / 28.7, 2 x 48^3 20.7 / 17.6
+//   FP32 IBM, 5       8 x 48^3 50.0 / 64.5, 8 x 56^3 81.6 / 75.8
+//   FP64 bounce-back  8 x 24^3 41.2 / 46.4, 8 x 32^3 84.5 / 83.6; 8 x 64^2 13.4 / 36.0
+//   FP64 IBM          4 x 32^3 86.2 / 53.6 (1 pass), 8 x 24^3 111 / 71 (5): graph
+//   convergence       5 (24-56) 31.5 / 26.2, 8 (24-64) 43.3 / 45.2, 10 53.2 / 61.9
 // The estimates are fits to 114 such batches; p counts populations in millions, an
 // FP64 one as 11.
 double run_us(const lbm_batch *b, const std::vector<int> &group) {
@@ -3026,9 +3030,10 @@ double graph_us(const lbm_batch *b) {
       iters = std::max(iters, c->scheme.ibm_iters);
     }
   }
-  const double launches = (ibm ? 5 : 3) + 4.1 * std::min(n, 5) + 5.5 * std::max(0, n - 5);
-  const double work = (f64 ? 14 : ibm ? 10 : 6) + (ibm ? 1.45 : 1.3) * p;
-  return std::max({(ibm ? 12.0 : 8.0) + 2 * n, launches, work}) + 2.9 * (iters - 1);
+  const int more = std::max(0, n - 5);
+  const double launches = ibm ? 5 + 4.1 * (n - more) + 5.5 * more : 1.5 + 3.4 * (n - more) + 5.0 * more;
+  const double work = (f64 ? 14 : ibm ? 10 : 5) + (ibm ? 1.45 : f64 ? 1.3 : 1.2) * p;
+  return std::max({ibm ? 12 + 2.0 * n : 7.3 + 1.3 * n, launches, work}) + 3.6 * (iters - 1);
 }
 
 // All nsteps of a batch in k_run.  In one launch whose threads hold both kinds'

@@ -213,7 +213,7 @@ def test_lattices_on_streams_of_their_own_share_the_sms(monkeypatch):
     stepped alone has them all again.  The fields do not depend on it."""
     import torch
     from paper_1906_05445_gb300 import lbm
-    p = W.Problem("share", W.D3Q19, 36, 36, 36, 0.7, W.MRT, W.FP64, (1e-4, -2e-4, 0.0), SPHERE,
+    p = W.Problem("share", W.D3Q19, 58, 58, 58, 0.7, W.MRT, W.FP32, (1e-4, -2e-4, 0.0), SPHERE,
                   W.BOUZIDI_QUAD, 0)
     monkeypatch.setenv("LBM_RUN", "0")
     ref = lbm.Lattice.from_problem(p)
