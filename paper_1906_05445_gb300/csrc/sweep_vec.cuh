@@ -322,9 +322,9 @@ template <typename S, int W, bool PACKED> constexpr int vec_regs() {
 // ring in shared memory.)
 // Blocks walk the lattice from its end when a.rev is set (every other step):
 // a step then starts on the nodes that the previous one wrote last, which L2
-// still holds, instead of on those it has already evicted.  128^3 without
-// solids, FP32 (packed): 50.9 -> 48.0 us per step (and 47.2 with evict-first
-// reads, LD_ONCE); 112^3 36.1 -> 32.6 (30.9); FP16 128^3 28.8 -> 26.7 (24.7).
+// still holds, instead of on those it has already evicted.  us per step without
+// solids: FP32 112^3 36.5 -> 33.6, 128^3 51.9 -> 48.6, 160^3 96.5 -> 94.3; FP16 128^3
+// 31.2 -> 29.0 (26.6 with evict-first reads, LD_ONCE).
 template <int LAT, int CM, typename S, int W, bool PACKED, int POL>
 __global__ void __maxnreg__((vec_regs<S, W, PACKED>()))
     k_bulk_vec(const KArgs a) {
@@ -340,7 +340,9 @@ __global__ void __maxnreg__((vec_regs<S, W, PACKED>()))
 // arguments stay constant-bank operands (indexing the argument array by a
 // run-time k holds them in registers: 92 instead of 80, one block per SM
 // fewer).
-// The single-lattice kernel's register limits.
+// The single-lattice kernel's register limits (FP32 at 64, with 404 bytes of spill
+// stores: two empty 128^3 101.7 us per step against 100.6 at 80, eight 64^3 spheres
+// 77.2 against 86.5).
 template <int LAT, int CM, typename S, int W, bool PACKED>
 __global__ void __maxnreg__((vec_regs<S, W, PACKED>()))
     k_bulk_vec_group(const __grid_constant__ GroupArgs g) {
