@@ -264,7 +264,10 @@ lbm_status lbm_get_distributions(lbm_ctx *ctx, double *host_f, size_t n);
 /* Advance nsteps time steps (asynchronous).  One step: geometry of moving
  * solids and refilling of uncovered nodes, IBM forcing (Sec. 2.1), the fused
  * pull collide-stream sweep with interpolated bounce-back on cut links
- * (Sec. 2.2) and the momentum exchange of Eq. 17. */
+ * (Sec. 2.2) and the momentum exchange of Eq. 17.  A small lattice with
+ * solids at rest runs the steps of a call (nsteps >= 2) in launches of up to
+ * 256 steps on every SM, or on its share of them where lattices on other
+ * streams stepped since its last call. */
 lbm_status lbm_step(lbm_ctx *ctx, int nsteps);
 /* Advance n distinct lattices nsteps steps together (asynchronous): each
  * step runs every lattice's boundary and IBM work as lbm_step does, and the
