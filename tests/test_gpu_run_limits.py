@@ -1,6 +1,8 @@
 """Where the multi-step launch of small lattices (k_run) meets the rest of the
-library: geometry changed between launches.  Every case is compared with the
-same steps as launches of their own (LBM_RUN=0).
+library: geometry changed between launches, the ring of force records, captures,
+long calls, refused launches, few and many blocks, lattices on several streams and
+in batches, missing memory.  Compared with the same steps as launches of their own
+(LBM_RUN=0).
 """
 import numpy as np
 import pytest
